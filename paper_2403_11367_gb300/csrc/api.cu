@@ -141,7 +141,7 @@ struct reloc_ctx {
     DevBuf trgb, tgimg, tabc, tloss, tgrad, adam_m, adam_v;
     DevBuf tdep, talp, twarp, tjac, tgw, tgda, trel;     // re-projection loss
     int64_t adam_t = 0;
-    PinBuf pin;
+    PinBuf pin, gemm_status;
     double inst_ratio = 3.0;        // instance capacity per (view, subset Gaussian), learned
     // batch options
     int use_graph = 1;
@@ -259,6 +259,7 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
     for (DevBuf *b : bufs) b->release();
     if (ctx->prop) proposal_destroy(ctx->prop);
     ctx->pin.release();
+    ctx->gemm_status.release();
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
@@ -1499,16 +1500,17 @@ extern "C" reloc_status reloc_gemm_bf16(reloc_ctx *ctx, const uint16_t *A_dev, c
     if (((uintptr_t)A_dev & 15) || ((uintptr_t)B_dev & 15)) return fail(RELOC_EINVAL, "gemm: A, B need 16-byte alignment");
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
-    CKS(ctx->flags.ensure(64));
+    // the status word lies in pinned host memory, which the kernel writes only
+    // when a wait gives up: no memset before and no copy after the launch
+    CKS(ctx->gemm_status.ensure(64));
+    volatile int *status = (volatile int *)ctx->gemm_status.p;
     DevBuf &part = ctx->chunk_sums;     // scratch for split-K partials
     if (split_k > 1) CKS(part.ensure(4 * (size_t)split_k * M * N));
-    CK(cudaMemsetAsync(ctx->flags.p, 0, 4, st));
+    *status = 0;
     CK(launch_gemm_bf16((const __nv_bfloat16 *)A_dev, (const __nv_bfloat16 *)B_dev, bias_dev, C_dev, nullptr, M, N, K,
-                        K, K, N, relu, split_k, part.as<float>(), ctx->flags.as<int>(), st));
-    int status = 0;
-    CK(cudaMemcpyAsync(&status, ctx->flags.p, 4, cudaMemcpyDeviceToHost, st));
+                        K, K, N, relu, split_k, part.as<float>(), (int *)ctx->gemm_status.p, st));
     CK(cudaStreamSynchronize(st));
-    if (status) return fail(RELOC_ETIMEOUT, "gemm: a tensor-core wait gave up");
+    if (*status) return fail(RELOC_ETIMEOUT, "gemm: a tensor-core wait gave up");
     return RELOC_OK;
 }
 

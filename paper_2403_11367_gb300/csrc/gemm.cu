@@ -7,43 +7,51 @@
 // contraction of the learned candidate proposal (convolutions via im2col and
 // the MLP, forward and backward).
 //
-// One CTA of 128 threads computes a 128 x BN tile (BN in {16, 32, ..., 256}),
-// warp-specialised over a ring of GEMM_STAGES shared-memory stages:
+// Persistent: as many CTAs as fit take 128 x BN output tiles (BN in {16, 32,
+// ..., 256}) in turn.  A CTA of 192 threads is warp-specialised over a ring of
+// shared-memory stages and two TMEM accumulators:
 //   - one lane of warp 0 loads the A (128 x 64) and B (BN x 64) tiles of each
 //     K step with TMA (cp.async.bulk.tensor, one box per operand: 64 BF16 =
 //     128 bytes of K by the tile's rows, 128-byte swizzle, so the tiles land
 //     in the canonical K-major SWIZZLE_128B layout: 128-byte rows whose 16-byte
 //     chunks are XOR-permuted by the row within each 8-row, 1024-byte group)
 //     and signals the stage's "full" mbarrier through the copies'
-//     transaction count;
+//     transaction count; the ring runs on from one tile into the next;
 //   - one lane of warp 1 waits for a full stage, issues its four
-//     tcgen05.mma (K = 16 each) into the TMEM accumulator and commits them to
+//     tcgen05.mma (K = 16 each) into the tile's accumulator and commits them to
 //     the stage's "empty" mbarrier, which releases the stage to the loader
-//     once the MMAs have read it; after the last K step it commits to a
-//     "done" mbarrier;
-//   - all four warps wait for "done" and read the accumulator with
-//     tcgen05.ld (each warp its 32 TMEM lanes), applying bias and ReLU.
-// So the loads of the next stages are in flight while the tensor cores work
-// on the current one.  With split_k > 1, CTA z covers the K range
-// [z*Ks, (z+1)*Ks) and writes FP32 partials C[z][M][N], summed later in a
-// fixed order.
+//     once the MMAs have read it; after the tile's last K step it commits to the
+//     accumulator's "tfull" mbarrier;
+//   - warps 2..5 wait for "tfull", read the accumulator with tcgen05.ld (each
+//     warp its 32 TMEM lanes), hand it back ("tempty"), and write the tile out
+//     while the tensor cores work on the next one: 32 x 32 pieces go through
+//     shared memory so that a row's 32 values leave as one 128-byte store (a
+//     lane's own row written straight from its registers put every lane of a
+//     store on another line, and the write took several times as long as the
+//     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us).  Bias and
+//     ReLU are applied there.
+// With split_k > 1 a tile covers the K range [z*Ks, (z+1)*Ks) and writes FP32
+// partials C[z][M][N], summed later in a fixed order.
 //
 // Every mbarrier wait is bounded (GEMM_WAIT_NS of the global timer): past it
-// the CTA records an error in *status and stops issuing; the loader then
-// waits (bounded) for its own copies in flight, the MMA lane commits "done"
-// (which tracks every MMA it issued) and all threads wait for it (bounded)
-// before the tensor memory is freed, so nothing the CTA started still writes
-// shared or tensor memory when it exits.
+// the CTA records an error in *status and every role stops at its next wait;
+// the loader then waits (bounded) for its own copies in flight, the MMA lane
+// commits "done" (which tracks every MMA it issued) and all threads wait for it
+// (bounded) before the tensor memory is freed, so nothing the CTA started still
+// writes shared or tensor memory when it exits.
+#include <atomic>
+
 #include "internal.cuh"
 
 #include <cuda.h>
 
 namespace reloc {
 
-constexpr int GEMM_THREADS = 128;
+constexpr int GEMM_THREADS = 192;                   // loader, MMA, four epilogue warps
+constexpr int GEMM_EPI_WARP0 = 2, GEMM_EPI_WARPS = 4;
 constexpr int GEMM_BM = 128;
 constexpr int GEMM_BK = 64;
-constexpr int GEMM_STAGES = 4;
+constexpr int GEMM_EPI_LD = 36;                     // floats per staged row: 16-byte rows, no bank conflict
 constexpr unsigned long long GEMM_WAIT_NS = 1000000000ull;   // 1 s per wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
@@ -119,6 +127,32 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
                  : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+
+// W columns (16 or 32) of this warp's 32 TMEM lanes, one lane's row per thread.
+template <int W> __device__ __forceinline__ void tmem_ld(uint32_t addr, uint32_t (&r)[W]);
+template <> __device__ __forceinline__ void tmem_ld<16>(uint32_t addr, uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(addr));
+}
+template <> __device__ __forceinline__ void tmem_ld<32>(uint32_t addr, uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
+                   "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+                   "=r"(r[30]), "=r"(r[31])
+                 : "r"(addr));
+}
+
 struct GemmArgs {
     const float *bias;          // [N] or null
     float *Cf;                  // FP32 output (or split-K partials) or null
@@ -127,8 +161,10 @@ struct GemmArgs {
     int ldc;                    // row stride of C (elements)
     int relu;
     int split_k;                // >= 1; > 1 writes partials Cf[z][M][ldc]
+    int n_tn, n_tiles;          // column tiles, all tiles (row tiles x column tiles x split_k)
+    int vec;                    // 16-byte (BF16: 8-byte) stores allowed: ldc, N and the bases
     int inject;                 // test only: the MMA lane waits on a barrier nothing arrives at
-    int *status;                // error flag (1: an mbarrier wait gave up)
+    int *status;                // error flag (1: an mbarrier wait gave up), device or pinned host memory
 };
 
 template <int BN>
@@ -136,7 +172,12 @@ struct GemmSmem {
     static constexpr uint32_t A_BYTES = GEMM_BM * GEMM_BK * 2;
     static constexpr uint32_t B_BYTES = BN * GEMM_BK * 2;
     static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-    static constexpr size_t TOTAL = (size_t)GEMM_STAGES * STAGE + 1024;   // + alignment slack
+    // four stages of the widest tile fill the SM's shared memory; narrower
+    // tiles take the loads' latency on four stages too, two CTAs to an SM
+    static constexpr int STAGES = 4;
+    static constexpr size_t EPI = (size_t)GEMM_EPI_WARPS * 32 * GEMM_EPI_LD * 4;
+    static constexpr size_t TOTAL = (size_t)STAGES * STAGE + EPI + 1024;   // + alignment slack
+    static constexpr uint32_t TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;       // two accumulators, power of two >= 32
 };
 
 template <int BN>
@@ -144,32 +185,35 @@ __global__ void __launch_bounds__(GEMM_THREADS)
 k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs g)
 {
     using SM = GemmSmem<BN>;
+    constexpr int STAGES = SM::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t bar_full[GEMM_STAGES], bar_empty[GEMM_STAGES], bar_done, bar_never;
+    __shared__ __align__(8) uint64_t bar_full[STAGES], bar_empty[STAGES], bar_tfull[2], bar_tempty[2], bar_done,
+        bar_never;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
+    __shared__ volatile int abort_s;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * GEMM_BM, n0 = blockIdx.y * BN;
-    const int kz = blockIdx.z;
     const int k_per = g.K / g.split_k;                  // multiple of 64 by construction
-    const int kbeg = kz * k_per;
     const int n_k = k_per / GEMM_BK;
-    constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;   // power of two >= 32
+    const int n_mn = g.n_tiles / g.split_k;
     constexpr uint32_t IDESC = instr_desc_bf16(GEMM_BM, BN);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
-                     "r"(TMEM_COLS)
+                     "r"(SM::TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 32) {
         abort_s = 0;
-        for (int s = 0; s < GEMM_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(smem_u32(&bar_tfull[s]), 1);
+            mbar_init(smem_u32(&bar_tempty[s]), GEMM_EPI_WARPS);
         }
         mbar_init(smem_u32(&bar_done), 1);
         mbar_init(smem_u32(&bar_never), 1);
@@ -180,118 +224,161 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_s;
     const uint32_t sbase = smem_u32(smem);
+    // a bounded wait that gave up stops every role of the CTA
+    auto wait = [&](uint64_t &bar, uint32_t parity) -> bool {
+        if (abort_s) return false;
+        if (mbar_wait(smem_u32(&bar), parity)) return true;
+        abort_s = 1;
+        if (g.status) atomicExch_system(g.status, 1);
+        return false;
+    };
 
     if (tid == 0) {
-        // ---- loader: K step it into stage it % GEMM_STAGES ------------------
-        int issued = 0;
-        for (int it = 0; it < n_k; ++it) {
-            const int s = it % GEMM_STAGES;
-            const uint32_t ph = (uint32_t)(it / GEMM_STAGES) & 1u;
-            // the stage is free once the MMAs of K step it - GEMM_STAGES have read it
-            if (it >= GEMM_STAGES && !mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1u)) {
-                abort_s = 1;
-                if (g.status) atomicExch(g.status, 1);
-                break;
+        // ---- loader: the CTA's K steps, numbered through its tiles, into stage it % STAGES
+        int it = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
+            const int z = t / n_mn, mn = t - z * n_mn;
+            const int m0 = mn / g.n_tn * GEMM_BM, n0 = mn % g.n_tn * BN, kbeg = z * k_per;
+            for (int k = 0; k < n_k; ++k, ++it) {
+                const int s = it % STAGES;
+                const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
+                // the stage is free once the MMAs of K step it - STAGES have read it
+                if (it >= STAGES && !wait(bar_empty[s], ph ^ 1u)) { ok = false; break; }
+                if (abort_s) { ok = false; break; }
+                const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
+                const uint32_t fb = smem_u32(&bar_full[s]);
+                mbar_expect_tx(fb, SM::STAGE);
+                tma_load_2d(sa, &tmA, kbeg + k * GEMM_BK, m0, fb);
+                tma_load_2d(sb, &tmB, kbeg + k * GEMM_BK, n0, fb);
             }
-            if (abort_s) break;
-            const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
-            const uint32_t fb = smem_u32(&bar_full[s]);
-            mbar_expect_tx(fb, SM::STAGE);
-            const int k0 = kbeg + it * GEMM_BK;
-            tma_load_2d(sa, &tmA, k0, m0, fb);
-            tma_load_2d(sb, &tmB, k0, n0, fb);
-            ++issued;
         }
         // copies still in flight land before the CTA may exit: the last one
         // issued on each stage completes that stage's current phase
-        for (int it = issued - GEMM_STAGES < 0 ? 0 : issued - GEMM_STAGES; it < issued; ++it)
-            if (!mbar_wait(smem_u32(&bar_full[it % GEMM_STAGES]), (uint32_t)(it / GEMM_STAGES) & 1u) && g.status)
-                atomicExch(g.status, 1);
+        for (int i = it - STAGES < 0 ? 0 : it - STAGES; i < it; ++i)
+            if (!mbar_wait(smem_u32(&bar_full[i % STAGES]), (uint32_t)(i / STAGES) & 1u) && g.status)
+                atomicExch_system(g.status, 1);
     } else if (tid == 32) {
         // ---- MMA issuer ----------------------------------------------------------
-        if (g.inject) {
-            // test only: a wait that nothing completes runs out
-            if (!mbar_wait(smem_u32(&bar_never), 0u)) {
-                abort_s = 1;
-                if (g.status) atomicExch(g.status, 1);
-            }
-        }
-        for (int it = 0; it < n_k && !abort_s; ++it) {
-            const int s = it % GEMM_STAGES;
-            const uint32_t ph = (uint32_t)(it / GEMM_STAGES) & 1u;
-            if (!mbar_wait(smem_u32(&bar_full[s]), ph)) {
-                abort_s = 1;
-                if (g.status) atomicExch(g.status, 1);
-                break;
-            }
+        bool ok = true;
+        if (g.inject) ok = wait(bar_never, 0u);          // test only: a wait that nothing completes runs out
+        int it = 0, i = 0;
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++i) {
+            // the accumulator is free once the epilogue of tile i - 2 has read it
+            if (i >= 2 && !wait(bar_tempty[i & 1], ((uint32_t)(i >> 1) & 1u) ^ 1u)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
+            const uint32_t acc_t = tmem + (uint32_t)((i & 1) * BN);
+            for (int k = 0; k < n_k; ++k, ++it) {
+                const int s = it % STAGES;
+                if (!wait(bar_full[s], (uint32_t)(it / STAGES) & 1u)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
 #pragma unroll
-            for (int j = 0; j < GEMM_BK / 16; ++j) {
-                // K step j: 16 BF16 = 32 bytes further along the 128-byte rows
-                const uint64_t da = smem_desc_sw128(sa + 32 * j);
-                const uint64_t db = smem_desc_sw128(sb + 32 * j);
-                const uint32_t acc = (it > 0 || j > 0) ? 1u : 0u;
-                asm volatile("{\n\t.reg .pred p;\n\t"
-                             "setp.ne.u32 p, %4, 0;\n\t"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-                             "l"(da), "l"(db), "r"(IDESC), "r"(acc)
+                for (int j = 0; j < GEMM_BK / 16; ++j) {
+                    // K step j: 16 BF16 = 32 bytes further along the 128-byte rows
+                    const uint64_t da = smem_desc_sw128(sa + 32 * j);
+                    const uint64_t db = smem_desc_sw128(sb + 32 * j);
+                    const uint32_t acc = (k > 0 || j > 0) ? 1u : 0u;
+                    asm volatile("{\n\t.reg .pred p;\n\t"
+                                 "setp.ne.u32 p, %4, 0;\n\t"
+                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc_t),
+                                 "l"(da), "l"(db), "r"(IDESC), "r"(acc)
+                                 : "memory");
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             ::"r"(smem_u32(&bar_empty[s]))
                              : "memory");
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         ::"r"(smem_u32(&bar_empty[s]))
-                         : "memory");
+            if (ok)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             ::"r"(smem_u32(&bar_tfull[i & 1]))
+                             : "memory");
         }
         // "done" completes once every MMA this lane issued has finished
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                      ::"r"(smem_u32(&bar_done))
                      : "memory");
-    }
-    __syncwarp();
-    __syncthreads();
-    if (!mbar_wait(smem_u32(&bar_done), 0u)) {
-        abort_s = 1;
-        if (g.status) atomicExch(g.status, 1);
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    __syncthreads();
-
-    // ---- epilogue: TMEM -> registers -> global ------------------------------
-    if (!abort_s) {
-        const int row = m0 + warp * 32 + lane;
-        const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-        const bool any = n_k > 0;
+    } else if (warp >= GEMM_EPI_WARP0) {
+        // ---- epilogue: TMEM -> registers -> shared memory -> global -----------------
+        constexpr int CW = BN < 32 ? BN : 32;           // columns per piece
+        const int quad = warp & 3;                      // the 32 TMEM lanes this warp may read
+        float *const st = reinterpret_cast<float *>(smem + (size_t)STAGES * SM::STAGE) +
+                          (warp - GEMM_EPI_WARP0) * 32 * GEMM_EPI_LD;
+        int i = 0;
+        for (int t = blockIdx.x; t < g.n_tiles; t += gridDim.x, ++i) {
+            const int z = t / n_mn, mn = t - z * n_mn;
+            const int row0 = mn / g.n_tn * GEMM_BM + quad * 32, n0 = mn % g.n_tn * BN;
+            // every lane waits for itself; one that gave up takes the warp out
+            if (!__all_sync(0xffffffffu, wait(bar_tfull[i & 1], (uint32_t)(i >> 1) & 1u))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t src = tmem + (uint32_t)((i & 1) * BN) + ((uint32_t)(quad * 32) << 16);
+            const int rows = min(32, g.M - row0);
+            const int64_t crow = (int64_t)z * g.M * (g.split_k > 1) + row0;
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            uint32_t r[16];
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                           "=r"(r[14]), "=r"(r[15])
-                         : "r"(lane_addr + c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < g.M) {
+            for (int c0 = 0; c0 < BN; c0 += CW) {
+                uint32_t r[CW];
+                tmem_ld<CW>(src + c0, r);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (c0 + CW == BN) {
+                    // the accumulator is read: hand it back before the last stores
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bar_tempty[i & 1]));
+                }
+                if (n0 + c0 >= g.N || rows <= 0) continue;   // uniform over the warp
+                __syncwarp();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int col = n0 + c0 + i;
-                    if (col >= g.N) continue;
-                    float v = any ? __uint_as_float(r[i]) : 0.f;
-                    if (g.split_k > 1) {
-                        g.Cf[((int64_t)kz * g.M + row) * g.ldc + col] = v;
-                        continue;
+                for (int c = 0; c < CW; c += 4)
+                    *reinterpret_cast<float4 *>(st + lane * GEMM_EPI_LD + c) =
+                        make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]), __uint_as_float(r[c + 2]),
+                                    __uint_as_float(r[c + 3]));
+                __syncwarp();
+                const int cn = min(CW, g.N - n0 - c0);      // valid columns of the piece
+                if (g.vec) {
+                    constexpr int LPR = CW / 4, RPS = 32 / LPR;   // lanes per row, rows per store
+                    const int c = (lane % LPR) * 4, col = n0 + c0 + c;
+                    if (c < cn) {                           // N is a multiple of 4: whole groups
+                        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (g.bias) b = make_float4(g.bias[col], g.bias[col + 1], g.bias[col + 2], g.bias[col + 3]);
+#pragma unroll
+                        for (int rr = lane / LPR; rr < 32; rr += RPS) {
+                            if (rr >= rows) break;
+                            float4 v = *reinterpret_cast<const float4 *>(st + rr * GEMM_EPI_LD + c);
+                            if (g.bias) { v.x += b.x; v.y += b.y; v.z += b.z; v.w += b.w; }
+                            if (g.relu) {
+                                v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f);
+                                v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
+                            }
+                            const int64_t o = (crow + rr) * g.ldc + col;
+                            if (g.Cf) *reinterpret_cast<float4 *>(g.Cf + o) = v;
+                            if (g.Cb) {
+                                __nv_bfloat162 h[2] = {__floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
+                                *reinterpret_cast<uint2 *>(g.Cb + o) = *reinterpret_cast<const uint2 *>(h);
+                            }
+                        }
                     }
-                    if (g.bias) v += g.bias[col];
-                    if (g.relu) v = fmaxf(v, 0.f);
-                    if (g.Cf) g.Cf[(int64_t)row * g.ldc + col] = v;
-                    if (g.Cb) g.Cb[(int64_t)row * g.ldc + col] = __float2bfloat16_rn(v);
+                } else if (lane < cn) {
+                    const int col = n0 + c0 + lane;
+                    const float b = g.bias ? g.bias[col] : 0.f;
+                    for (int rr = 0; rr < rows; ++rr) {
+                        float v = st[rr * GEMM_EPI_LD + lane];
+                        if (g.bias) v += b;
+                        if (g.relu) v = fmaxf(v, 0.f);
+                        const int64_t o = (crow + rr) * g.ldc + col;
+                        if (g.Cf) g.Cf[o] = v;
+                        if (g.Cb) g.Cb[o] = __float2bfloat16_rn(v);
+                    }
                 }
             }
         }
     }
+    __syncwarp();
+    __syncthreads();
+    if (!mbar_wait(smem_u32(&bar_done), 0u) && g.status) atomicExch_system(g.status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SM::TMEM_COLS) : "memory");
 }
 
 // Sum split-K partials in a fixed order and apply the epilogue.
@@ -302,8 +389,20 @@ __global__ void k_gemm_reduce(const float *__restrict__ part, int split, int M, 
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)M * N) return;
     const int row = (int)(i / N), col = (int)(i % N);
+    // eight partials in flight, added in order (few outputs of many partials
+    // leave the loop waiting for one load at a time otherwise)
     float v = 0.f;
-    for (int z = 0; z < split; ++z) v += part[((int64_t)z * M + row) * ldc + col];
+    const float *p = part + (int64_t)row * ldc + col;
+    const int64_t step = (int64_t)M * ldc;
+    int z = 0;
+    for (; z + 8 <= split; z += 8) {
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = p[(z + j) * step];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v += x[j];
+    }
+    for (; z < split; ++z) v += p[z * step];
     if (bias) v += bias[col];
     if (relu) v = fmaxf(v, 0.f);
     if (Cf) Cf[(int64_t)row * ldc + col] = v;
@@ -350,19 +449,48 @@ static cudaError_t make_map(CUtensorMap *map, const __nv_bfloat16 *base, int row
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// CTAs of k_gemm_bf16<BN> that fit on the current device at once: by shared
+// memory and registers, and at most 512 TMEM columns to an SM.  0 on error.
 template <int BN>
-static cudaError_t gemm_t(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int lda, int ldb, const GemmArgs &g,
-                          cudaStream_t st)
+static int gemm_resident()
+{
+    constexpr int MAX_DEV = 64;
+    static std::atomic<int> cached[MAX_DEV];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return 0;
+    int c = cached[dev].load();
+    if (!c) {
+        int sms = 0, per_sm = 0;
+        if (cudaFuncSetAttribute(k_gemm_bf16<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)GemmSmem<BN>::TOTAL) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemm_bf16<BN>, GEMM_THREADS,
+                                                          GemmSmem<BN>::TOTAL) != cudaSuccess)
+            return 0;
+        const int by_tmem = 512 / (int)GemmSmem<BN>::TMEM_COLS;
+        c = sms * (per_sm < 1 ? 1 : per_sm < by_tmem ? per_sm : by_tmem);
+        cached[dev].store(c);
+    }
+    return c;
+}
+
+template <int BN>
+static cudaError_t gemm_t(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int lda, int ldb, GemmArgs g, cudaStream_t st)
 {
     CUtensorMap ma, mb;
     cudaError_t e = make_map(&ma, A, g.M, g.K, lda, GEMM_BM);
     if (e == cudaSuccess) e = make_map(&mb, B, g.N, g.K, ldb, BN);
     if (e != cudaSuccess) return e;
-    constexpr size_t SMEM = GemmSmem<BN>::TOTAL;
-    e = cudaFuncSetAttribute(k_gemm_bf16<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)ceil_div(g.M, GEMM_BM), (unsigned)ceil_div(g.N, BN), (unsigned)g.split_k);
-    k_gemm_bf16<BN><<<grid, GEMM_THREADS, SMEM, st>>>(ma, mb, g);
+    const int resident = gemm_resident<BN>();
+    if (resident <= 0) {
+        e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaErrorInvalidValue;
+    }
+    g.n_tn = (int)ceil_div(g.N, BN);
+    const int64_t tiles = ceil_div(g.M, GEMM_BM) * g.n_tn * g.split_k;
+    if (tiles > (int64_t)1 << 30) return cudaErrorInvalidValue;
+    g.n_tiles = (int)tiles;
+    k_gemm_bf16<BN><<<(unsigned)min64(tiles, resident), GEMM_THREADS, GemmSmem<BN>::TOTAL, st>>>(ma, mb, g);
     return cudaGetLastError();
 }
 
@@ -381,14 +509,23 @@ cudaError_t launch_gemm_bf16(const __nv_bfloat16 *A, const __nv_bfloat16 *B, con
         ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || (split_k > 1 && !partials))
         return cudaErrorInvalidValue;
     if (take_fault(FAULT_GEMM_WAIT)) inject = 1;
-    GemmArgs g{bias, Cf, Cb, M, N, K, ldc, relu, split_k, inject, status};
+    GemmArgs g{};
+    g.bias = bias; g.Cf = Cf; g.Cb = Cb;
+    g.M = M; g.N = N; g.K = K; g.ldc = ldc;
+    g.relu = relu; g.split_k = split_k; g.inject = inject; g.status = status;
     if (split_k > 1) {
         g.Cf = partials;
         g.Cb = nullptr;
         g.bias = nullptr;
         g.relu = 0;
     }
-    const int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
+    g.vec = N % 4 == 0 && ldc % 4 == 0 && ((uintptr_t)g.Cf & 15) == 0 && ((uintptr_t)g.Cb & 7) == 0;
+    // The widest tile that N fills, halved while that leaves fewer columns to
+    // the busiest SM: rounds of one tile an SM x BN is the time of the MMAs,
+    // and 16-row outputs of 1024 columns would run on 4 SMs at BN = 256.
+    int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
+    auto columns = [&](int bn) { return ceil_div(ceil_div(M, GEMM_BM) * ceil_div(N, bn) * split_k, 152) * bn; };
+    while (BN > 32 && columns(BN / 2) < columns(BN)) BN /= 2;
     cudaError_t e;
     switch (BN) {
     case 16: e = gemm_t<16>(A, B, lda, ldb, g, st); break;
