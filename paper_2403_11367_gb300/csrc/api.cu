@@ -135,13 +135,13 @@ struct reloc_ctx {
     DevBuf nvis, ninst, scores, degen, best, best_score, view_sel, flags;
     DevBuf bqueue;                       // the blend's work counter and heavy-tile list
     DevBuf hq, hrgb, hdepth;
-    DevBuf pnp_X, pnp_out;
+    DevBuf pnp_X;
     DevBuf gbuf, gcoef, gpart, gpose;    // NCC pose gradients
     // map training: render and dL/dC scratch, loss, parameter gradients, Adam moments
     DevBuf trgb, tgimg, tabc, tloss, tgrad, adam_m, adam_v;
     DevBuf tdep, talp, twarp, tjac, tgw, tgda, trel;     // re-projection loss
     int64_t adam_t = 0;
-    PinBuf pin, gemm_status;
+    PinBuf pin, gemm_status, pnp_out;
     double inst_ratio = 3.0;        // instance capacity per (view, subset Gaussian), learned
     // batch options
     int use_graph = 1;
@@ -254,12 +254,13 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
                       &ctx->qpart, &ctx->qstats, &ctx->nvis, &ctx->ninst, &ctx->scores, &ctx->degen,
                       &ctx->best, &ctx->best_score, &ctx->view_sel, &ctx->flags, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
                       &ctx->hdepth, &ctx->prop_in, &ctx->prop_seed, &ctx->prop_logits, &ctx->prop_idx,
-                      &ctx->prop_mrg, &ctx->prop_loss, &ctx->pnp_X, &ctx->pnp_out, &ctx->gbuf, &ctx->gcoef,
+                      &ctx->prop_mrg, &ctx->prop_loss, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
                       &ctx->gpart, &ctx->gpose};
     for (DevBuf *b : bufs) b->release();
     if (ctx->prop) proposal_destroy(ctx->prop);
     ctx->pin.release();
     ctx->gemm_status.release();
+    ctx->pnp_out.release();
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
@@ -1783,14 +1784,13 @@ extern "C" reloc_status reloc_refine_pnp(reloc_ctx *ctx, const double *pose_rend
             return fail(RELOC_ENUMERIC, "non-finite pose");
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
-    CKS(ctx->pnp_X.ensure(32 * (size_t)n_pairs + (256 << 10)));   // points, then per-block sums and state
-    CKS(ctx->pnp_out.ensure(sizeof(double) * 20));
+    CKS(ctx->pnp_X.ensure(32 * (size_t)n_pairs + (256 << 10)));   // points, then per-block sums
+    CKS(ctx->pnp_out.ensure(sizeof(double) * 20));                // pinned: the kernel writes the answer there
     CK(launch_refine_pnp(pose_render, pose_init, cam->fx, cam->fy, cam->cx, cam->cy, cam->width, cam->height,
                          depth_dev, alpha_dev, pairs_dev, n_pairs, o.max_iters, o.huber_px, o.alpha_min, o.tol,
-                         ctx->pnp_X.as<double>(), ctx->pnp_out.as<double>(), st));
-    double h[20];
-    CK(cudaMemcpyAsync(h, ctx->pnp_out.p, sizeof h, cudaMemcpyDeviceToHost, st));
+                         ctx->pnp_X.as<double>(), (double *)ctx->pnp_out.p, st));
     CK(cudaStreamSynchronize(st));
+    const double *h = (const double *)ctx->pnp_out.p;
     memset(out, 0, sizeof *out);
     memcpy(out->pose, h, sizeof(double) * 16);
     out->rms_px = h[16];
