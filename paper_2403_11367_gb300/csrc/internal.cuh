@@ -49,9 +49,11 @@ constexpr int SORT_THREADS = 256;
 constexpr int SORT_IPT = 8;
 constexpr int SORT_CHUNK = SORT_THREADS * SORT_IPT;   // 2048 items per block
 constexpr int RADIX = 256;
-// Tile binning (sort.cu): chunks of bin_chunk depth-ordered Gaussians.
-constexpr int BIN_CHUNK_MIN = 2048;
-constexpr int BIN_TILES_PER_CHUNK_STEP = 8192;        // bin_chunk grows by 2048 per 8192 tiles
+// Tile binning (sort.cu): chunks of bin_chunk depth-ordered Gaussians, 256 to
+// 2048 of them (more on very large tile grids).
+constexpr int BIN_CHUNK_MAX = 2048, BIN_CHUNK_MIN = 256;
+constexpr int64_t BIN_CHUNKS_WANTED = 4096;
+constexpr int BIN_TILES_PER_CHUNK_STEP = 8192;        // bin_chunk grows in proportion past 8192 tiles
 constexpr int TILE_COUNT_SMEM = 48 * 1024;            // difference-array band
 constexpr int TILE_EMIT_WARPS = 8;                    // tile rows per K4 block
 constexpr int TILE_EMIT_SMEM_MAX = 64 * 1024;         // slot counters: 8 rows x ntx <= 2048
@@ -129,13 +131,14 @@ cudaError_t launch_radix_pass(const RadixPass &p, cudaStream_t st);
 
 // K3: per chunk of each view's depth-ordered visible Gaussians (sorted_g,
 // n_vis[v] at vd_off[v]) the number covering each tile -> bhist[chunk][tile]
-// (n_chunks = cb_base[V], host copy); rectangles in depth order -> srect;
+// (n_chunks = cb_base[V], view_chunks = the most of one view, host copies);
+// rectangles in depth order -> srect;
 // then per view the chunk prefix per tile (in place), ranges[v][tile] =
 // [begin, end) of the tile's list relative to io_off[v] (empty [0, 0)) and
 // n_inst[v].  A view over its capacity sets *overflow.
 cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, const uint2 *rect, const Layout &L,
-                              const CamParams &cp, int n_chunks, uint2 *srect, uint32_t *bhist, int2 *ranges,
-                              uint32_t *n_inst, int *overflow, cudaStream_t st);
+                              const CamParams &cp, int n_chunks, int view_chunks, uint2 *srect, uint32_t *bhist,
+                              int2 *ranges, uint32_t *n_inst, int *overflow, cudaStream_t st);
 
 // K4: every (tile, Gaussian) instance into inst_gauss at io_off[v] + its slot,
 // each tile's list in (depth, index) order.  Views over capacity emit nothing.

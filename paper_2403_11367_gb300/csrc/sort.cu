@@ -351,20 +351,20 @@ k_tile_count(const uint32_t *__restrict__ sorted_g, const uint32_t *__restrict__
 // tile's start), totals -> ranges[v][tile].y; then a block per view scans
 // the totals in tile order into ranges[v][tile] = [begin, end) (empty tiles
 // [0, 0)) and n_inst[v].  The chunk prefix: a block per (view, 32 tiles),
-// eight threads per tile, each holding up to TCOL_SEG of the tile's chunks in
+// SEGS threads per tile, each holding up to TCOL_SEG of the tile's chunks in
 // registers (all its loads in flight at once), so a view's ~80 chunks are
-// scanned as eight short runs plus a prefix over the eight run totals.
+// scanned as eight short runs plus a prefix over the eight run totals, and the
+// hundreds of smaller chunks of a call of few views as 32 runs.
 constexpr int TCOL_TILES = 32;
-constexpr int TCOL_SEGS = 8;
-constexpr int TCOL_THREADS = TCOL_TILES * TCOL_SEGS;
 constexpr int TCOL_SEG = 16;                         // chunks per run in registers
 constexpr int TSCAN_THREADS = 1024;
 
-__global__ void __launch_bounds__(TCOL_THREADS, 4)
+template <int SEGS>
+__global__ void __launch_bounds__(TCOL_TILES * SEGS, SEGS > 8 ? 1 : 4)
 k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, uint32_t *__restrict__ bhist,
                   int2 *__restrict__ ranges)
 {
-    __shared__ uint32_t s_run[TCOL_SEGS][TCOL_TILES];
+    __shared__ uint32_t s_run[SEGS][TCOL_TILES];
     const int v = blockIdx.y;
     const int tl = threadIdx.x % TCOL_TILES, sg = threadIdx.x / TCOL_TILES;
     const int t = blockIdx.x * TCOL_TILES + tl;
@@ -373,7 +373,7 @@ k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, ui
     const int64_t nv = min64(n_vis[v], S);
     const int nch = (int)ceil_div(nv, cp.bin_chunk);
     uint32_t *h = bhist + (int64_t)nt * L.cb_base[v] + t;
-    const int per = (int)ceil_div(nch, TCOL_SEGS);      // chunks of this thread's run
+    const int per = (int)ceil_div(nch, SEGS);      // chunks of this thread's run
     const int c0 = sg * per, c1 = min(nch, c0 + per);
     uint32_t sum = 0;
     if (per <= TCOL_SEG) {                              // uniform over the block
@@ -395,10 +395,10 @@ k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, ui
                 hp[(int64_t)j * nt] = run;
                 run += x[j];
             }
-        if (sg == TCOL_SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
+        if (sg == SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
         return;
     }
-    // long views (more than TCOL_SEGS * TCOL_SEG chunks) or tiles past the
+    // long views (more than SEGS * TCOL_SEG chunks) or tiles past the
     // grid: runs summed first, then rewritten
     if (t < nt)
         for (int c = c0; c < c1; ++c) sum += h[(int64_t)c * nt];
@@ -412,7 +412,7 @@ k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, ui
         h[(int64_t)c * nt] = run;
         run += x;
     }
-    if (sg == TCOL_SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
+    if (sg == SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
 }
 
 __global__ void __launch_bounds__(TSCAN_THREADS)
@@ -438,8 +438,8 @@ k_tile_scan(Layout L, CamParams cp, int2 *__restrict__ ranges, uint32_t *__restr
 }
 
 cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, const uint2 *rect, const Layout &L,
-                              const CamParams &cp, int n_chunks, uint2 *srect, uint32_t *bhist, int2 *ranges,
-                              uint32_t *n_inst, int *overflow, cudaStream_t st)
+                              const CamParams &cp, int n_chunks, int view_chunks, uint2 *srect, uint32_t *bhist,
+                              int2 *ranges, uint32_t *n_inst, int *overflow, cudaStream_t st)
 {
     if (L.V <= 0) return cudaSuccess;
     if (n_chunks > 0) {
@@ -448,8 +448,13 @@ cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, c
         const size_t smem = 4 * (size_t)(band_rows + 1) * W;
         k_tile_count<<<n_chunks, BIN_THREADS, smem, st>>>(sorted_g, n_vis, rect, L, cp, band_rows, srect, bhist);
     }
-    k_tile_chunk_scan<<<dim3((unsigned)ceil_div(cp.n_tiles, TCOL_TILES), L.V), TCOL_THREADS, 0, st>>>(
-        n_vis, L, cp, bhist, ranges);
+    const dim3 cgrid((unsigned)ceil_div(cp.n_tiles, TCOL_TILES), L.V);
+    // by the chunks a view may have; about a third of them hold visible Gaussians,
+    // and the wide form costs the 64 views of 157 chunks 48 us more (147 for 99 us)
+    if (view_chunks <= 4 * 8 * TCOL_SEG)
+        k_tile_chunk_scan<8><<<cgrid, TCOL_TILES * 8, 0, st>>>(n_vis, L, cp, bhist, ranges);
+    else
+        k_tile_chunk_scan<32><<<cgrid, TCOL_TILES * 32, 0, st>>>(n_vis, L, cp, bhist, ranges);
     k_tile_scan<<<L.V, TSCAN_THREADS, 0, st>>>(L, cp, ranges, n_inst, overflow);
     return cudaGetLastError();
 }
@@ -474,7 +479,7 @@ cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, c
 // spans are spread over the lanes), and then cnt[x] += popc(M[x]).
 // k_tile_emit_smem: any row width, slots in shared memory, a lane per
 // column of each queued pair.
-constexpr int EMIT_STAGE = BIN_CHUNK_MIN;             // a whole chunk of the usual size: one barrier
+constexpr int EMIT_STAGE = BIN_CHUNK_MAX;             // a whole chunk of the usual size: one barrier
 constexpr int EMIT_FLAT_MAX_NTX = 256;
 constexpr int EMIT_Q = 256;                           // queue ring entries per warp (>= 31 + 128)
 constexpr int EMIT_JCAP = 4;                          // columns a pair's own lane writes
