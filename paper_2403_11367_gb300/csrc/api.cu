@@ -129,7 +129,7 @@ struct reloc_ctx {
     std::vector<int64_t> order;
     BlockIndex blocks;
     // workspace (sized for the largest sub-batch of a call)
-    DevBuf gidx, tables, rec, rect, dkey, k1a, v1a, k1b, v1b, hist1, chunk_sums, dtot;
+    DevBuf gidx, tables, rec, rect, dkey, kva, v1b, hist1, chunk_sums, dtot;
     DevBuf srect, bhist, inst, ranges, partials, qpart, qstats;
     // per-call results (all views / queries of the call)
     DevBuf nvis, ninst, scores, degen, best, best_score, view_sel, flags;
@@ -235,7 +235,7 @@ extern "C" reloc_status reloc_create(const reloc_config *cfg, int device, reloc_
         reloc_destroy(ctx);
         return fail(RELOC_ECUDA, "stream/event creation failed");
     }
-    if (configure_tile_kernels() != cudaSuccess) {
+    if (configure_sort_kernels() != cudaSuccess) {
         cudaGetLastError();
         reloc_destroy(ctx);
         return fail(RELOC_ECUDA, "kernel attribute setup failed");
@@ -249,7 +249,7 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
     if (!ctx) return RELOC_OK;
     cudaSetDevice(ctx->device);
     DevBuf *bufs[] = {&ctx->mean, &ctx->attr, &ctx->gidx, &ctx->tables, &ctx->rec, &ctx->rect,
-                      &ctx->dkey, &ctx->k1a, &ctx->v1a, &ctx->k1b, &ctx->v1b, &ctx->hist1, &ctx->chunk_sums,
+                      &ctx->dkey, &ctx->kva, &ctx->v1b, &ctx->hist1, &ctx->dtot, &ctx->chunk_sums,
                       &ctx->srect, &ctx->bhist, &ctx->inst, &ctx->ranges, &ctx->partials,
                       &ctx->qpart, &ctx->qstats, &ctx->nvis, &ctx->ninst, &ctx->scores, &ctx->degen,
                       &ctx->best, &ctx->best_score, &ctx->view_sel, &ctx->flags, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
@@ -520,7 +520,7 @@ struct CallOut {
 // A run of consecutive queries whose workspace fits the memory budget.
 struct SubBatch {
     int q0 = 0, q1 = 0, v0 = 0, v1 = 0;
-    int64_t S_tot = 0, VS = 0, VI = 0;
+    int64_t S_tot = 0, S_max = 0, VS = 0, VI = 0;      // S_max: the longest view's Gaussians
     int c1 = 0, cb = 0, cb_view = 0, pblk = 0, n_runs = 0;     // cb_view: binning chunks of the longest view
     std::vector<int32_t> view_q, c1_base, cb_base, q_view, q_pblk;
     std::vector<int64_t> vd_off, io_off, q_gsub, run_begin, run_off;
@@ -543,12 +543,12 @@ static int64_t inst_cap(const reloc_ctx *ctx, int64_t S, int64_t override_cap)
 }
 
 // Workspace bytes of one query: per view, the per-Gaussian arrays (records,
-// rectangle, tile count, depth key, two key/value radix buffers, depth-ordered
+// rectangle, depth key, a key/value sort buffer, the depth order, depth-ordered
 // rectangle, radix histograms), the instance list, ranges, NCC partials per
 // warp block and the per-chunk tile counts; plus the gathered subset.
 static int64_t query_bytes(int64_t S, int V, int64_t cap, const CamParams &cp)
 {
-    const int64_t per_view = S * 89 + cap * 4 + (int64_t)cp.n_tiles * 8 + (int64_t)blend_units(cp) * 24 +
+    const int64_t per_view = S * 85 + cap * 4 + (int64_t)cp.n_tiles * 8 + (int64_t)blend_units(cp) * 24 +
                              4 * (int64_t)cp.n_tiles * ceil_div(S, cp.bin_chunk) + 1024;
     return (int64_t)V * per_view + S * 4 + 4096;
 }
@@ -593,6 +593,7 @@ static void plan_batches(const reloc_ctx *ctx, const std::vector<QuerySpec> &qs,
             const QuerySpec &Qs = qs[sb.q0 + k];
             const int64_t cap = inst_cap(ctx, Qs.S, caps[sb.q0 + k]);
             sb.q_gsub[k + 1] = sb.q_gsub[k] + Qs.S;
+            sb.S_max = std::max(sb.S_max, Qs.S);
             sb.q_view[k + 1] = sb.q_view[k] + Qs.V;
             sb.q_pblk[k + 1] = sb.q_pblk[k] + (int32_t)ceil_div(Qs.S, PROJ_THREADS);
             sb.q_img[k] = Qs.img;
@@ -686,7 +687,12 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     stage_mark(ctx, sbi, RELOC_STAGE_DEPTH_SORT, st, capturing);
     CK(cudaMemsetAsync(nvis, 0, 4 * (size_t)L.V, st));
     CK(cudaMemsetAsync(ninst, 0, 4 * (size_t)L.V, st));
-    if (sb.c1 > 0) {
+    if (sb.c1 > 0 && sb.S_max <= DEPTH_SORT_CLUSTER_MAX) {
+        // the rectangles in depth order are written after the sort: their buffer serves as scratch
+        CK(launch_depth_sort(ctx->dkey.as<uint32_t>(), ctx->kva.as<uint2>(), ctx->srect.as<uint2>(),
+                             ctx->v1b.as<uint32_t>(), L, sb.S_max, nvis, st));
+        launches += 1;
+    } else if (sb.c1 > 0) {
         RadixPass p{};
         p.seg_off = L.vd_off;
         p.chunk_base = L.c1_base;
@@ -698,8 +704,8 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         uint32_t *dtot = ctx->dtot.as<uint32_t>();
         CK(cudaMemsetAsync(dtot, 0, 16 * (size_t)RADIX * L.V, st));
         p.dtot = dtot;
-        uint32_t *ka = ctx->k1a.as<uint32_t>(), *va = ctx->v1a.as<uint32_t>();
-        uint32_t *kb = ctx->k1b.as<uint32_t>(), *vb = ctx->v1b.as<uint32_t>();
+        uint32_t *ka = ctx->kva.as<uint32_t>(), *va = ka + sb.VS;
+        uint32_t *kb = ctx->srect.as<uint32_t>(), *vb = ctx->v1b.as<uint32_t>();
         // pass 0: dense (view, Gaussian) arrays; culled pairs are dropped
         p.keys_in = ctx->dkey.as<uint32_t>();
         p.vals_in = nullptr;
@@ -873,7 +879,9 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         // ---- workspace: the largest sub-batch --------------------------------
         int64_t S_tot = 1, VS = 1, VI = 1, c1 = 1, cb = 1, V = 1, Qm = 1;
         size_t tab = 0;
+        bool passes = false;            // a sub-batch whose depth sort takes a launch chain per pass
         for (auto &sb : sbs) {
+            passes = passes || sb.S_max > DEPTH_SORT_CLUSTER_MAX;
             S_tot = std::max(S_tot, sb.S_tot);
             VS = std::max(VS, sb.VS);
             VI = std::max(VI, sb.VI);
@@ -888,12 +896,12 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         CKS(ctx->rec.ensure(48 * (size_t)VS));
         CKS(ctx->rect.ensure(8 * (size_t)VS));
         CKS(ctx->dkey.ensure(4 * (size_t)VS));
-        CKS(ctx->k1a.ensure(4 * (size_t)VS));
-        CKS(ctx->v1a.ensure(4 * (size_t)VS));
-        CKS(ctx->k1b.ensure(4 * (size_t)VS));
+        CKS(ctx->kva.ensure(8 * (size_t)VS));
         CKS(ctx->v1b.ensure(4 * (size_t)VS));
-        CKS(ctx->hist1.ensure(4 * (size_t)RADIX * c1));
-        CKS(ctx->dtot.ensure(16 * (size_t)RADIX * V));
+        if (passes) {
+            CKS(ctx->hist1.ensure(4 * (size_t)RADIX * c1));
+            CKS(ctx->dtot.ensure(16 * (size_t)RADIX * V));
+        }
         CKS(ctx->srect.ensure(8 * (size_t)VS));
         CKS(ctx->bhist.ensure(4 * (size_t)cp.n_tiles * cb));
         CKS(ctx->inst.ensure(4 * (size_t)VI));

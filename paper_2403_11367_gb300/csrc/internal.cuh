@@ -110,6 +110,19 @@ cudaError_t launch_project(const float *mx, const float *my, const float *mz, co
                            const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
                            float4 *rec, uint2 *rect, uint32_t *dkey, cudaStream_t st);
 
+// Depth sort of every view's visible Gaussians in one launch: out[vd_off[v] + k]
+// = index of the k-th nearest (ties by index), n_vis[v] their number.  dkey:
+// dense depth keys, 0xFFFFFFFF where culled; bufA, bufB: scratch of one uint2
+// per (view, Gaussian); longest: the most Gaussians of one view.
+cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, const Layout &L,
+                              int64_t longest, uint32_t *n_vis, cudaStream_t st);
+// Calls with a view of more Gaussians than this take the passes below, one launch
+// chain each, over the whole GPU.  The line lies where a driving view sees about
+// a third of its subset: 64 views of 320k Gaussians (100k visible) 278 us in
+// clusters, 470 in passes; 64 views of 500k with 270k visible 928 and 819; one
+// view of 500k with 443k visible 110 and 82; of 2M with 1.8M visible 369 and 155.
+constexpr int64_t DEPTH_SORT_CLUSTER_MAX = (int64_t)1 << 20;
+
 // Stable LSD radix sort pass over segments (views).  Segment s holds
 // seg_off[s+1] - seg_off[s] slots at seg_off[s], of which len[s] are valid
 // (len null: all).  filt != null: pass over dense arrays keeping items with
@@ -146,8 +159,9 @@ cudaError_t launch_tile_emit(const uint32_t *sorted_g, const uint2 *srect, const
                              const uint32_t *n_inst, const uint32_t *bhist, const int2 *ranges, const Layout &L,
                              const CamParams &cp, int n_chunks, uint32_t *inst_gauss, cudaStream_t st);
 
-// Allow K4 its largest shared-memory footprint (once per device, before any capture).
-cudaError_t configure_tile_kernels();
+// Kernel attributes of the sort and binning kernels: K4's largest shared-memory
+// footprint, the depth sort's cluster size (once per device, before any capture).
+cudaError_t configure_sort_kernels();
 
 // Pose refinement by PnP on one view's depth (pnp.cu), one cooperative launch:
 // out[20] = pose[16], rms, cost, n_used, iterations (device or pinned host

@@ -6,7 +6,9 @@
 // list:
 //   1. a stable LSD radix sort of the visible (view, Gaussian) pairs by the
 //      float32 depth bit pattern (4 passes of 8 bits; the first pass also
-//      drops invisible pairs, so compaction costs nothing extra);
+//      drops invisible pairs, so compaction costs nothing extra): one
+//      thread-block cluster per view runs all four passes (k_depth_sort), and
+//      views of more Gaussians than that suits take a launch chain per pass;
 //   2. per chunk of that depth order, tile coverage counts (K3: 2D difference
 //      arrays), scanned into each tile's list start and each chunk's slot in it;
 //   3. emission of every (tile, Gaussian) instance straight into its slot, a
@@ -18,6 +20,8 @@
 // Every per-view array sits at a host-planned offset with a host-planned
 // capacity, and chunk tables map a block to its view and chunk, so valid
 // lengths stay in device memory: no host round trip between stages.
+#include <cooperative_groups.h>
+
 #include "internal.cuh"
 
 namespace reloc {
@@ -61,7 +65,211 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *s_tmp,
     return r;
 }
 
-// ------------------------------------------------------------ upsweep ------
+// --------------------------------------------- depth sort, one launch ------
+// A cluster of C blocks (1 .. 16, a power of two) per view runs the four passes
+// of the stable LSD sort.  Per pass, block r takes the r-th share of the items
+// and warp w the w-th share of those:
+//   count    each warp counts its items' digits in its own shared-memory
+//            histogram;
+//   offsets  the blocks' digit counts are read across the cluster (distributed
+//            shared memory), and digit d of warp w of block r starts at the
+//            total of the smaller digits, plus digit d of the blocks before r,
+//            plus digit d of the warps before w;
+//   scatter  each warp walks its items again in order, 32 at a time, ranks the
+//            lanes of equal digit by ballots and writes (key, index) straight
+//            to its place.
+// Cluster barriers (release / acquire, so they order the items in global memory
+// too) stand between the passes.  Pass 0 reads the view's dense depth keys and
+// drops the culled ones, the last pass writes indices only.
+// What bounds it: for few views the latency of the four dependent passes (12
+// launches of 4 to 7 us each as a chain: 76 us for one driving view of 320k keys,
+// 104k of them visible, 50 us so; 72 and 27 us for one of 10k), for many the
+// scattered 8-byte stores, about one lane a clock and SM (64 driving views 470 us
+// as a chain, 278 us so).  The first items of each lane stay in registers
+// between count and scatter; the cluster's counts are read with all loads in
+// flight (one after the other they cost more than the pass's items: 88 us for the
+// one driving view).  Shared memory holds counters only, so a view's visible count
+// is not bounded by it.
+constexpr int DS_MAX_CLUSTER = 16;
+constexpr int DS_WIDE_VIEWS = 8;
+constexpr int DS_KEPT0 = 16, DS_KEPT = 8;            // items per lane kept in registers between count and scatter
+constexpr int DS_UNROLL = 4;                         // further items per lane in flight
+
+template <int NW>
+struct DepthSortShared {
+    uint32_t w[NW][RADIX];                           // a warp's digit counts, then its running offsets
+    uint32_t cnt[RADIX];                             // the block's digit counts, read by the whole cluster
+    uint32_t tmp[33];
+};
+
+// One pass over n items: of dense keys (FIRST: culled ones dropped, values the
+// positions) or (key, value) pairs, to pairs or (LAST) values.  Returns the
+// items kept.
+template <int NW, bool FIRST, bool LAST>
+__device__ __forceinline__ uint32_t depth_sort_pass(DepthSortShared<NW> &sm, uint32_t n, int shift,
+                                                    const uint32_t *__restrict__ keys, const uint2 *src, uint2 *dst,
+                                                    uint32_t *out)
+{
+    namespace cg = cooperative_groups;
+    constexpr int KEPT = FIRST ? DS_KEPT0 : DS_KEPT;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = lanemask_lt();
+    uint32_t *const sw = sm.w[warp];
+    // this block's and this warp's shares, whole rounds of 32
+    const uint32_t per_b = ((n + C - 1) / C + 31) / 32 * 32;
+    const uint32_t b0 = min(n, rank * per_b), b1 = min(n, b0 + per_b);
+    const uint32_t per_w = ((b1 - b0 + NW - 1) / NW + 31) / 32 * 32;
+    const uint32_t w0 = min(b1, b0 + warp * per_w), w1 = min(b1, w0 + per_w);
+    auto load = [&](uint32_t i, uint2 &t) {
+        if (i < w1) {
+            if (FIRST) t.x = __ldg(keys + i);
+            else t = src[i];
+        }
+    };
+    // digit of item i (RADIX: none)
+    auto digit = [&](uint32_t i, const uint2 &t) -> uint32_t {
+        if (i >= w1 || (FIRST && t.x == 0xFFFFFFFFu)) return (uint32_t)RADIX;
+        return (t.x >> shift) & 255u;
+    };
+    uint2 kept[KEPT];
+#pragma unroll
+    for (int u = 0; u < KEPT; ++u) load(w0 + lane + 32 * u, kept[u]);
+    for (int d = lane; d < RADIX; d += 32) sw[d] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < KEPT; ++u) {
+        const uint32_t d = digit(w0 + lane + 32 * u, kept[u]);
+        if (d != (uint32_t)RADIX) atomicAdd(sw + d, 1u);
+    }
+    for (uint32_t i = w0 + lane + 32 * KEPT; i < w1; i += 32 * DS_UNROLL) {
+        uint2 t[DS_UNROLL];
+#pragma unroll
+        for (int u = 0; u < DS_UNROLL; ++u) load(i + 32 * u, t[u]);
+#pragma unroll
+        for (int u = 0; u < DS_UNROLL; ++u) {
+            const uint32_t d = digit(i + 32 * u, t[u]);
+            if (d != (uint32_t)RADIX) atomicAdd(sw + d, 1u);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < RADIX) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) c += sm.w[w][threadIdx.x];
+        sm.cnt[threadIdx.x] = c;
+    }
+    cl.sync();
+    uint32_t total = 0, before = 0;
+    if (threadIdx.x < RADIX) {
+        uint32_t c[DS_MAX_CLUSTER];                  // all the remote loads in flight
+#pragma unroll
+        for (int r = 0; r < DS_MAX_CLUSTER; ++r) c[r] = r < C ? cl.map_shared_rank(sm.cnt, r)[threadIdx.x] : 0u;
+#pragma unroll
+        for (int r = 0; r < DS_MAX_CLUSTER; ++r) {
+            before += r < rank ? c[r] : 0u;
+            total += c[r];
+        }
+    }
+    uint32_t all;
+    uint32_t run = block_excl_scan(total, sm.tmp, &all) + before;
+    if (threadIdx.x < RADIX) {
+        uint32_t c[NW];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) c[w] = sm.w[w][threadIdx.x];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            sm.w[w][threadIdx.x] = run;
+            run += c[w];
+        }
+    }
+    __syncthreads();
+    auto place = [&](uint32_t i, const uint2 &t) {
+        const uint32_t d = digit(i, t);
+        // lanes holding the same digit (or none): the intersection of nine
+        // ballots, one per bit of d (0 .. RADIX)
+        unsigned peers = 0xffffffffu;
+#pragma unroll
+        for (int b = 0; b < 9; ++b) {
+            const bool set = ((d >> b) & 1u) != 0u;
+            const unsigned bal = __ballot_sync(0xffffffffu, set);
+            peers &= set ? bal : ~bal;
+        }
+        const bool valid = d != (uint32_t)RADIX;
+        uint32_t at = 0;
+        if (valid) at = sw[d];
+        __syncwarp();
+        if (valid && (peers & lt) == 0) sw[d] = at + __popc(peers);
+        __syncwarp();
+        if (valid) {
+            at += __popc(peers & lt);
+            if (LAST) out[at] = t.y;
+            else dst[at] = FIRST ? make_uint2(t.x, i) : t;
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < KEPT; ++u)
+        if (w0 + 32 * u < w1) place(w0 + lane + 32 * u, kept[u]);        // uniform over the warp
+    for (uint32_t i = w0 + 32 * KEPT; i < w1; i += 32 * DS_UNROLL) {
+        uint2 t[DS_UNROLL];
+#pragma unroll
+        for (int u = 0; u < DS_UNROLL; ++u) load(i + lane + 32 * u, t[u]);
+#pragma unroll
+        for (int u = 0; u < DS_UNROLL; ++u)
+            if (i + 32 * u < w1) place(i + lane + 32 * u, t[u]);
+    }
+    cl.sync();                                       // items written; the counts may be rewritten (and the block may exit)
+    return all;
+}
+
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 16 ? 2 : 1)
+k_depth_sort(const uint32_t *__restrict__ dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, Layout L, uint32_t *n_vis)
+{
+    __shared__ DepthSortShared<NW> sm;
+    const int C = (int)cooperative_groups::this_cluster().num_blocks();
+    const int v = blockIdx.x / C;
+    const int64_t off = L.vd_off[v];
+    uint2 *const A = bufA + off, *const B = bufB + off;
+    uint32_t n = (uint32_t)(L.vd_off[v + 1] - off);
+    n = depth_sort_pass<NW, true, false>(sm, n, 0, dkey + off, nullptr, A, nullptr);
+    if (blockIdx.x % C == 0 && threadIdx.x == 0) n_vis[v] = n;
+    depth_sort_pass<NW, false, false>(sm, n, 8, nullptr, A, B, nullptr);
+    depth_sort_pass<NW, false, false>(sm, n, 16, nullptr, B, A, nullptr);
+    depth_sort_pass<NW, false, true>(sm, n, 24, nullptr, A, nullptr, out + off);
+}
+
+cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, const Layout &L,
+                              int64_t longest, uint32_t *n_vis, cudaStream_t st)
+{
+    if (L.V <= 0) return cudaSuccess;
+    // one block per 2048 keys of the longest view, at most the whole cluster, and
+    // half of it once the views alone fill the GPU: 64 driving views 278 us at 8
+    // blocks, 339 at 16, 298 at 4; 16 views 153 at 16, 168 at 8; one view 50 at
+    // 16, 77 at 8; a view of 10k keys 27 at 8, 35 at 2
+    const int most = L.V <= 32 ? DS_MAX_CLUSTER : DS_MAX_CLUSTER / 2;
+    int C = 1;
+    while (C < most && (int64_t)C * 2048 < longest) C *= 2;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(C * L.V));
+    const bool wide = L.V <= DS_WIDE_VIEWS;
+    cfg.blockDim = dim3(wide ? 1024 : 512);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return wide ? cudaLaunchKernelEx(&cfg, k_depth_sort<32>, dkey, bufA, bufB, out, L, n_vis)
+                : cudaLaunchKernelEx(&cfg, k_depth_sort<16>, dkey, bufA, bufB, out, L, n_vis);
+}
+
+// --------------------------------------- depth sort, launches per pass -----
+// For views of more than DEPTH_SORT_CLUSTER_MAX Gaussians, whose passes need
+// the whole GPU: upsweep, digit offsets and scatter over SORT_CHUNK items a
+// block.
 // Per chunk digit counts -> hist[s][d][k] (digit-major inside a segment, so
 // one exclusive scan of the segment's block gives every chunk's offsets).
 // Each key adds 1 to its warp's own histogram with a shared-memory atomic;
@@ -844,8 +1052,11 @@ cudaError_t launch_tile_emit(const uint32_t *sorted_g, const uint2 *srect, const
     return cudaGetLastError();
 }
 
-cudaError_t configure_tile_kernels()
+cudaError_t configure_sort_kernels()
 {
+    cudaError_t e = cudaFuncSetAttribute(k_depth_sort<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_depth_sort<32>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_tile_emit_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_EMIT_SMEM_MAX);
 }
 
