@@ -141,7 +141,7 @@ struct reloc_ctx {
     DevBuf trgb, tgimg, tabc, tloss, tgrad, adam_m, adam_v;
     DevBuf tdep, talp, twarp, tjac, tgw, tgda, trel;     // re-projection loss
     int64_t adam_t = 0;
-    PinBuf pin, gemm_status, pnp_out;
+    PinBuf pin, gemm_status, pnp_out, prop_loss;
     double inst_ratio = 3.0;        // instance capacity per (view, subset Gaussian), learned
     // batch options
     int use_graph = 1;
@@ -159,7 +159,7 @@ struct reloc_ctx {
     ProposalNet *prop = nullptr;
     int prop_enabled = 0, prop_k = 8;
     float prop_margin = 0.f;
-    DevBuf prop_in, prop_seed, prop_logits, prop_idx, prop_mrg, prop_loss;
+    DevBuf prop_in, prop_seed, prop_logits, prop_idx, prop_mrg;
     // profiling
     bool prof = false;
     std::vector<cudaEvent_t> ev;    // (RELOC_STAGE_COUNT + 1) per sub-batch
@@ -254,13 +254,14 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
                       &ctx->qpart, &ctx->qstats, &ctx->nvis, &ctx->ninst, &ctx->scores, &ctx->degen,
                       &ctx->best, &ctx->best_score, &ctx->view_sel, &ctx->flags, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
                       &ctx->hdepth, &ctx->prop_in, &ctx->prop_seed, &ctx->prop_logits, &ctx->prop_idx,
-                      &ctx->prop_mrg, &ctx->prop_loss, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
+                      &ctx->prop_mrg, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
                       &ctx->gpart, &ctx->gpose};
     for (DevBuf *b : bufs) b->release();
     if (ctx->prop) proposal_destroy(ctx->prop);
     ctx->pin.release();
     ctx->gemm_status.release();
     ctx->pnp_out.release();
+    ctx->prop_loss.release();
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
@@ -1208,12 +1209,10 @@ static reloc_status apply_proposal(reloc_ctx *ctx, std::vector<QuerySpec> &qs, c
                    ctx->prop_mrg.as<float>(), st));
     std::vector<int32_t> idx((size_t)Ql * ctx->prop_k);
     std::vector<float> mrg(Ql);
-    int status = 0;
     CK(cudaMemcpyAsync(idx.data(), ctx->prop_idx.p, 4 * idx.size(), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(mrg.data(), ctx->prop_mrg.p, 4 * (size_t)Ql, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&status, proposal_status(ctx->prop), 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (status) return fail(RELOC_ETIMEOUT, "proposal: a tensor-core wait gave up");
+    if (proposal_status(ctx->prop)) return fail(RELOC_ETIMEOUT, "proposal: a tensor-core wait gave up");
     // (d) the candidate subsets
     for (int j = 0; j < Ql; ++j) {
         QuerySpec &q = qs[sel[j]];
@@ -1504,16 +1503,12 @@ extern "C" reloc_status reloc_proposal_train_step(reloc_ctx *ctx, const uint16_t
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CKS(ctx->prop_loss.ensure(4 * (size_t)batch));
-    CK(proposal_train_step(ctx->prop, (const __nv_bfloat16 *)inputs_dev, labels_dev, batch, lr, update != 0,
-                           ctx->prop_loss.as<float>(), st));
-    std::vector<float> rows(batch);
-    int status = 0;
-    CK(cudaMemcpyAsync(rows.data(), ctx->prop_loss.p, 4 * (size_t)batch, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&status, proposal_status(ctx->prop), 4, cudaMemcpyDeviceToHost, st));
+    float *rows = (float *)ctx->prop_loss.p;             // pinned: the loss kernel writes the rows there
+    CK(proposal_train_step(ctx->prop, (const __nv_bfloat16 *)inputs_dev, labels_dev, batch, lr, update != 0, rows, st));
     CK(cudaStreamSynchronize(st));
-    if (status) return fail(RELOC_ETIMEOUT, "proposal: a tensor-core wait gave up");
+    if (proposal_status(ctx->prop)) return fail(RELOC_ETIMEOUT, "proposal: a tensor-core wait gave up");
     double sum = 0;
-    for (float r : rows) sum += r;
+    for (int b = 0; b < batch; ++b) sum += rows[b];
     if (loss_host) *loss_host = (float)(sum / batch);
     return RELOC_OK;
 }

@@ -38,110 +38,51 @@ cudaError_t launch_downsample_gray(const float *img, int H, int W, int f, int ch
 }
 
 // im2col for a 3x3 / stride 2 / pad 1 convolution: X [B][H][W][C] ->
-// col [B*Ho*Wo][Kp], zero beyond K = 9 C.
-__global__ void k_im2col(const __nv_bfloat16 *__restrict__ x, int B, int H, int W, int C, int Ho, int Wo, int Kp,
-                         __nv_bfloat16 *__restrict__ col)
+// col [B*Ho*Wo][Kp], zero beyond K = 9 C.  A thread writes eight columns, 16
+// bytes: eight channels of one tap, or for the two-channel input four taps.
+// Bound by its writes (211 MB for the five layers at batch 256; one value a
+// thread took 650 us there).
+constexpr int COL_THREADS = 256;
+__global__ void __launch_bounds__(COL_THREADS)
+k_im2col(const __nv_bfloat16 *__restrict__ x, int M, int H, int W, int C, int Ho, int Wo, int Kp,
+         __nv_bfloat16 *__restrict__ col)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)B * Ho * Wo * Kp;
-    if (i >= total) return;
-    const int k = (int)(i % Kp);
-    const int64_t row = i / Kp;
-    const int ox = (int)(row % Wo), oy = (int)((row / Wo) % Ho), b = (int)(row / ((int64_t)Wo * Ho));
-    __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-    if (k < 9 * C) {
-        const int ci = k % C, kk = k / C, ky = kk / 3, kx = kk % 3;
-        const int y = 2 * oy - 1 + ky, xx = 2 * ox - 1 + kx;
-        if (y >= 0 && y < H && xx >= 0 && xx < W) v = x[(((int64_t)b * H + y) * W + xx) * C + ci];
+    const int G = Kp / 8, rows = COL_THREADS / G;         // groups of a row, rows of a block
+    const int r = threadIdx.x / G, g = threadIdx.x - r * G;
+    const int64_t row64 = (int64_t)blockIdx.x * rows + r;
+    if (r >= rows || row64 >= M) return;
+    const int row = (int)row64;
+    const int ox = row % Wo, t = row / Wo, oy = t % Ho, b = t / Ho;
+    const __nv_bfloat16 *xb = x + (int64_t)b * H * W * C;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (C == 2) {
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int tap = 4 * g + j, y = 2 * oy - 1 + tap / 3, xx = 2 * ox - 1 + tap % 3;
+            if (tap < 9 && y >= 0 && y < H && xx >= 0 && xx < W)
+                w[j] = *reinterpret_cast<const uint32_t *>(xb + ((int64_t)y * W + xx) * 2);
+        }
+        v = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+        const int k = 8 * g, tap = k / C, ci = k - tap * C;
+        const int y = 2 * oy - 1 + tap / 3, xx = 2 * ox - 1 + tap % 3;
+        if (tap < 9 && y >= 0 && y < H && xx >= 0 && xx < W)
+            v = *reinterpret_cast<const uint4 *>(xb + ((int64_t)y * W + xx) * C + ci);
     }
-    col[i] = v;
+    *reinterpret_cast<uint4 *>(col + row64 * Kp + 8 * g) = v;
 }
 
+// C 2 or a multiple of 8; Kp a multiple of 8, at most 8 * 256; x on 4 (C = 2) or 16 bytes.
 cudaError_t launch_im2col(const __nv_bfloat16 *x, int B, int H, int W, int C, int Ho, int Wo, int Kp,
                           __nv_bfloat16 *col, cudaStream_t st)
 {
-    const int64_t n = (int64_t)B * Ho * Wo * Kp;
-    k_im2col<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(x, B, H, W, C, Ho, Wo, Kp, col);
+    if ((C != 2 && C % 8) || Kp % 8 || Kp / 8 > COL_THREADS) return cudaErrorInvalidValue;
+    const int M = B * Ho * Wo;
+    k_im2col<<<(unsigned)ceil_div(M, COL_THREADS / (Kp / 8)), COL_THREADS, 0, st>>>(x, M, H, W, C, Ho, Wo, Kp, col);
     return cudaGetLastError();
 }
 
-// col2im (gather form, fixed summation order): dX[b][y][x][c] = sum over the
-// (ky, kx) whose output position (oy, ox) with y = 2 oy - 1 + ky,
-// x = 2 ox - 1 + kx lies in the output, of dcol[(b, oy, ox)][(ky, kx, c)].
-__global__ void k_col2im(const float *__restrict__ dcol, int B, int H, int W, int C, int Ho, int Wo, int Kp,
-                         __nv_bfloat16 *__restrict__ dx_bf, float *__restrict__ dx_f)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)B * H * W * C;
-    if (i >= total) return;
-    const int c = (int)(i % C);
-    const int64_t p = i / C;
-    const int x = (int)(p % W), y = (int)((p / W) % H), b = (int)(p / ((int64_t)W * H));
-    float s = 0.f;
-    for (int ky = 0; ky < 3; ++ky) {
-        const int ty = y + 1 - ky;
-        if (ty < 0 || (ty & 1)) continue;
-        const int oy = ty >> 1;
-        if (oy >= Ho) continue;
-        for (int kx = 0; kx < 3; ++kx) {
-            const int tx = x + 1 - kx;
-            if (tx < 0 || (tx & 1)) continue;
-            const int ox = tx >> 1;
-            if (ox >= Wo) continue;
-            s += dcol[(((int64_t)b * Ho + oy) * Wo + ox) * Kp + (ky * 3 + kx) * C + c];
-        }
-    }
-    if (dx_bf) dx_bf[i] = __float2bfloat16_rn(s);
-    if (dx_f) dx_f[i] = s;
-}
-
-cudaError_t launch_col2im(const float *dcol, int B, int H, int W, int C, int Ho, int Wo, int Kp, __nv_bfloat16 *dx_bf,
-                          float *dx_f, cudaStream_t st)
-{
-    const int64_t n = (int64_t)B * H * W * C;
-    k_col2im<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(dcol, B, H, W, C, Ho, Wo, Kp, dx_bf, dx_f);
-    return cudaGetLastError();
-}
-
-// out[c][r] = in[r][c] for r < R, c < Cc; out is Cp rows of Rp values (zero
-// padding, Rp >= R, Cp >= Cc) with row stride ldo >= Rp.  in: BF16 or FP32
-// (converted).
-template <typename T>
-__global__ void k_transpose(const T *__restrict__ in, int R, int Cc, int ld_in, __nv_bfloat16 *__restrict__ out, int Rp,
-                            int Cp, int ldo)
-{
-    __shared__ float t[32][33];
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int r = r0 + j, c = c0 + threadIdx.x;
-        float v = 0.f;
-        if (r < R && c < Cc) v = (float)in[(int64_t)r * ld_in + c];
-        t[j][threadIdx.x] = v;
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int c = c0 + j, r = r0 + threadIdx.x;
-        if (c < Cp && r < Rp) out[(int64_t)c * ldo + r] = __float2bfloat16_rn(t[threadIdx.x][j]);
-    }
-}
-
-cudaError_t launch_transpose_bf16(const __nv_bfloat16 *in, int R, int Cc, int ld_in, __nv_bfloat16 *out, int Rp, int Cp,
-                                  cudaStream_t st, int ldo)
-{
-    dim3 grid((unsigned)ceil_div(Cp, 32), (unsigned)ceil_div(Rp, 32));
-    k_transpose<__nv_bfloat16><<<grid, dim3(32, 8), 0, st>>>(in, R, Cc, ld_in, out, Rp, Cp, ldo > 0 ? ldo : Rp);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_transpose_f32(const float *in, int R, int Cc, int ld_in, __nv_bfloat16 *out, int Rp, int Cp,
-                                 cudaStream_t st)
-{
-    dim3 grid((unsigned)ceil_div(Cp, 32), (unsigned)ceil_div(Rp, 32));
-    k_transpose<float><<<grid, dim3(32, 8), 0, st>>>(in, R, Cc, ld_in, out, Rp, Cp, Rp);
-    return cudaGetLastError();
-}
-
-// d (FP32) *= (y > 0), written as BF16 (the gradient through a ReLU).
 // A backward signal carried as two BF16 terms: out [M][2N] holds hi =
 // bf16(x) in columns 0..N-1 and lo = bf16(x - hi) in N..2N-1, so hi + lo
 // keeps ~16 significant bits of x and the GEMMs that contract it (over 2N
@@ -152,29 +93,122 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &hi, __nv_bflo
     lo = __float2bfloat16_rn(x - __bfloat162float(hi));
 }
 
-// ReLU backward of d [M][N] at the stored activations y, split into hi | lo.
-__global__ void k_relu_back(const float *__restrict__ d, const __nv_bfloat16 *__restrict__ y, int64_t M, int N,
-                            __nv_bfloat16 *__restrict__ out)
+// Gradient through a ReLU at the stored activations y [M][N], split into hi | lo,
+// with the bias gradient's per-block column sums (of hi + lo) in part[block][N].
+// The incoming gradient is d [M][N] (C2I false), or the col2im of dcol (true):
+// row p = (b, y, x) of the layer's input sums, over the (ky, kx) in order whose
+// output position (oy, ox) with y = 2 oy - 1 + ky, x = 2 ox - 1 + kx lies in the
+// output, dcol[(b, oy, ox)][(ky, kx, c)].  A thread takes four columns of every
+// `step`-th row, so rows are read and written whole, the col2im's result never
+// goes to memory, and the sums cost no pass of their own (as separate kernels of
+// one value a thread, and a block per column for the sums: 254 + 148 + 733 us of
+// a step of batch 256).
+struct Col2Im {
+    int H, W, Ho, Wo, Kp;
+};
+constexpr int RB_THREADS = 256;
+template <bool C2I>
+__global__ void __launch_bounds__(RB_THREADS)
+k_relu_back(const float *__restrict__ d, Col2Im g, const __nv_bfloat16 *__restrict__ y, int M, int N,
+            __nv_bfloat16 *__restrict__ out, float *__restrict__ part)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M * N) return;
-    const int64_t r = i / N;
-    const int c = (int)(i - r * N);
-    __nv_bfloat16 hi, lo;
-    split_bf16((float)y[i] > 0.f ? d[i] : 0.f, hi, lo);
-    out[r * 2 * N + c] = hi;
-    out[r * 2 * N + N + c] = lo;
+    extern __shared__ float4 s_sum[];                     // [rows of a block][N / 4]
+    const int NG = N / 4, rows = RB_THREADS / NG > 0 ? RB_THREADS / NG : 1;
+    const int gpt = NG > RB_THREADS ? NG / RB_THREADS : 1;   // column groups a thread walks (N a multiple of 1024 then)
+    const int r = threadIdx.x / (NG < RB_THREADS ? NG : RB_THREADS);
+    const int c0 = threadIdx.x - r * NG;
+    for (int q = 0; q < gpt; ++q) {
+        const int c = (NG < RB_THREADS ? c0 : (int)threadIdx.x + q * RB_THREADS) * 4;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows)
+            for (int64_t row = (int64_t)blockIdx.x * rows + r; row < M; row += (int64_t)gridDim.x * rows) {
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (C2I) {
+                    const int p = (int)row, px = p % g.W, t = p / g.W, py = t % g.H, b = t / g.H;
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky) {
+                        const int ty = py + 1 - ky, oy = ty >> 1;
+                        if ((ty & 1) || oy < 0 || oy >= g.Ho) continue;
+#pragma unroll
+                        for (int kx = 0; kx < 3; ++kx) {
+                            const int tx = px + 1 - kx, ox = tx >> 1;
+                            if ((tx & 1) || ox < 0 || ox >= g.Wo) continue;
+                            const float4 v = __ldg(reinterpret_cast<const float4 *>(
+                                d + (((int64_t)b * g.Ho + oy) * g.Wo + ox) * g.Kp + (ky * 3 + kx) * N + c));
+                            x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
+                        }
+                    }
+                } else {
+                    x = __ldg(reinterpret_cast<const float4 *>(d + row * N + c));
+                }
+                const uint2 yb = __ldg(reinterpret_cast<const uint2 *>(y + row * N + c));
+                const __nv_bfloat162 y01 = *reinterpret_cast<const __nv_bfloat162 *>(&yb.x);
+                const __nv_bfloat162 y23 = *reinterpret_cast<const __nv_bfloat162 *>(&yb.y);
+                __nv_bfloat162 h[2], l[2];
+                split_bf16((float)y01.x > 0.f ? x.x : 0.f, h[0].x, l[0].x);
+                split_bf16((float)y01.y > 0.f ? x.y : 0.f, h[0].y, l[0].y);
+                split_bf16((float)y23.x > 0.f ? x.z : 0.f, h[1].x, l[1].x);
+                split_bf16((float)y23.y > 0.f ? x.w : 0.f, h[1].y, l[1].y);
+                sum.x += (float)h[0].x + (float)l[0].x;
+                sum.y += (float)h[0].y + (float)l[0].y;
+                sum.z += (float)h[1].x + (float)l[1].x;
+                sum.w += (float)h[1].y + (float)l[1].y;
+                __nv_bfloat16 *o = out + row * 2 * N + c;
+                *reinterpret_cast<uint2 *>(o) = *reinterpret_cast<const uint2 *>(h);
+                *reinterpret_cast<uint2 *>(o + N) = *reinterpret_cast<const uint2 *>(l);
+            }
+        if (rows == 1) {
+            *reinterpret_cast<float4 *>(part + (int64_t)blockIdx.x * N + c) = sum;
+            continue;
+        }
+        if (r < rows) s_sum[r * NG + c / 4] = sum;
+        __syncthreads();
+        if (r == 0) {
+            for (int k = 1; k < rows; ++k) {
+                const float4 v = s_sum[k * NG + c / 4];
+                sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+            }
+            *reinterpret_cast<float4 *>(part + (int64_t)blockIdx.x * N + c) = sum;
+        }
+    }
 }
 
-cudaError_t launch_relu_back(const float *d, const __nv_bfloat16 *y, int64_t M, int N, __nv_bfloat16 *out,
-                             cudaStream_t st)
+// db[c] = sum of part[0 .. n_part)[c], in a fixed order: eight runs a column.
+__global__ void __launch_bounds__(256) k_colsum_final(const float *__restrict__ part, int n_part, int N, float *__restrict__ db)
 {
-    const int64_t n = M * N;
-    k_relu_back<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(d, y, M, N, out);
+    __shared__ float s[8][32];
+    const int c = blockIdx.x * 32 + (threadIdx.x & 31), run = threadIdx.x >> 5;
+    float a = 0.f;
+    if (c < N)
+        for (int k = run; k < n_part; k += 8) a += part[(int64_t)k * N + c];
+    s[run][threadIdx.x & 31] = a;
+    __syncthreads();
+    if (run == 0 && c < N) {
+        for (int k = 1; k < 8; ++k) a += s[k][threadIdx.x];
+        db[c] = a;
+    }
+}
+
+// ReLU backward into out [M][2N] (hi | lo) and the bias gradient db [N].  d
+// [M][N], or with Ho > 0 the next layer's dcol [B*Ho*Wo][Kp], M = B*H*W.  N a
+// multiple of 4, and of 1024 above 1024.  part: RELU_BACK_BLOCKS * N floats.
+cudaError_t launch_relu_back(const float *d, int H, int W, int Ho, int Wo, int Kp, const __nv_bfloat16 *y, int M, int N,
+                             __nv_bfloat16 *out, float *part, float *db, cudaStream_t st)
+{
+    const int NG = N / 4;
+    if (M <= 0 || N % 4 || (NG > RB_THREADS && NG % RB_THREADS)) return cudaErrorInvalidValue;
+    const int rows = NG < RB_THREADS ? RB_THREADS / NG : 1;
+    const int blocks = (int)min64(ceil_div(M, rows), RELU_BACK_BLOCKS);
+    const size_t smem = rows > 1 ? sizeof(float4) * rows * NG : 0;
+    const Col2Im g{H, W, Ho, Wo, Kp};
+    if (Ho > 0) k_relu_back<true><<<blocks, RB_THREADS, smem, st>>>(d, g, y, M, N, out, part);
+    else k_relu_back<false><<<blocks, RB_THREADS, smem, st>>>(d, g, y, M, N, out, part);
+    k_colsum_final<<<(unsigned)ceil_div(N, 32), 256, 0, st>>>(part, blocks, N, db);
     return cudaGetLastError();
 }
 
-// db[c] = sum over the R rows of the split signal d [R][2 Cc] (hi + lo), FP32.
+// db[c] = sum over the R rows of the split signal d [R][2 Cc] (hi + lo), FP32
+// (the logits' few rows and columns).
 __global__ void k_colsum(const __nv_bfloat16 *__restrict__ d, int R, int Cc, float *__restrict__ db)
 {
     __shared__ float s[256];
@@ -230,10 +264,12 @@ cudaError_t launch_softmax_ce(const float *logits, const int32_t *labels, int B,
 }
 
 // Adam (Kingma and Ba): m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
-// w -= lr * (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps).  Also refreshes
-// the BF16 copy of the weight (w_bf may be null for biases).
+// w -= lr * (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps), over all n
+// parameters in one launch (two per tensor cost more in launches than the
+// update takes).  Also refreshes the weights' BF16 copies: parameter i of
+// [T.begin[k], T.end[k]) is T.bf[k] + i - T.begin[k] there (biases have none).
 __global__ void k_adam(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v, const float *__restrict__ g,
-                       int64_t n, float lr, float b1, float b2, float eps, float c1, float c2,
+                       int64_t n, float lr, float b1, float b2, float eps, float c1, float c2, AdamTensors T,
                        __nv_bfloat16 *__restrict__ w_bf)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -245,13 +281,17 @@ __global__ void k_adam(float *__restrict__ w, float *__restrict__ m, float *__re
     v[i] = vi;
     const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     w[i] = wi;
-    if (w_bf) w_bf[i] = __float2bfloat16_rn(wi);
+    int64_t at = -1;
+#pragma unroll
+    for (int k = 0; k < AdamTensors::N; ++k)
+        if (i >= T.begin[k] && i < T.end[k]) at = T.bf[k] + (i - T.begin[k]);
+    if (at >= 0) w_bf[at] = __float2bfloat16_rn(wi);
 }
 
 cudaError_t launch_adam(float *w, float *m, float *v, const float *g, int64_t n, float lr, float b1, float b2, float eps,
-                        float c1, float c2, __nv_bfloat16 *w_bf, cudaStream_t st)
+                        float c1, float c2, const AdamTensors &T, __nv_bfloat16 *w_bf, cudaStream_t st)
 {
-    k_adam<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(w, m, v, g, n, lr, b1, b2, eps, c1, c2, w_bf);
+    k_adam<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(w, m, v, g, n, lr, b1, b2, eps, c1, c2, T, w_bf);
     return cudaGetLastError();
 }
 

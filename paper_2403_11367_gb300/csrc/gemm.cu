@@ -2,10 +2,12 @@
 //
 //   C[m][n] = sum_k A[m][k] * B[n][k]   (+ bias[n], ReLU, optional)
 //
-// A and B are row-major with K contiguous ("K-major"), BF16; the accumulator
-// is FP32 in tensor memory; C is written as FP32 or BF16.  This is the dense
-// contraction of the learned candidate proposal (convolutions via im2col and
-// the MLP, forward and backward).
+// A and B are BF16; the accumulator is FP32 in tensor memory; C is written as
+// FP32 or BF16.  This is the dense contraction of the learned candidate proposal
+// (convolutions via im2col and the MLP, forward and backward).  An operand is
+// K-major (rows of contiguous K, as above) or MN-major (stored transposed, as
+// the backward pass has it: the rows of a weight gradient's operands are the
+// contracted index), which the tensor cores read as it is.
 //
 // Persistent: as many CTAs as fit take 128 x BN output tiles (BN in {16, 32,
 // ..., 256}) in turn.  A CTA of 192 threads is warp-specialised over a ring of
@@ -30,6 +32,10 @@
 //     store on another line, and the write took several times as long as the
 //     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us).  Bias and
 //     ReLU are applied there.
+// An MN-major operand's tile is loaded as boxes of 64 columns (128 bytes) by the
+// 64 rows of the K step, in the canonical MN-major SWIZZLE_128B layout; its
+// transposed copy (four launches per weight gradient, two per input gradient,
+// 720 us of a training step of batch 256) is never made.
 // With split_k > 1 a tile covers the K range [z*Ks, (z+1)*Ks) and writes FP32
 // partials C[z][M][N], summed later in a fixed order.
 //
@@ -74,22 +80,29 @@ __device__ __forceinline__ unsigned long long global_ns()
 // boundaries), layout type 2 = 128-byte swizzle in 61-63).  A K step of 16
 // BF16 inside the row advances the start by 32 bytes; the swizzle is applied
 // to the resulting addresses.
+//
+// MN-major SWIZZLE_128B: 64 columns (128 bytes) of one k to a row, 8 rows to a
+// 1024-byte group; the stride byte offset leads to the next 8 rows (1024), the
+// leading byte offset to the next 64 columns (a box of 64 rows: 8192).  A K step
+// of 16 is two groups of rows: 2048 bytes.
+constexpr uint32_t MN_BOX = 64 * 64 * 2;
+template <bool MN>
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
 {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)(16 >> 4) << 16;
+    d |= (uint64_t)((MN ? MN_BOX : 16u) >> 4) << 16;
     d |= (uint64_t)(1024 >> 4) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
     return d;
 }
 
-// Instruction descriptor, kind::f16: FP32 accumulate, BF16 A and B, both
-// K-major, N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N)
+// Instruction descriptor, kind::f16: FP32 accumulate, BF16 A and B, bits 15 and
+// 16 set for an MN-major A and B, N >> 3 in bits 17-22, M >> 4 in bits 24-28.
+__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N, bool a_mn, bool b_mn)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // Wait until the phase of the given parity has completed, or GEMM_WAIT_NS.
@@ -163,6 +176,9 @@ struct GemmArgs {
     int split_k;                // >= 1; > 1 writes partials Cf[z][M][ldc]
     int n_tn, n_tiles;          // column tiles, all tiles (row tiles x column tiles x split_k)
     int vec;                    // 16-byte (BF16: 8-byte) stores allowed: ldc, N and the bases
+    // MN-major operands hold half the contracted rows: K index k >= half reads
+    // row k - half, of A's columns + a_xoff (the low terms of a split signal)
+    int half, a_xoff;
     int inject;                 // test only: the MMA lane waits on a barrier nothing arrives at
     int *status;                // error flag (1: an mbarrier wait gave up), device or pinned host memory
 };
@@ -180,7 +196,7 @@ struct GemmSmem {
     static constexpr uint32_t TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;       // two accumulators, power of two >= 32
 };
 
-template <int BN>
+template <int BN, bool AMN, bool BMN>
 __global__ void __launch_bounds__(GEMM_THREADS)
 k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs g)
 {
@@ -197,7 +213,8 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const int k_per = g.K / g.split_k;                  // multiple of 64 by construction
     const int n_k = k_per / GEMM_BK;
     const int n_mn = g.n_tiles / g.split_k;
-    constexpr uint32_t IDESC = instr_desc_bf16(GEMM_BM, BN);
+    constexpr uint32_t IDESC = instr_desc_bf16(GEMM_BM, BN, AMN, BMN);
+    static_assert(!BMN || BN % 64 == 0, "whole boxes");
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
@@ -249,8 +266,20 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
                 const uint32_t fb = smem_u32(&bar_full[s]);
                 mbar_expect_tx(fb, SM::STAGE);
-                tma_load_2d(sa, &tmA, kbeg + k * GEMM_BK, m0, fb);
-                tma_load_2d(sb, &tmB, kbeg + k * GEMM_BK, n0, fb);
+                const int k0 = kbeg + k * GEMM_BK, r = k0 >= g.half ? k0 - g.half : k0;
+                if (AMN) {
+                    const int x = m0 + (k0 >= g.half ? g.a_xoff : 0);
+                    tma_load_2d(sa, &tmA, x, r, fb);
+                    tma_load_2d(sa + MN_BOX, &tmA, x + 64, r, fb);
+                } else {
+                    tma_load_2d(sa, &tmA, k0, m0, fb);
+                }
+                if (BMN) {
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * MN_BOX, &tmB, n0 + 64 * j, r, fb);
+                } else {
+                    tma_load_2d(sb, &tmB, k0, n0, fb);
+                }
             }
         }
         // copies still in flight land before the CTA may exit: the last one
@@ -275,9 +304,9 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
 #pragma unroll
                 for (int j = 0; j < GEMM_BK / 16; ++j) {
-                    // K step j: 16 BF16 = 32 bytes further along the 128-byte rows
-                    const uint64_t da = smem_desc_sw128(sa + 32 * j);
-                    const uint64_t db = smem_desc_sw128(sb + 32 * j);
+                    // K step j: 16 BF16 = 32 bytes further along the 128-byte rows, or 16 rows on
+                    const uint64_t da = smem_desc_sw128<AMN>(sa + (AMN ? 2048 : 32) * j);
+                    const uint64_t db = smem_desc_sw128<BMN>(sb + (BMN ? 2048 : 32) * j);
                     const uint32_t acc = (k > 0 || j > 0) ? 1u : 0u;
                     asm volatile("{\n\t.reg .pred p;\n\t"
                                  "setp.ne.u32 p, %4, 0;\n\t"
@@ -433,8 +462,8 @@ static EncodeTiledFn encode_tiled()
     return fn;
 }
 
-// Row-major BF16 matrix [rows][ld] (K = cols used), boxes of 64 K-elements
-// (128 bytes) by box_rows rows, 128-byte swizzle; rows beyond `rows` read 0.
+// Row-major BF16 matrix [rows][ld], cols used, in boxes of 64 columns (128 bytes)
+// by box_rows rows, 128-byte swizzle; what lies beyond rows or cols reads 0.
 static cudaError_t make_map(CUtensorMap *map, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows)
 {
     EncodeTiledFn fn = encode_tiled();
@@ -449,9 +478,15 @@ static cudaError_t make_map(CUtensorMap *map, const __nv_bfloat16 *base, int row
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// CTAs of k_gemm_bf16<BN> that fit on the current device at once: by shared
+// An operand as it lies in memory: rows x cols used of row stride ld.
+struct GemmOperand {
+    const __nv_bfloat16 *p;
+    int rows, cols, ld;
+};
+
+// CTAs of k_gemm_bf16 that fit on the current device at once: by shared
 // memory and registers, and at most 512 TMEM columns to an SM.  0 on error.
-template <int BN>
+template <int BN, bool AMN, bool BMN>
 static int gemm_resident()
 {
     constexpr int MAX_DEV = 64;
@@ -461,10 +496,10 @@ static int gemm_resident()
     int c = cached[dev].load();
     if (!c) {
         int sms = 0, per_sm = 0;
-        if (cudaFuncSetAttribute(k_gemm_bf16<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_gemm_bf16<BN, AMN, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)GemmSmem<BN>::TOTAL) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemm_bf16<BN>, GEMM_THREADS,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemm_bf16<BN, AMN, BMN>, GEMM_THREADS,
                                                           GemmSmem<BN>::TOTAL) != cudaSuccess)
             return 0;
         const int by_tmem = 512 / (int)GemmSmem<BN>::TMEM_COLS;
@@ -474,14 +509,14 @@ static int gemm_resident()
     return c;
 }
 
-template <int BN>
-static cudaError_t gemm_t(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int lda, int ldb, GemmArgs g, cudaStream_t st)
+template <int BN, bool AMN, bool BMN>
+static cudaError_t gemm_t(const GemmOperand &A, const GemmOperand &B, GemmArgs g, cudaStream_t st)
 {
     CUtensorMap ma, mb;
-    cudaError_t e = make_map(&ma, A, g.M, g.K, lda, GEMM_BM);
-    if (e == cudaSuccess) e = make_map(&mb, B, g.N, g.K, ldb, BN);
+    cudaError_t e = make_map(&ma, A.p, A.rows, A.cols, A.ld, AMN ? GEMM_BK : GEMM_BM);
+    if (e == cudaSuccess) e = make_map(&mb, B.p, B.rows, B.cols, B.ld, BMN ? GEMM_BK : BN);
     if (e != cudaSuccess) return e;
-    const int resident = gemm_resident<BN>();
+    const int resident = gemm_resident<BN, AMN, BMN>();
     if (resident <= 0) {
         e = cudaGetLastError();
         return e != cudaSuccess ? e : cudaErrorInvalidValue;
@@ -490,7 +525,42 @@ static cudaError_t gemm_t(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int ld
     const int64_t tiles = ceil_div(g.M, GEMM_BM) * g.n_tn * g.split_k;
     if (tiles > (int64_t)1 << 30) return cudaErrorInvalidValue;
     g.n_tiles = (int)tiles;
-    k_gemm_bf16<BN><<<(unsigned)min64(tiles, resident), GEMM_THREADS, GemmSmem<BN>::TOTAL, st>>>(ma, mb, g);
+    k_gemm_bf16<BN, AMN, BMN><<<(unsigned)min64(tiles, resident), GEMM_THREADS, GemmSmem<BN>::TOTAL, st>>>(ma, mb, g);
+    return cudaGetLastError();
+}
+
+// The widest tile that N fills, halved while that leaves fewer columns to the
+// busiest SM: rounds of one tile an SM x BN is the time of the MMAs, and 128
+// rows by 1024 columns would run on 4 SMs at BN = 256.
+static int gemm_bn(int M, int N, int split_k, int least)
+{
+    int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
+    if (BN < least) BN = least;
+    auto columns = [&](int bn) { return ceil_div(ceil_div(M, GEMM_BM) * ceil_div(N, bn) * split_k, 152) * bn; };
+    while (BN / 2 >= (least > 32 ? least : 32) && columns(BN / 2) < columns(BN)) BN /= 2;
+    return BN;
+}
+
+// Fills in the output side of g and runs the epilogue's reduction after `run`.
+template <typename F>
+static cudaError_t gemm_split(GemmArgs &g, const float *bias, float *Cf, __nv_bfloat16 *Cb, int M, int N, int K, int ldc,
+                              int relu, int split_k, float *partials, int *status, cudaStream_t st, int inject, F run)
+{
+    g.bias = bias; g.Cf = Cf; g.Cb = Cb;
+    g.M = M; g.N = N; g.K = K; g.ldc = ldc;
+    g.relu = relu; g.split_k = split_k; g.status = status;
+    g.inject = take_fault(FAULT_GEMM_WAIT) ? 1 : inject;
+    if (split_k > 1) {
+        g.Cf = partials;
+        g.Cb = nullptr;
+        g.bias = nullptr;
+        g.relu = 0;
+    }
+    g.vec = N % 4 == 0 && ldc % 4 == 0 && ((uintptr_t)g.Cf & 15) == 0 && ((uintptr_t)g.Cb & 7) == 0;
+    cudaError_t e = run();
+    if (e != cudaSuccess || split_k == 1) return e;
+    const int64_t n = (int64_t)M * N;
+    k_gemm_reduce<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(partials, split_k, M, N, ldc, bias, relu, Cf, Cb);
     return cudaGetLastError();
 }
 
@@ -508,36 +578,59 @@ cudaError_t launch_gemm_bf16(const __nv_bfloat16 *A, const __nv_bfloat16 *B, con
     if (K % GEMM_BK || split_k < 1 || (K / split_k) % GEMM_BK || (lda % 8) || (ldb % 8) ||
         ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || (split_k > 1 && !partials))
         return cudaErrorInvalidValue;
-    if (take_fault(FAULT_GEMM_WAIT)) inject = 1;
     GemmArgs g{};
-    g.bias = bias; g.Cf = Cf; g.Cb = Cb;
-    g.M = M; g.N = N; g.K = K; g.ldc = ldc;
-    g.relu = relu; g.split_k = split_k; g.inject = inject; g.status = status;
-    if (split_k > 1) {
-        g.Cf = partials;
-        g.Cb = nullptr;
-        g.bias = nullptr;
-        g.relu = 0;
-    }
-    g.vec = N % 4 == 0 && ldc % 4 == 0 && ((uintptr_t)g.Cf & 15) == 0 && ((uintptr_t)g.Cb & 7) == 0;
-    // The widest tile that N fills, halved while that leaves fewer columns to
-    // the busiest SM: rounds of one tile an SM x BN is the time of the MMAs,
-    // and 16-row outputs of 1024 columns would run on 4 SMs at BN = 256.
-    int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
-    auto columns = [&](int bn) { return ceil_div(ceil_div(M, GEMM_BM) * ceil_div(N, bn) * split_k, 152) * bn; };
-    while (BN > 32 && columns(BN / 2) < columns(BN)) BN /= 2;
-    cudaError_t e;
-    switch (BN) {
-    case 16: e = gemm_t<16>(A, B, lda, ldb, g, st); break;
-    case 32: e = gemm_t<32>(A, B, lda, ldb, g, st); break;
-    case 64: e = gemm_t<64>(A, B, lda, ldb, g, st); break;
-    case 128: e = gemm_t<128>(A, B, lda, ldb, g, st); break;
-    default: e = gemm_t<256>(A, B, lda, ldb, g, st); break;
-    }
-    if (e != cudaSuccess || split_k == 1) return e;
-    const int64_t n = (int64_t)M * N;
-    k_gemm_reduce<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(partials, split_k, M, N, ldc, bias, relu, Cf, Cb);
-    return cudaGetLastError();
+    g.half = K;                                          // no second half
+    const GemmOperand a{A, M, K, lda}, b{B, N, K, ldb};
+    return gemm_split(g, bias, Cf, Cb, M, N, K, ldc, relu, split_k, partials, status, st, inject, [&]() {
+        switch (gemm_bn(M, N, split_k, 16)) {
+        case 16: return gemm_t<16, false, false>(a, b, g, st);
+        case 32: return gemm_t<32, false, false>(a, b, g, st);
+        case 64: return gemm_t<64, false, false>(a, b, g, st);
+        case 128: return gemm_t<128, false, false>(a, b, g, st);
+        default: return gemm_t<256, false, false>(a, b, g, st);
+        }
+    });
+}
+
+// Weight gradient gW [N][Kc] = (hi + lo)^T X for a split signal dY [R][2 N] (hi |
+// lo) and X [R][Kc]: the contraction runs over the 2 R rows hi then lo, X read
+// twice, both operands as they lie.  R a multiple of 64, N and Kc of 8.
+cudaError_t launch_gemm_weight_grad(const __nv_bfloat16 *dY, const __nv_bfloat16 *X, float *gW, int R, int N, int Kc,
+                                    int split_k, float *partials, int *status, cudaStream_t st)
+{
+    const int K = 2 * R;
+    if (R <= 0 || R % GEMM_BK || N % 8 || Kc % 8 || split_k < 1 || (K / GEMM_BK) % split_k ||
+        ((uintptr_t)dY & 15) || ((uintptr_t)X & 15) || (split_k > 1 && !partials))
+        return cudaErrorInvalidValue;
+    GemmArgs g{};
+    g.half = R;
+    g.a_xoff = N;
+    const GemmOperand a{dY, R, 2 * N, 2 * N}, b{X, R, Kc, Kc};
+    return gemm_split(g, nullptr, gW, nullptr, N, Kc, K, Kc, 0, split_k, partials, status, st, 0, [&]() {
+        switch (gemm_bn(N, Kc, split_k, 64)) {
+        case 64: return gemm_t<64, true, true>(a, b, g, st);
+        case 128: return gemm_t<128, true, true>(a, b, g, st);
+        default: return gemm_t<256, true, true>(a, b, g, st);
+        }
+    });
+}
+
+// Input gradient dX [R][Kc] = (hi + lo) W for a split signal dY [R][2 N] and the
+// weights W [N][Kc] as they lie (read twice).  N a multiple of 64, Kc of 8.
+cudaError_t launch_gemm_input_grad(const __nv_bfloat16 *dY, const __nv_bfloat16 *W, float *dX, int R, int N, int Kc,
+                                   int *status, cudaStream_t st)
+{
+    if (R <= 0 || N % GEMM_BK || Kc % 8 || ((uintptr_t)dY & 15) || ((uintptr_t)W & 15)) return cudaErrorInvalidValue;
+    GemmArgs g{};
+    g.half = N;
+    const GemmOperand a{dY, R, 2 * N, 2 * N}, b{W, N, Kc, Kc};
+    return gemm_split(g, nullptr, dX, nullptr, R, Kc, 2 * N, Kc, 0, 1, nullptr, status, st, 0, [&]() {
+        switch (gemm_bn(R, Kc, 1, 64)) {
+        case 64: return gemm_t<64, false, true>(a, b, g, st);
+        case 128: return gemm_t<128, false, true>(a, b, g, st);
+        default: return gemm_t<256, false, true>(a, b, g, st);
+        }
+    });
 }
 
 }  // namespace reloc

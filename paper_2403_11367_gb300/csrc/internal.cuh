@@ -273,18 +273,30 @@ struct ProposalNet;
 int64_t proposal_param_count();
 ProposalNet *proposal_create(uint64_t seed, cudaError_t *err);
 void proposal_destroy(ProposalNet *P);
-cudaError_t proposal_get(const ProposalNet *P, int which, float *flat);   // 0 params, 1 grads
+cudaError_t proposal_get(ProposalNet *P, int which, float *flat);   // 0 params, 1 grads
 cudaError_t proposal_set(ProposalNet *P, const float *flat);
 cudaError_t proposal_forward(ProposalNet *P, const __nv_bfloat16 *in, int B, float *out, cudaStream_t st);
 cudaError_t proposal_train_step(ProposalNet *P, const __nv_bfloat16 *in, const int32_t *labels, int B, float lr,
-                                bool update, float *loss_rows_dev, cudaStream_t st);
+                                bool update, float *loss_rows, cudaStream_t st);
 const float *proposal_logits(const ProposalNet *P);
-int *proposal_status(const ProposalNet *P);
+// != 0 once a tensor-core wait of a finished launch gave up
+int proposal_status(const ProposalNet *P);
 cudaError_t proposal_make_input(const float *query, const float *seed_rgb, int H, int W, __nv_bfloat16 *out,
                                 cudaStream_t st);
 cudaError_t launch_gemm_bf16(const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *bias, float *Cf,
                              __nv_bfloat16 *Cb, int M, int N, int K, int lda, int ldb, int ldc, int relu, int split_k,
                              float *partials, int *status, cudaStream_t st, int inject = 0);
+
+cudaError_t launch_gemm_weight_grad(const __nv_bfloat16 *dY, const __nv_bfloat16 *X, float *gW, int R, int N, int Kc,
+                                    int split_k, float *partials, int *status, cudaStream_t st);
+cudaError_t launch_gemm_input_grad(const __nv_bfloat16 *dY, const __nv_bfloat16 *W, float *dX, int R, int N, int Kc,
+                                   int *status, cudaStream_t st);
+constexpr int RELU_BACK_BLOCKS = 608;                 // four 256-thread blocks to an SM
+// Weight tensors inside the flat parameters and their places in the BF16 copies.
+struct AdamTensors {
+    static constexpr int N = 7;
+    int64_t begin[N], end[N], bf[N];
+};
 
 // Fault injection for tests (reloc_inject_faults): the number of upcoming
 // GEMM launches whose tensor-core waits are made to run out, and of upcoming

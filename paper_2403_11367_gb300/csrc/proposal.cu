@@ -23,17 +23,13 @@ namespace reloc {
 cudaError_t launch_downsample_gray(const float *img, int H, int W, int f, int ch, __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t launch_im2col(const __nv_bfloat16 *x, int B, int H, int W, int C, int Ho, int Wo, int Kp,
                           __nv_bfloat16 *col, cudaStream_t st);
-cudaError_t launch_col2im(const float *dcol, int B, int H, int W, int C, int Ho, int Wo, int Kp, __nv_bfloat16 *dx_bf,
-                          float *dx_f, cudaStream_t st);
-cudaError_t launch_transpose_bf16(const __nv_bfloat16 *in, int R, int Cc, int ld_in, __nv_bfloat16 *out, int Rp, int Cp,
-                                  cudaStream_t st, int ldo = 0);
-cudaError_t launch_relu_back(const float *d, const __nv_bfloat16 *y, int64_t M, int N, __nv_bfloat16 *out,
-                             cudaStream_t st);
+cudaError_t launch_relu_back(const float *d, int H, int W, int Ho, int Wo, int Kp, const __nv_bfloat16 *y, int M, int N,
+                             __nv_bfloat16 *out, float *part, float *db, cudaStream_t st);
 cudaError_t launch_colsum(const __nv_bfloat16 *d, int R, int Cc, float *db, cudaStream_t st);
 cudaError_t launch_softmax_ce(const float *logits, const int32_t *labels, int B, int C, float *loss_rows, float *dl,
                               __nv_bfloat16 *dlb, cudaStream_t st);
 cudaError_t launch_adam(float *w, float *m, float *v, const float *g, int64_t n, float lr, float b1, float b2, float eps,
-                        float c1, float c2, __nv_bfloat16 *w_bf, cudaStream_t st);
+                        float c1, float c2, const AdamTensors &T, __nv_bfloat16 *w_bf, cudaStream_t st);
 cudaError_t launch_to_bf16(const float *a, int64_t n, __nv_bfloat16 *b, cudaStream_t st);
 
 namespace {
@@ -65,6 +61,27 @@ struct Buf {
     template <typename T> T *as() const { return (T *)p; }
 };
 
+// Pinned host memory, which kernels can write to as well.
+struct HostBuf {
+    void *p = nullptr;
+    size_t bytes = 0;
+    cudaError_t ensure(size_t n)
+    {
+        if (n <= bytes && p) return cudaSuccess;
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        bytes = 0;
+        cudaError_t e = cudaMallocHost(&p, n);
+        if (e == cudaSuccess) bytes = n;
+        return e;
+    }
+    ~HostBuf()
+    {
+        if (p) cudaFreeHost(p);
+    }
+    template <typename T> T *as() const { return (T *)p; }
+};
+
 }  // namespace
 
 struct ProposalNet {
@@ -78,7 +95,9 @@ struct ProposalNet {
     int64_t steps = 0;
     // activations (sized for the largest batch seen)
     int cap_b = 0;
-    Buf col[5], y[5], h1, logits, dl, dlb, loss_rows, tA, tB, dmid, dmid_bf, dcol, part, status;
+    Buf col[5], y[5], h1, logits, dl, dlb, dmid, dmid_bf, dcol, part, csum;
+    HostBuf status;              // written by the GEMMs only when a wait gives up
+    HostBuf xfer;                // parameters or gradients on their way out
 };
 
 int64_t proposal_param_count()
@@ -159,7 +178,7 @@ ProposalNet *proposal_create(uint64_t seed, cudaError_t *err)
     cudaMemset(P->grad.p, 0, 4 * o);
     cudaMemset(P->m.p, 0, 4 * o);
     cudaMemset(P->v.p, 0, 4 * o);
-    cudaMemset(P->status.p, 0, 64);
+    memset(P->status.p, 0, 64);
     for (int t = 0; t < 7; ++t)
         launch_to_bf16(P->master.as<float>() + P->w_off[t], (int64_t)P->wn[t] * P->wk[t],
                        P->wbf.as<__nv_bfloat16>() + P->wbf_off[t], 0);
@@ -186,24 +205,26 @@ static void flat_to_master(const ProposalNet *P, const float *flat, std::vector<
     }
 }
 
-static void master_to_flat(const ProposalNet *P, const std::vector<float> &master, float *flat)
+static void master_to_flat(const ProposalNet *P, const float *master, float *flat)
 {
     int64_t f = 0;
     for (int t = 0; t < 7; ++t) {
         const int kreal = t < 5 ? P->conv[t].K : P->wk[t];
-        for (int r = 0; r < P->wn[t]; ++r)
-            for (int k = 0; k < kreal; ++k) flat[f++] = master[P->w_off[t] + (int64_t)r * P->wk[t] + k];
-        for (int r = 0; r < P->wn[t]; ++r) flat[f++] = master[P->b_off[t] + r];
+        for (int r = 0; r < P->wn[t]; ++r, f += kreal)
+            memcpy(flat + f, master + P->w_off[t] + (int64_t)r * P->wk[t], sizeof(float) * kreal);
+        memcpy(flat + f, master + P->b_off[t], sizeof(float) * P->wn[t]);
+        f += P->wn[t];
     }
 }
 
-cudaError_t proposal_get(const ProposalNet *P, int which, float *flat)
+cudaError_t proposal_get(ProposalNet *P, int which, float *flat)
 {
-    std::vector<float> h(P->n_master);
-    const Buf &b = which == 0 ? P->master : P->grad;
-    cudaError_t e = cudaMemcpy(h.data(), b.p, 4 * P->n_master, cudaMemcpyDeviceToHost);
+    cudaError_t e = P->xfer.ensure(4 * P->n_master);
     if (e != cudaSuccess) return e;
-    master_to_flat(P, h, flat);
+    const Buf &b = which == 0 ? P->master : P->grad;
+    e = cudaMemcpy(P->xfer.p, b.p, 4 * P->n_master, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return e;
+    master_to_flat(P, P->xfer.as<float>(), flat);
     return cudaSuccess;
 }
 
@@ -226,29 +247,24 @@ static cudaError_t ensure_batch(ProposalNet *P, int B)
 {
     if (B <= P->cap_b) return cudaSuccess;
     cudaError_t e;
-    size_t max_col = 0, max_mid = 0, max_tr = 0;
+    size_t max_col = 0, max_mid = 0;
     for (int l = 0; l < 5; ++l) {
         const Conv &c = P->conv[l];
         const size_t M = (size_t)B * c.Ho * c.Wo;
         if ((e = P->col[l].ensure(2 * M * c.Kp)) != cudaSuccess) return e;
         if ((e = P->y[l].ensure(2 * M * c.Cout)) != cudaSuccess) return e;
-        max_col = std::max(max_col, M * c.Kp);
+        if (l > 0) max_col = std::max(max_col, M * c.Kp);
         max_mid = std::max(max_mid, M * c.Cout);
-        max_tr = std::max(max_tr, M * (size_t)std::max(c.Kp, c.Cout));
     }
-    max_mid = std::max(max_mid, (size_t)B * FC1_IN);
-    max_tr = std::max(max_tr, (size_t)FC1_IN * FC1_OUT);
-    max_tr = std::max(max_tr, (size_t)B * FC1_IN);
+    max_mid = std::max(max_mid, (size_t)B * FC1_OUT);
     if ((e = P->h1.ensure(2 * (size_t)B * FC1_OUT)) != cudaSuccess) return e;
     if ((e = P->logits.ensure(4 * (size_t)B * FC2_OUT)) != cudaSuccess) return e;
     if ((e = P->dl.ensure(4 * (size_t)B * FC2_OUT)) != cudaSuccess) return e;
     // backward signals are carried as hi | lo BF16 pairs: twice the columns
     if ((e = P->dlb.ensure(2 * 2 * (size_t)B * FC2_OUT)) != cudaSuccess) return e;
-    if ((e = P->loss_rows.ensure(4 * (size_t)B)) != cudaSuccess) return e;
-    if ((e = P->tA.ensure(2 * 2 * max_tr)) != cudaSuccess) return e;
-    if ((e = P->tB.ensure(2 * 2 * max_tr)) != cudaSuccess) return e;
-    if ((e = P->dmid.ensure(4 * std::max(max_mid, (size_t)B * FC1_OUT))) != cudaSuccess) return e;
-    if ((e = P->dmid_bf.ensure(2 * 2 * std::max(max_mid, (size_t)B * FC1_OUT))) != cudaSuccess) return e;
+    if ((e = P->dmid.ensure(4 * (size_t)B * FC1_IN)) != cudaSuccess) return e;      // the FC layers' input gradients
+    if ((e = P->dmid_bf.ensure(2 * 2 * max_mid)) != cudaSuccess) return e;
+    if ((e = P->csum.ensure(4 * (size_t)RELU_BACK_BLOCKS * FC1_IN)) != cudaSuccess) return e;
     if ((e = P->dcol.ensure(4 * max_col)) != cudaSuccess) return e;
     if ((e = P->part.ensure(4 * (size_t)32 * 1024 * 1024)) != cudaSuccess) return e;   // split-K partials
     P->cap_b = B;
@@ -299,86 +315,74 @@ static int split_for(int K, int cap)
 // pass is that of the stored forward activations and weights.
 
 // weight gradient gW[N][Kc] = dY^T X for the split dY [M][2N] and X [M][Kc]
-// (BF16), M % 32 == 0: one GEMM over the 2M stacked rows, hi^T X + lo^T X
+// (BF16), M % 64 == 0
 static cudaError_t weight_grad(ProposalNet *P, const __nv_bfloat16 *dY, int M, int N, const __nv_bfloat16 *X, int Kc,
                                float *gW, cudaStream_t st)
 {
-    __nv_bfloat16 *tA = P->tA.as<__nv_bfloat16>(), *tB = P->tB.as<__nv_bfloat16>();
-    const int M2 = 2 * M;
-    PK(launch_transpose_bf16(dY, M, N, 2 * N, tA, M, N, st, M2));          // [N][0, M): hi^T
-    PK(launch_transpose_bf16(dY + N, M, N, 2 * N, tA + M, M, N, st, M2));  // [N][M, 2M): lo^T
-    PK(launch_transpose_bf16(X, M, Kc, Kc, tB, M, Kc, st, M2));             // [Kc][2M]: X^T twice
-    PK(launch_transpose_bf16(X, M, Kc, Kc, tB + M, M, Kc, st, M2));
-    const int split = split_for(M2, std::max(1, (int)std::min<int64_t>(128, (int64_t)32 * 1024 * 1024 / ((int64_t)N * Kc))));
-    return launch_gemm_bf16(tA, tB, nullptr, gW, nullptr, N, Kc, M2, M2, M2, Kc, 0, split, P->part.as<float>(),
-                            P->status.as<int>(), st);
-}
-
-// input gradient dX[M][Kc] (FP32) = dY W for the split dY [M][2N] and the BF16
-// weights W [N][Kc]: one GEMM over 2N, B = [W^T | W^T] ([Kc][2N])
-static cudaError_t input_grad(ProposalNet *P, const __nv_bfloat16 *dY, int M, int N, const __nv_bfloat16 *W, int Kc,
-                              float *dX, cudaStream_t st)
-{
-    __nv_bfloat16 *tB = P->tB.as<__nv_bfloat16>();
-    PK(launch_transpose_bf16(W, N, Kc, Kc, tB, N, Kc, st, 2 * N));
-    PK(launch_transpose_bf16(W, N, Kc, Kc, tB + N, N, Kc, st, 2 * N));
-    return launch_gemm_bf16(dY, tB, nullptr, dX, nullptr, M, Kc, 2 * N, 2 * N, 2 * N, Kc, 0, 1, nullptr,
-                            P->status.as<int>(), st);
+    const int split = split_for(2 * M, std::max(1, (int)std::min<int64_t>(128, (int64_t)32 * 1024 * 1024 / ((int64_t)N * Kc))));
+    return launch_gemm_weight_grad(dY, X, gW, M, N, Kc, split, P->part.as<float>(), P->status.as<int>(), st);
 }
 
 // One training step on a batch (B % 64 == 0): forward, loss, backward; Adam
-// update if `update`.  loss_dev: mean loss written as float.
+// update if `update`.  loss_rows [B] (device or pinned host memory): the rows'
+// losses.
 cudaError_t proposal_train_step(ProposalNet *P, const __nv_bfloat16 *in, const int32_t *labels, int B, float lr,
-                                bool update, float *loss_sum_dev, cudaStream_t st)
+                                bool update, float *loss_rows, cudaStream_t st)
 {
     PK(proposal_forward(P, in, B, nullptr, st));
     float *g = P->grad.as<float>();
     __nv_bfloat16 *wbf = P->wbf.as<__nv_bfloat16>();
-    PK(launch_softmax_ce(P->logits.as<float>(), labels, B, FC2_OUT, P->loss_rows.as<float>(), P->dl.as<float>(),
+    PK(launch_softmax_ce(P->logits.as<float>(), labels, B, FC2_OUT, loss_rows, P->dl.as<float>(),
                          P->dlb.as<__nv_bfloat16>(), st));
-    if (loss_sum_dev) PK(cudaMemcpyAsync(loss_sum_dev, P->loss_rows.p, 4 * (size_t)B, cudaMemcpyDeviceToDevice, st));
+    int *status = P->status.as<int>();
+    float *csum = P->csum.as<float>();
+    __nv_bfloat16 *dy = P->dmid_bf.as<__nv_bfloat16>();
     // FC2
     PK(weight_grad(P, P->dlb.as<__nv_bfloat16>(), B, FC2_OUT, P->h1.as<__nv_bfloat16>(), FC1_OUT, g + P->w_off[6], st));
     PK(launch_colsum(P->dlb.as<__nv_bfloat16>(), B, FC2_OUT, g + P->b_off[6], st));
-    PK(input_grad(P, P->dlb.as<__nv_bfloat16>(), B, FC2_OUT, wbf + P->wbf_off[6], FC1_OUT, P->dmid.as<float>(), st));
-    PK(launch_relu_back(P->dmid.as<float>(), P->h1.as<__nv_bfloat16>(), B, FC1_OUT, P->dmid_bf.as<__nv_bfloat16>(), st));
+    PK(launch_gemm_input_grad(P->dlb.as<__nv_bfloat16>(), wbf + P->wbf_off[6], P->dmid.as<float>(), B, FC2_OUT, FC1_OUT,
+                              status, st));
     // FC1
+    PK(launch_relu_back(P->dmid.as<float>(), 0, 0, 0, 0, 0, P->h1.as<__nv_bfloat16>(), B, FC1_OUT, dy, csum,
+                        g + P->b_off[5], st));
     const __nv_bfloat16 *x5 = P->y[4].as<__nv_bfloat16>();
-    PK(weight_grad(P, P->dmid_bf.as<__nv_bfloat16>(), B, FC1_OUT, x5, FC1_IN, g + P->w_off[5], st));
-    PK(launch_colsum(P->dmid_bf.as<__nv_bfloat16>(), B, FC1_OUT, g + P->b_off[5], st));
-    PK(input_grad(P, P->dmid_bf.as<__nv_bfloat16>(), B, FC1_OUT, wbf + P->wbf_off[5], FC1_IN, P->dmid.as<float>(), st));
-    // conv layers, last to first; dmid holds dL/dY_l (FP32, NHWC)
+    PK(weight_grad(P, dy, B, FC1_OUT, x5, FC1_IN, g + P->w_off[5], st));
+    PK(launch_gemm_input_grad(dy, wbf + P->wbf_off[5], P->dmid.as<float>(), B, FC1_OUT, FC1_IN, status, st));
+    // conv layers, last to first; the gradient of layer l's output comes as dmid (l = 4: FP32, NHWC) or
+    // as the dcol of layer l + 1
     for (int l = 4; l >= 0; --l) {
         const Conv &c = P->conv[l];
         const int M = B * c.Ho * c.Wo;
-        PK(launch_relu_back(P->dmid.as<float>(), P->y[l].as<__nv_bfloat16>(), M, c.Cout,
-                            P->dmid_bf.as<__nv_bfloat16>(), st));
-        PK(weight_grad(P, P->dmid_bf.as<__nv_bfloat16>(), M, c.Cout, P->col[l].as<__nv_bfloat16>(), c.Kp,
-                       g + P->w_off[l], st));
-        PK(launch_colsum(P->dmid_bf.as<__nv_bfloat16>(), M, c.Cout, g + P->b_off[l], st));
+        if (l == 4) {
+            PK(launch_relu_back(P->dmid.as<float>(), 0, 0, 0, 0, 0, P->y[l].as<__nv_bfloat16>(), M, c.Cout, dy, csum,
+                                g + P->b_off[l], st));
+        } else {
+            const Conv &n = P->conv[l + 1];
+            PK(launch_relu_back(P->dcol.as<float>(), n.H, n.W, n.Ho, n.Wo, n.Kp, P->y[l].as<__nv_bfloat16>(), M, c.Cout, dy,
+                                csum, g + P->b_off[l], st));
+        }
+        PK(weight_grad(P, dy, M, c.Cout, P->col[l].as<__nv_bfloat16>(), c.Kp, g + P->w_off[l], st));
         if (l == 0) break;
-        PK(input_grad(P, P->dmid_bf.as<__nv_bfloat16>(), M, c.Cout, wbf + P->wbf_off[l], c.Kp, P->dcol.as<float>(), st));
-        PK(launch_col2im(P->dcol.as<float>(), B, c.H, c.W, c.Cin, c.Ho, c.Wo, c.Kp, nullptr, P->dmid.as<float>(), st));
+        PK(launch_gemm_input_grad(dy, wbf + P->wbf_off[l], P->dcol.as<float>(), M, c.Cout, c.Kp, status, st));
     }
     if (update) {
         P->steps++;
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
         const float c1 = 1.f - std::pow(b1, (float)P->steps), c2 = 1.f - std::pow(b2, (float)P->steps);
+        AdamTensors T;
         for (int t = 0; t < 7; ++t) {
-            const int64_t nw = (int64_t)P->wn[t] * P->wk[t];
-            PK(launch_adam(P->master.as<float>() + P->w_off[t], P->m.as<float>() + P->w_off[t],
-                           P->v.as<float>() + P->w_off[t], g + P->w_off[t], nw, lr, b1, b2, eps, c1, c2,
-                           wbf + P->wbf_off[t], st));
-            PK(launch_adam(P->master.as<float>() + P->b_off[t], P->m.as<float>() + P->b_off[t],
-                           P->v.as<float>() + P->b_off[t], g + P->b_off[t], P->wn[t], lr, b1, b2, eps, c1, c2, nullptr,
-                           st));
+            T.begin[t] = P->w_off[t];
+            T.end[t] = P->b_off[t];
+            T.bf[t] = P->wbf_off[t];
         }
+        PK(launch_adam(P->master.as<float>(), P->m.as<float>(), P->v.as<float>(), g, P->n_master, lr, b1, b2, eps, c1, c2, T,
+                       wbf, st));
     }
     return cudaSuccess;
 }
 
 const float *proposal_logits(const ProposalNet *P) { return P->logits.as<float>(); }
-int *proposal_status(const ProposalNet *P) { return P->status.as<int>(); }
+int proposal_status(const ProposalNet *P) { return *(volatile int *)P->status.p; }
 
 cudaError_t proposal_make_input(const float *query, const float *seed_rgb, int H, int W, __nv_bfloat16 *out,
                                 cudaStream_t st)
