@@ -116,6 +116,40 @@ struct PinBuf {
     }
 };
 
+// A call's results and counters, one block (the same layout on the device and
+// in the pinned read-back): doubles first, then 32-bit words, the counters that
+// the host does not read last.
+struct ResultBlock {
+    int *overflow = nullptr;            // any view over its instance capacity
+    double *scores = nullptr;           // [V]
+    double *best_score = nullptr;       // [Q]
+    uint32_t *nvis = nullptr, *ninst = nullptr;      // [V]
+    int *degen = nullptr;               // [V]
+    int *best = nullptr;                // [Q]
+    int *done = nullptr;                // [V] tile scan: finished blocks
+    int *queues = nullptr;              // [sub-batches][4] blend queue counters
+};
+
+size_t result_scratch_bytes(int64_t V, int64_t n_sb) { return 4 * (size_t)(V + 4 * n_sb); }
+
+// Places a block at base (null: only its size).  Returns its bytes.
+size_t result_block(char *base, int64_t V, int64_t Q, int64_t n_sb, ResultBlock *out)
+{
+    const size_t bytes = 64 + 8 * (size_t)(V + Q) + 4 * (size_t)(3 * V + Q) + result_scratch_bytes(V, n_sb);
+    if (out) {
+        out->overflow = (int *)base;
+        out->scores = (double *)(base + 64);
+        out->best_score = out->scores + V;
+        out->nvis = (uint32_t *)(out->best_score + Q);
+        out->ninst = out->nvis + V;
+        out->degen = (int *)(out->ninst + V);
+        out->best = out->degen + V;
+        out->done = out->best + Q;
+        out->queues = out->done + V;
+    }
+    return bytes;
+}
+
 }  // namespace
 
 struct reloc_ctx {
@@ -130,10 +164,11 @@ struct reloc_ctx {
     BlockIndex blocks;
     // workspace (sized for the largest sub-batch of a call)
     DevBuf gidx, tables, rec, rect, dkey, kva, v1b, hist1, chunk_sums, dtot;
-    DevBuf srect, bhist, inst, ranges, partials, qpart, qstats;
-    // per-call results (all views / queries of the call)
-    DevBuf nvis, ninst, scores, degen, best, best_score, view_sel, flags;
-    DevBuf bqueue;                       // the blend's work counter and heavy-tile list
+    DevBuf srect, bhist, inst, ranges, partials, qpart;
+    // per-call results (all views / queries of the call) and counters, zeroed and read back as one
+    DevBuf res, view_sel;
+    ResultBlock res_at;
+    DevBuf bqueue;                       // the blend's heavy-tile list
     DevBuf hq, hrgb, hdepth;
     DevBuf pnp_X;
     DevBuf gbuf, gcoef, gpart, gpose;    // NCC pose gradients
@@ -251,8 +286,7 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
     DevBuf *bufs[] = {&ctx->mean, &ctx->attr, &ctx->gidx, &ctx->tables, &ctx->rec, &ctx->rect,
                       &ctx->dkey, &ctx->kva, &ctx->v1b, &ctx->hist1, &ctx->dtot, &ctx->chunk_sums,
                       &ctx->srect, &ctx->bhist, &ctx->inst, &ctx->ranges, &ctx->partials,
-                      &ctx->qpart, &ctx->qstats, &ctx->nvis, &ctx->ninst, &ctx->scores, &ctx->degen,
-                      &ctx->best, &ctx->best_score, &ctx->view_sel, &ctx->flags, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
+                      &ctx->qpart, &ctx->res, &ctx->view_sel, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
                       &ctx->hdepth, &ctx->prop_in, &ctx->prop_seed, &ctx->prop_logits, &ctx->prop_idx,
                       &ctx->prop_mrg, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
                       &ctx->gpart, &ctx->gpose};
@@ -669,25 +703,21 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
 {
     const int64_t HW = (int64_t)cp.width * cp.height;
     const Layout &L = sb.L;
-    int *d_overflow = ctx->flags.as<int>();
-    uint32_t *nvis = ctx->nvis.as<uint32_t>() + sb.v0;
-    uint32_t *ninst = ctx->ninst.as<uint32_t>() + sb.v0;
+    const ResultBlock &R = ctx->res_at;
+    int *d_overflow = R.overflow;
+    uint32_t *nvis = R.nvis + sb.v0;
+    uint32_t *ninst = R.ninst + sb.v0;
 
-    stage_mark(ctx, sbi, RELOC_STAGE_CULL, st, capturing);
-    if (sb.S_tot > 0) {
-        CK(launch_gather_subset(sb.d_run_begin, sb.d_run_off, sb.n_runs, sb.S_tot, ctx->gidx.as<uint32_t>(), st));
-        launches += 1;
-    }
+    stage_mark(ctx, sbi, RELOC_STAGE_CULL, st, capturing);       // the gather is part of the projection's launch
     stage_mark(ctx, sbi, RELOC_STAGE_PROJECT, st, capturing);
-    if (sb.pblk > 0) {
+    if (sb.pblk > 0 || o.score) {
         CK(launch_project(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n, ctx->mean.as<float>() + 2 * ctx->n,
-                          ctx->attr.p, ctx->precision, ctx->sh_degree, ctx->n, ctx->gidx.as<uint32_t>(), L, sb.pblk,
-                          sb.d_views, cp, ctx->rec.as<float4>(), ctx->rect.as<uint2>(), ctx->dkey.as<uint32_t>(), st));
+                          ctx->attr.p, ctx->precision, ctx->sh_degree, ctx->n, sb.d_run_begin, sb.d_run_off, sb.n_runs,
+                          ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->rec.as<float4>(),
+                          ctx->rect.as<uint2>(), ctx->dkey.as<uint32_t>(), o.score ? ctx->qpart.as<double>() : nullptr, st));
         launches += 1;
     }
     stage_mark(ctx, sbi, RELOC_STAGE_DEPTH_SORT, st, capturing);
-    CK(cudaMemsetAsync(nvis, 0, 4 * (size_t)L.V, st));
-    CK(cudaMemsetAsync(ninst, 0, 4 * (size_t)L.V, st));
     if (sb.c1 > 0 && sb.S_max <= DEPTH_SORT_CLUSTER_MAX) {
         // the rectangles in depth order are written after the sort: their buffer serves as scratch
         CK(launch_depth_sort(ctx->dkey.as<uint32_t>(), ctx->kva.as<uint2>(), ctx->srect.as<uint2>(),
@@ -733,9 +763,13 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         }
     }
     stage_mark(ctx, sbi, RELOC_STAGE_TILE_COUNT, st, capturing);
+    // work queues of the sub-batch's blend and of its winners'
+    const BlendQueue queue{R.queues + 4 * sbi, ctx->bqueue.as<int>()};
+    const BlendQueue queue_w{R.queues + 4 * sbi + 2, ctx->bqueue.as<int>()};
     CK(launch_tile_count(ctx->v1b.as<uint32_t>(), nvis, ctx->rect.as<uint2>(), L, cp, sb.cb, sb.cb_view, ctx->srect.as<uint2>(),
-                         ctx->bhist.as<uint32_t>(), ctx->ranges.as<int2>(), ninst, d_overflow, st));
-    launches += sb.cb > 0 ? 3 : 2;
+                         ctx->bhist.as<uint32_t>(), ctx->ranges.as<int2>(), ninst, R.done + sb.v0, d_overflow,
+                         blend_heavy_first(L.V) ? queue : BlendQueue{nullptr, nullptr}, st));
+    launches += sb.cb > 0 ? 2 : 1;
     stage_mark(ctx, sbi, RELOC_STAGE_TILE_EMIT, st, capturing);
     if (sb.cb > 0) {
         CK(launch_tile_emit(ctx->v1b.as<uint32_t>(), ctx->srect.as<uint2>(), nvis, ninst, ctx->bhist.as<uint32_t>(),
@@ -744,18 +778,14 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     }
     const uint32_t *fgauss = ctx->inst.as<uint32_t>();
     stage_mark(ctx, sbi, RELOC_STAGE_BLEND, st, capturing);
-    if (o.score) {
-        CK(launch_query_stats(L, HW, cp.ncc_gray != 0, ctx->qpart.as<double>(), ctx->qstats.as<double>(), st));
-        launches += 2;
-    }
     float *rgb_out = o.target ? ctx->trgb.as<float>() : (o.rgb ? o.rgb + (int64_t)sb.v0 * 3 * HW : nullptr);
     const bool rp = o.target && o.rel;
     float *dep_out = rp ? ctx->tdep.as<float>() : (o.depth ? o.depth + (int64_t)sb.v0 * HW : nullptr);
     float *alp_out = rp ? ctx->talp.as<float>() : (o.alpha ? o.alpha + (int64_t)sb.v0 * HW : nullptr);
     CK(launch_blend(ctx->rec.as<float4>(), L, fgauss, ctx->ranges.as<int2>(), cp,
                     o.score ? ctx->partials.as<double>() : nullptr, rgb_out, dep_out, alp_out,
-                    nullptr, 0, d_overflow, ctx->bqueue.as<int>(), st));
-    launches += blend_launches(L.V);
+                    nullptr, 0, d_overflow, queue, st));
+    launches += blend_launches(L.V, false);
     stage_mark(ctx, sbi, RELOC_STAGE_SCORE, st, capturing);
     if (o.target) {
         // map training: the image loss and dL/dC, then back through the blend and the projection
@@ -799,9 +829,8 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         launches += 3;
     }
     if (o.score) {
-        CK(launch_ncc_finalize(ctx->partials.as<double>(), ctx->qstats.as<double>(), L, blend_units(cp),
-                               cp.ncc_gray ? HW : 3 * HW,
-                               ctx->scores.as<double>() + sb.v0, ctx->degen.as<int>() + sb.v0,
+        CK(launch_ncc_finalize(ctx->partials.as<double>(), ctx->qpart.as<double>(), L, blend_units(cp),
+                               cp.ncc_gray ? HW : 3 * HW, R.scores + sb.v0, R.degen + sb.v0,
                                o.grad ? ctx->gcoef.as<double>() : nullptr, st));
         launches += 1;
         if (o.grad) {
@@ -817,8 +846,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         }
         if (o.argmax) {
             int *vsel = ctx->view_sel.as<int>() + sb.q0;
-            CK(launch_argmax(ctx->scores.as<double>() + sb.v0, L, ctx->best.as<int>() + sb.q0,
-                             ctx->best_score.as<double>() + sb.q0, vsel, st));
+            CK(launch_argmax(R.scores + sb.v0, L, R.best + sb.q0, R.best_score + sb.q0, vsel, st));
             launches += 1;
             if (o.brgb || o.bdepth || o.balpha) {
                 const int nq = sb.q1 - sb.q0;
@@ -826,8 +854,8 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
                                 o.brgb ? o.brgb + (int64_t)sb.q0 * 3 * HW : nullptr,
                                 o.bdepth ? o.bdepth + (int64_t)sb.q0 * HW : nullptr,
                                 o.balpha ? o.balpha + (int64_t)sb.q0 * HW : nullptr, vsel, nq, d_overflow,
-                                ctx->bqueue.as<int>(), st));
-                launches += blend_launches(nq);
+                                queue_w, st));
+                launches += blend_launches(nq, true);
             }
         }
     }
@@ -929,32 +957,24 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             CKS(ctx->gcoef.ensure(32 * (size_t)V));
             CKS(ctx->gpart.ensure(48 * (size_t)pb));
         }
-        CKS(ctx->qpart.ensure(16 * 152 * (size_t)Qm));
-        CKS(ctx->qstats.ensure(16 * (size_t)Qm));
-        CKS(ctx->nvis.ensure(4 * (size_t)Vtot));
-        CKS(ctx->ninst.ensure(4 * (size_t)Vtot));
-        CKS(ctx->scores.ensure(8 * (size_t)Vtot));
-        CKS(ctx->degen.ensure(4 * (size_t)Vtot));
-        CKS(ctx->best.ensure(4 * (size_t)Q));
-        CKS(ctx->best_score.ensure(8 * (size_t)Q));
+        CKS(ctx->qpart.ensure(16 * QS_BLOCKS * (size_t)Qm));
         CKS(ctx->view_sel.ensure(4 * (size_t)Q));
-        CKS(ctx->flags.ensure(64));
-        CKS(ctx->bqueue.ensure(4 * (size_t)blend_queue_ints(cp, std::max<int64_t>(V, Qm))));
+        const size_t res_bytes = result_block(nullptr, Vtot, Q, (int64_t)sbs.size(), nullptr);
+        CKS(ctx->res.ensure(res_bytes));
+        result_block(ctx->res.as<char>(), Vtot, Q, (int64_t)sbs.size(), &ctx->res_at);
+        CKS(ctx->bqueue.ensure(4 * (size_t)blend_list_ints(cp, std::max<int64_t>(V, Qm))));
         CKS(ctx->tables.ensure(tab));
         // pinned staging: tables, then readback
         const size_t rb_off = align256(tab);
-        const size_t rb_bytes = 64 + (4 + 4 + 8 + 4) * (size_t)Vtot + (4 + 8) * (size_t)Q;
-        CKS(ctx->pin.ensure(rb_off + rb_bytes));
+        CKS(ctx->pin.ensure(rb_off + res_bytes));
         char *pin = (char *)ctx->pin.p;
         for (auto &sb : sbs) stage_tables(sb, pin, ctx->tables.as<char>());
-        // readback block: doubles first (8-byte aligned), then 32-bit words
-        int *h_overflow = (int *)(pin + rb_off);
-        double *h_scores = (double *)(pin + rb_off + 64);
-        double *h_bscore = h_scores + Vtot;
-        uint32_t *h_nvis = (uint32_t *)(h_bscore + Q);
-        uint32_t *h_ninst = h_nvis + Vtot;
-        int *h_degen = (int *)(h_ninst + Vtot);
-        int *h_best = h_degen + Vtot;
+        ResultBlock H;                   // the call's results on the host
+        const size_t rb_bytes = result_block(pin + rb_off, Vtot, Q, (int64_t)sbs.size(), &H) -
+                                result_scratch_bytes(Vtot, (int64_t)sbs.size());
+        const int *h_overflow = H.overflow, *h_degen = H.degen, *h_best = H.best;
+        const double *h_scores = H.scores, *h_bscore = H.best_score;
+        const uint32_t *h_nvis = H.nvis, *h_ninst = H.ninst;
         if (ctx->prof) {
             const size_t need = sbs.size() * (RELOC_STAGE_COUNT + 1);
             while (ctx->ev.size() < need) {
@@ -971,7 +991,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             st = ctx->cap_stream;
         }
         CK(cudaMemcpyAsync(ctx->tables.p, pin, tab, cudaMemcpyHostToDevice, st));
-        CK(cudaMemsetAsync(ctx->flags.p, 0, 64, st));
+        CK(cudaMemsetAsync(ctx->res.p, 0, res_bytes, st));       // flags, counts, counters
         if (o.target) {     // every attempt starts from zero (an overflow retry re-runs the call)
             CK(cudaMemsetAsync(ctx->tloss.p, 0, 8, st));
             CK(cudaMemsetAsync(o.tgrad, 0, sizeof(float) * 14 * (size_t)ctx->n, st));
@@ -1000,17 +1020,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             for (size_t k = 0; k < sbs.size(); ++k) CKS(enqueue_subbatch(ctx, sbs[k], (int)k, cp, o, st, false, launches));
         }
         // ---- readback --------------------------------------------------------------
-        CK(cudaMemcpyAsync(h_overflow, ctx->flags.p, 4, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(h_nvis, ctx->nvis.p, 4 * (size_t)Vtot, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(h_ninst, ctx->ninst.p, 4 * (size_t)Vtot, cudaMemcpyDeviceToHost, st));
-        if (o.score) {
-            CK(cudaMemcpyAsync(h_scores, ctx->scores.p, 8 * (size_t)Vtot, cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(h_degen, ctx->degen.p, 4 * (size_t)Vtot, cudaMemcpyDeviceToHost, st));
-            if (o.argmax) {
-                CK(cudaMemcpyAsync(h_best, ctx->best.p, 4 * (size_t)Q, cudaMemcpyDeviceToHost, st));
-                CK(cudaMemcpyAsync(h_bscore, ctx->best_score.p, 8 * (size_t)Q, cudaMemcpyDeviceToHost, st));
-            }
-        }
+        CK(cudaMemcpyAsync(pin + rb_off, ctx->res.p, rb_bytes, cudaMemcpyDeviceToHost, st));
         if (graph) {
             CK(cudaEventRecord(ctx->ev_out, st));
             CK(cudaStreamWaitEvent(ust, ctx->ev_out, 0));

@@ -96,19 +96,52 @@ __device__ __forceinline__ int find_segment(const int32_t *base, int n, int x)
 
 constexpr int PROJ_THREADS = 128;
 
+// ---- launch chaining ----------------------------------------------------------
+// The kernels of a call form one chain on its stream.  A kernel launched by
+// launch_chained is set up while the one before still runs (programmatic
+// dependent launch) and calls chain_wait() before it touches memory, which
+// returns once every earlier kernel of the chain has finished and its writes are
+// visible: some 1 us less between two kernels (a render of the 10k box 129 -> 120
+// us, a driving view 274 -> 263 us).  No kernel lets the next one's blocks be
+// placed before its own end (griddepcontrol.launch_dependents): with that, the
+// resident blocks of waiting kernels took 64 driving candidates from 3.85 to 4.28
+// ms and a batch of queries from 19.3 to 23.7 ms.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster,
+                                  A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- launchers (each returns the launch error) -------------------------------
 
-// K1: subset gather.  run_begin/run_off: n_runs block-ordered runs and their
-// exclusive prefix of lengths (device); writes gidx[total] map positions.
-cudaError_t launch_gather_subset(const int64_t *run_begin, const int64_t *run_off, int n_runs,
-                                 int64_t total, uint32_t *gidx, cudaStream_t st);
-
-// K2: projection of every query's subset into that query's views.
-// n_blocks = q_pblk[Q] (host copy).
+// K1 + K2: projection of every query's subset into that query's views.  n_blocks
+// = q_pblk[Q] (host copy).  run_begin, run_off: n_runs block-ordered runs and the
+// exclusive prefix of their lengths (device); the subset's map positions are
+// written to gidx.  qpart non-null: also the query images' partial sums
+// (QS_BLOCKS pairs of doubles a query: sum, sum of squares over the 3 H W
+// samples, or over the H W gray values (R + G + B) / 3 when cam.ncc_gray).
+constexpr int QS_BLOCKS = 304;
 cudaError_t launch_project(const float *mx, const float *my, const float *mz, const void *attr,
-                           int precision, int sh_degree, int64_t n_map, const uint32_t *gidx,
+                           int precision, int sh_degree, int64_t n_map, const int64_t *run_begin,
+                           const int64_t *run_off, int n_runs, uint32_t *gidx,
                            const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
-                           float4 *rec, uint2 *rect, uint32_t *dkey, cudaStream_t st);
+                           float4 *rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st);
 
 // Depth sort of every view's visible Gaussians in one launch: out[vd_off[v] + k]
 // = index of the k-th nearest (ties by index), n_vis[v] their number.  dkey:
@@ -142,16 +175,26 @@ struct RadixPass {
 };
 cudaError_t launch_radix_pass(const RadixPass &p, cudaStream_t st);
 
+// The blend's work queue: count[0] the ticket, count[1] the heavy tiles listed
+// (both zeroed before the call's first launch), list: view slot * n_tiles + tile
+// of each.  Lists of BLEND_HEAVY records or more are heavy.
+struct BlendQueue {
+    int *count, *list;
+};
+constexpr int BLEND_HEAVY = 1024;
+
 // K3: per chunk of each view's depth-ordered visible Gaussians (sorted_g,
 // n_vis[v] at vd_off[v]) the number covering each tile -> bhist[chunk][tile]
 // (n_chunks = cb_base[V], view_chunks = the most of one view, host copies);
 // rectangles in depth order -> srect;
 // then per view the chunk prefix per tile (in place), ranges[v][tile] =
 // [begin, end) of the tile's list relative to io_off[v] (empty [0, 0)) and
-// n_inst[v].  A view over its capacity sets *overflow.
+// n_inst[v].  A view over its capacity sets *overflow.  done: a zeroed counter
+// per view.  queue non-null: the heavy tiles are listed there for launch_blend.
 cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, const uint2 *rect, const Layout &L,
                               const CamParams &cp, int n_chunks, int view_chunks, uint2 *srect, uint32_t *bhist,
-                              int2 *ranges, uint32_t *n_inst, int *overflow, cudaStream_t st);
+                              int2 *ranges, uint32_t *n_inst, int *done, int *overflow, BlendQueue queue,
+                              cudaStream_t st);
 
 // K4: every (tile, Gaussian) instance into inst_gauss at io_off[v] + its slot,
 // each tile's list in (depth, index) order.  Views over capacity emit nothing.
@@ -177,23 +220,16 @@ cudaError_t measure_peaks(double *fp32_scalar_tflops, double *fp32_packed_tflops
 // Tile id of each instance of one view from its ranges (debug export).
 cudaError_t launch_fill_tiles(const int2 *ranges_view, int n_tiles, uint32_t *tiles_view, cudaStream_t st);
 
-// Query statistics S_q, S_qq over n samples of each of the Q query images
-// -> qstats[Q][2] (double).  block_scratch: Q * 2 * 152 doubles.
-// Query sums (sum q, sum q^2) over its 3 H W samples, or over its H W gray
-// values (R + G + B) / 3 when gray.
-cudaError_t launch_query_stats(const Layout &L, int64_t HW, bool gray, double *block_scratch, double *qstats,
-                               cudaStream_t st);
-
 // K6 (+ K7 partials): blend every (view, tile) of the layout, a warp per
 // 64-pixel block; optional image export (slot = view) and NCC partials
 // [V][blend_units(cam)][3] = {S_r, S_rr, S_rq} per warp block.
 // view_sel != null: blend only the n_sel views view_sel[0..n_sel), image
-// slot k for view_sel[k].  queue: blend_queue_ints(cam, n) device ints for n
-// views, the launch's work counter and list of heavy tiles (zeroed on the
-// stream as needed).  blend_launches(n) launches.
+// slot k for view_sel[k].  queue: a work queue of blend_list_ints(cam, n) entries
+// for n views, with the heavy tiles listed by launch_tile_count or, for selected
+// views, here.  blend_launches(n, selected) launches.
 cudaError_t launch_blend(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                          const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
-                         const int *view_sel, int n_sel, const int *overflow, int *queue, cudaStream_t st);
+                         const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st);
 
 // 64-pixel warp blocks of one view: the blend's unit of work and of NCC partials.
 inline int blend_units(const CamParams &cam) { return cam.n_tiles * (cam.tile_w * cam.tile_h / 64); }
@@ -201,16 +237,17 @@ inline int blend_units(const CamParams &cam) { return cam.n_tiles * (cam.tile_w 
 // work queue's tickets (heavy units counted twice) and its heavy-tile
 // entries stay far inside int32.  Sub-batches are cut to respect it.
 constexpr int64_t BLEND_MAX_UNITS = (int64_t)1 << 29;
-// Work-queue ints of a blend launch over n views.
-inline int64_t blend_queue_ints(const CamParams &cam, int64_t n) { return 4 + n * cam.n_tiles; }
-// Kernel launches of a blend over n views: the heavy-tile listing runs for
-// launches of several views (a one-view launch ends on its longest unit
-// whatever the order).
-__host__ __device__ __forceinline__ int blend_launches(int64_t n) { return n >= 4 ? 2 : 1; }
+inline int64_t blend_list_ints(const CamParams &cam, int64_t n) { return n * cam.n_tiles; }
+// Launches of several views hand out their heavy tiles first (a one-view launch
+// ends on its longest unit whatever the order); a launch of selected views lists
+// them itself.
+__host__ __device__ __forceinline__ bool blend_heavy_first(int64_t n) { return n >= 4; }
+inline int blend_launches(int64_t n, bool selected) { return selected && blend_heavy_first(n) ? 2 : 1; }
 
-// K7: NCC per view from its n_units partials and its query's statistics;
+// K7: NCC per view from its n_units partials and its query's partial sums
+// (launch_project);
 // coef (may be null): [V][4] = 1/sqrt(var_r var_q), NCC/var_r, mean r, mean q.
-cudaError_t launch_ncc_finalize(const double *partials, const double *qstats, const Layout &L, int n_units,
+cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, const Layout &L, int n_units,
                                 int64_t n_samples, double *scores, int *degenerate, double *coef, cudaStream_t st);
 
 // K6 backward: per (view, Gaussian) gradients with respect to the projected

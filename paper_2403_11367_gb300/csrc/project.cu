@@ -1,4 +1,5 @@
-// project.cu -- K1 block-subset gather and K2 EWA projection + SH colour.
+// project.cu -- K1 block-subset gather and K2 EWA projection + SH colour, one
+// launch, with the query images' sums.
 //
 // K2 follows Sec. III-A of 3DGS-ReLoc: t = W mu (world-to-camera), pinhole
 // projection m(mu) (Eq. proj), footprint covariance Sigma' = J W Sigma W^T J^T
@@ -13,25 +14,59 @@ namespace reloc {
 
 // ---------------------------------------------------------------- K1 ------
 
-__global__ void k_gather_subset(const int64_t *__restrict__ run_begin, const int64_t *__restrict__ run_off,
-                                int n_runs, int64_t S, uint32_t *__restrict__ gidx)
+// Map position of the i-th Gaussian of the sub-batch's gathered subsets: the run
+// (of the block-ordered map) that holds i, by bisection.
+__device__ __forceinline__ uint32_t subset_position(const int64_t *__restrict__ run_begin,
+                                                    const int64_t *__restrict__ run_off, int n_runs, int64_t i)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S) return;
     int lo = 0, hi = n_runs - 1;             // last run with run_off[r] <= i
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (run_off[mid] <= i) lo = mid; else hi = mid - 1;
     }
-    gidx[i] = (uint32_t)(run_begin[lo] + (i - run_off[lo]));
+    return (uint32_t)(run_begin[lo] + (i - run_off[lo]));
 }
 
-cudaError_t launch_gather_subset(const int64_t *run_begin, const int64_t *run_off, int n_runs, int64_t total,
-                                 uint32_t *gidx, cudaStream_t st)
+// ------------------------------------------------------ query statistics ---
+// Sum and sum of squares of block b's share of query q's samples, in FP64 (its
+// rate bounds this, so it runs in blocks beside the projection's, which wait on
+// memory); the QS_BLOCKS partials of a query are added by k_ncc_finalize.  Fixed
+// shares and order: the sums are deterministic.
+__device__ __forceinline__ void query_partial(const float *__restrict__ q, int b, int64_t HW, int gray,
+                                              double *__restrict__ out)
 {
-    if (total <= 0 || n_runs <= 0) return cudaSuccess;
-    k_gather_subset<<<(unsigned)ceil_div(total, 256), 256, 0, st>>>(run_begin, run_off, n_runs, total, gidx);
-    return cudaGetLastError();
+    __shared__ double s[2][PROJ_THREADS / 32];
+    const int64_t n = gray ? HW : 3 * HW;
+    double a = 0, c = 0;
+    constexpr int64_t STEP = (int64_t)QS_BLOCKS * PROJ_THREADS;
+    for (int64_t j = (int64_t)b * PROJ_THREADS + threadIdx.x; j < n; j += 4 * STEP) {
+        float v[4][3];                           // the samples of four steps in flight
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t k = j + u * STEP;
+            v[u][0] = k < n ? q[k] : 0.f;
+            v[u][1] = k < n && gray ? q[HW + k] : 0.f;
+            v[u][2] = k < n && gray ? q[2 * HW + k] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const double x = gray ? ((double)v[u][0] + (double)v[u][1] + (double)v[u][2]) / 3.0 : (double)v[u][0];
+            a += x;
+            c += x * x;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        c += __shfl_down_sync(0xffffffffu, c, o);
+    }
+    if ((threadIdx.x & 31) == 0) { s[0][threadIdx.x >> 5] = a; s[1][threadIdx.x >> 5] = c; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < PROJ_THREADS / 32; ++w) { a += s[0][w]; c += s[1][w]; }
+        out[0] = a;
+        out[1] = c;
+    }
 }
 
 // ---------------------------------------------------------------- K2 ------
@@ -134,12 +169,19 @@ __device__ __forceinline__ bool footprint_axes(const F (&n)[6], F eps, F &sxx, F
 template <typename T, int DEG>
 __global__ void __launch_bounds__(PROJ_THREADS)
 k_project(const float *__restrict__ mx, const float *__restrict__ my, const float *__restrict__ mz,
-          const T *__restrict__ attr, int64_t n_map, const uint32_t *__restrict__ gidx, Layout L,
+          const T *__restrict__ attr, int64_t n_map, const int64_t *__restrict__ run_begin,
+          const int64_t *__restrict__ run_off, int n_runs, uint32_t *__restrict__ gidx, Layout L, int n_blocks,
           const ViewParams *__restrict__ views, CamParams cam, float4 *__restrict__ rec,
-          uint2 *__restrict__ rect, uint32_t *__restrict__ dkey)
+          uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, double *__restrict__ qpart)
 {
     constexpr int K = (DEG + 1) * (DEG + 1);
     __shared__ ViewParams s_view[PROJ_VIEW_BATCH];
+    chain_wait();
+    if ((int)blockIdx.x >= n_blocks) {           // the query images' blocks
+        const int k = (int)blockIdx.x - n_blocks, q = k / QS_BLOCKS;
+        query_partial(L.q_img[q], k - q * QS_BLOCKS, (int64_t)cam.width * cam.height, cam.ncc_gray, qpart + 2 * (int64_t)k);
+        return;
+    }
 
     // this block's query and Gaussians
     const int qi = find_segment(L.q_pblk, L.Q, (int)blockIdx.x);
@@ -153,7 +195,9 @@ k_project(const float *__restrict__ mx, const float *__restrict__ my, const floa
     float m[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // M = R S, row-major
     float sh[3 * K];
     if (active) {
-        const int64_t g = gidx[L.q_gsub[qi] + i];
+        const int64_t at = L.q_gsub[qi] + i;
+        const int64_t g = subset_position(run_begin, run_off, n_runs, at);
+        gidx[at] = (uint32_t)g;                  // for the gradient chains
         mu0 = __ldg(mx + g); mu1 = __ldg(my + g); mu2 = __ldg(mz + g);
         float s0 = ldattr(attr + (ATTR_SCALE + 0) * n_map + g);
         float s1 = ldattr(attr + (ATTR_SCALE + 1) * n_map + g);
@@ -285,35 +329,27 @@ k_project(const float *__restrict__ mx, const float *__restrict__ my, const floa
     }
 }
 
-template <typename T>
-static cudaError_t project_t(const float *mx, const float *my, const float *mz, const T *attr, int sh_degree,
-                             int64_t n_map, const uint32_t *gidx, const Layout &L, int n_blocks,
-                             const ViewParams *views, const CamParams &cam, float4 *rec, uint2 *rect,
-                             uint32_t *dkey, cudaStream_t st)
-{
-    dim3 grid((unsigned)n_blocks);
-    switch (sh_degree) {
-    case 0: k_project<T, 0><<<grid, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, rec, rect, dkey); break;
-    case 1: k_project<T, 1><<<grid, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, rec, rect, dkey); break;
-    case 2: k_project<T, 2><<<grid, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, rec, rect, dkey); break;
-    case 3: k_project<T, 3><<<grid, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, rec, rect, dkey); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
 cudaError_t launch_project(const float *mx, const float *my, const float *mz, const void *attr, int precision,
-                           int sh_degree, int64_t n_map, const uint32_t *gidx, const Layout &L, int n_blocks,
-                           const ViewParams *views, const CamParams &cam, float4 *rec, uint2 *rect,
-                           uint32_t *dkey, cudaStream_t st)
+                           int sh_degree, int64_t n_map, const int64_t *run_begin, const int64_t *run_off, int n_runs,
+                           uint32_t *gidx, const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
+                           float4 *rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st)
 {
-    if (n_blocks <= 0) return cudaSuccess;
-    switch (precision) {
-    case 0: return project_t(mx, my, mz, (const float *)attr, sh_degree, n_map, gidx, L, n_blocks, views, cam, rec, rect, dkey, st);
-    case 1: return project_t(mx, my, mz, (const __half *)attr, sh_degree, n_map, gidx, L, n_blocks, views, cam, rec, rect, dkey, st);
-    case 2: return project_t(mx, my, mz, (const __nv_bfloat16 *)attr, sh_degree, n_map, gidx, L, n_blocks, views, cam, rec, rect, dkey, st);
-    default: return cudaErrorInvalidValue;
-    }
+    const int64_t grid = n_blocks + (qpart ? (int64_t)QS_BLOCKS * L.Q : 0);
+    if (grid <= 0) return cudaSuccess;
+    if (grid > 0x7fffffff) return cudaErrorInvalidValue;
+#define RELOC_PROJECT_CASE(P_, T_, D_)                                                                              \
+    if (precision == P_ && sh_degree == D_)                                                                        \
+        return launch_chained(k_project<T_, D_>, dim3((unsigned)grid), dim3(PROJ_THREADS), 0, st, 1, mx, my, mz,     \
+                              (const T_ *)attr, n_map, run_begin, run_off, n_runs, gidx, L, n_blocks, views, cam, rec, \
+                              rect, dkey, qpart);
+#define RELOC_PROJECT_DEGREES(P_, T_) \
+    RELOC_PROJECT_CASE(P_, T_, 0) RELOC_PROJECT_CASE(P_, T_, 1) RELOC_PROJECT_CASE(P_, T_, 2) RELOC_PROJECT_CASE(P_, T_, 3)
+    RELOC_PROJECT_DEGREES(0, float)
+    RELOC_PROJECT_DEGREES(1, __half)
+    RELOC_PROJECT_DEGREES(2, __nv_bfloat16)
+#undef RELOC_PROJECT_DEGREES
+#undef RELOC_PROJECT_CASE
+    return cudaErrorInvalidValue;
 }
 
 // ------------------------------------------------------------ pose chain --

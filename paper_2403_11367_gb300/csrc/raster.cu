@@ -6,14 +6,11 @@
 // D(x) = sum_i z_i q_i(x) T_i with T_i = prod_{j<i} (1 - q_j(x)), footprint
 // q_i(x) = o_i exp(-1/2 d^T Sigma'^-1 d) (Eq. footprint without the Jacobian
 // normalisation), d = x - mu_hat.  NCC is Eq. ncc over all 3*H*W samples.
+#include <atomic>
+
 #include "internal.cuh"
 
 namespace reloc {
-
-// ------------------------------------------------------ query statistics ---
-
-constexpr int QS_BLOCKS = 152;
-constexpr int QS_THREADS = 256;
 
 __device__ __forceinline__ double warp_sum_d(double x)
 {
@@ -86,67 +83,6 @@ __device__ __forceinline__ float warp_reduce_scatter(float (&v)[NP], int lane)
 #pragma unroll
     for (int o = 16 / NP; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
-}
-
-// Fixed grid and fixed reduction order: the sums are deterministic.
-// grid (QS_BLOCKS, Q): block (b, q) sums its share of query q.
-__global__ void __launch_bounds__(QS_THREADS) k_query_stats(Layout L, int64_t HW, int gray, double *part)
-{
-    __shared__ double s[2][QS_THREADS / 32];
-    const float *q = L.q_img[blockIdx.y];
-    const int64_t n = gray ? HW : 3 * HW;
-    double a = 0, b = 0;
-    for (int64_t j = (int64_t)blockIdx.x * QS_THREADS + threadIdx.x; j < n; j += (int64_t)QS_BLOCKS * QS_THREADS) {
-        const double x = gray ? ((double)q[j] + (double)q[HW + j] + (double)q[2 * HW + j]) / 3.0 : (double)q[j];
-        a += x;
-        b += x * x;
-    }
-    a = warp_sum_d(a);
-    b = warp_sum_d(b);
-    if ((threadIdx.x & 31) == 0) { s[0][threadIdx.x >> 5] = a; s[1][threadIdx.x >> 5] = b; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double A = 0, B = 0;
-        for (int w = 0; w < QS_THREADS / 32; ++w) { A += s[0][w]; B += s[1][w]; }
-        double *o = part + 2 * ((int64_t)blockIdx.y * QS_BLOCKS + blockIdx.x);
-        o[0] = A;
-        o[1] = B;
-    }
-}
-
-// A block per query: its QS_BLOCKS partials summed by a fixed tree (one per
-// thread, then a warp and a block reduction), so the sums are deterministic.
-constexpr int QSF_THREADS = 160;                 // >= QS_BLOCKS, whole warps
-static_assert(QSF_THREADS >= QS_BLOCKS && QSF_THREADS % 32 == 0, "one partial per thread");
-__global__ void __launch_bounds__(QSF_THREADS) k_query_stats_final(const double *part, double *qstats)
-{
-    __shared__ double s[2][QSF_THREADS / 32];
-    const int q = blockIdx.x, k = threadIdx.x;
-    double A = 0, B = 0;
-    if (k < QS_BLOCKS) {
-        A = part[2 * ((int64_t)q * QS_BLOCKS + k)];
-        B = part[2 * ((int64_t)q * QS_BLOCKS + k) + 1];
-    }
-    A = warp_sum_d(A);
-    B = warp_sum_d(B);
-    if ((k & 31) == 0) { s[0][k >> 5] = A; s[1][k >> 5] = B; }
-    __syncthreads();
-    if (k == 0) {
-        A = 0;
-        B = 0;
-        for (int w = 0; w < QSF_THREADS / 32; ++w) { A += s[0][w]; B += s[1][w]; }
-        qstats[2 * q] = A;
-        qstats[2 * q + 1] = B;
-    }
-}
-
-cudaError_t launch_query_stats(const Layout &L, int64_t HW, bool gray, double *block_scratch, double *qstats,
-                               cudaStream_t st)
-{
-    if (L.Q <= 0) return cudaSuccess;
-    k_query_stats<<<dim3(QS_BLOCKS, L.Q), QS_THREADS, 0, st>>>(L, HW, gray ? 1 : 0, block_scratch);
-    k_query_stats_final<<<L.Q, QSF_THREADS, 0, st>>>(block_scratch, qstats);
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ K6 -----
@@ -527,7 +463,7 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
 // SMs) takes the launch's units -- (view, tile, 64-pixel block) of every view
 // of every query in the call -- from one queue (an atomic ticket per unit).
 // The units of heavy tiles (lists of at least BLEND_HEAVY records, listed by
-// k_blend_heavy: the horizon's tiles, whose units run up to twenty times the
+// k_tile_chunk_scan: the horizon's tiles, whose units run up to twenty times the
 // mean) are handed out first, the rest in view-major order (the heavy ones
 // skipped there), so that no long unit starts near the end of the launch.
 // A warp holds its next ticket, the next unit's view and list range while it
@@ -540,22 +476,19 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
 // launches; the export launches (DA) carry depth and alpha sums too and get
 // 72 (28 blocks per SM) rather than spill (same-box A/B: winner export
 // 0.233 -> 0.208 ms).
-constexpr int BLEND_HEAVY = 1024;
-constexpr int BQ_LIST = 4;                       // queue[0] ticket, [1] heavy count, list from [4]
-
-// queue[BQ_LIST + k] = vi * n_tiles + tile for each (view slot, tile) whose
-// list holds at least BLEND_HEAVY records; queue[1] counts them (zeroed on
-// the stream before the launch).  Nothing is listed after an overflow.
+// Lists the heavy tiles of selected views (k_tile_chunk_scan lists those of a
+// sub-batch's own views).  Nothing is listed after an overflow.
 __global__ void k_blend_heavy(const int2 *__restrict__ ranges, const int *__restrict__ view_sel, int n_views,
-                              int n_tiles, const int *__restrict__ overflow, int *__restrict__ queue)
+                              int n_tiles, const int *__restrict__ overflow, BlendQueue queue)
 {
+    chain_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n_views * n_tiles || *overflow != 0) return;
     const int vi = (int)(i / n_tiles), t = (int)(i - (int64_t)vi * n_tiles);
-    const int v = view_sel ? view_sel[vi] : vi;
+    const int v = view_sel[vi];
     if (v < 0) return;
     const int2 r = ranges[(int64_t)v * n_tiles + t];
-    if (r.y - r.x >= BLEND_HEAVY) queue[BQ_LIST + atomicAdd(queue + 1, 1)] = (int)i;
+    if (r.y - r.x >= BLEND_HEAVY) queue.list[atomicAdd(queue.count + 1, 1)] = (int)i;
 }
 
 template <int TW, int TH, int RPL, bool DA>
@@ -563,17 +496,18 @@ __global__ void __launch_bounds__(32, RPL == 1 ? (DA ? 28 : 32) : 24)
 k_blend(const float4 *__restrict__ rec, Layout L, const uint32_t *__restrict__ inst_gauss,
         const int2 *__restrict__ ranges, CamParams cam, double *__restrict__ partials, float *__restrict__ rgb,
         float *__restrict__ depth, float *__restrict__ alpha, const int *__restrict__ view_sel, int n_views,
-        const int *__restrict__ overflow, int *__restrict__ queue)
+        const int *__restrict__ overflow, BlendQueue queue)
 {
     __shared__ float4 s_rec[4][32 * RPL];
+    chain_wait();
     constexpr int WPT = BlockGeom<TW, TH>::WPT;
     const int upv = cam.n_tiles * WPT;                          // units per view
     const int64_t total = (int64_t)upv * n_views;
     const bool ovf = *overflow != 0;
     // heavy units, handed out first (and skipped in order) when the launch
     // listed them
-    const bool listed = blend_launches(n_views) > 1;
-    const int64_t hh = listed ? (int64_t)queue[1] * WPT : 0;
+    const bool listed = blend_heavy_first(n_views);
+    const int64_t hh = listed ? (int64_t)queue.count[1] * WPT : 0;
     const int lane = threadIdx.x;
     // view and list range of unit u (empty past the end or after an overflow)
     auto locate = [&](int64_t u, int &v, int2 &r) {
@@ -589,10 +523,10 @@ k_blend(const float4 *__restrict__ rec, Layout L, const uint32_t *__restrict__ i
     auto next = [&](int64_t &u, int &v, int2 &r) {
         while (true) {
             int64_t t = 0;
-            if (lane == 0) t = atomicAdd(queue, 1);
+            if (lane == 0) t = atomicAdd(queue.count, 1);
             t = __shfl_sync(0xffffffffu, t, 0);
             if (t < hh) {
-                const int h = queue[BQ_LIST + (int)(t / WPT)];
+                const int h = queue.list[(int)(t / WPT)];
                 u = (int64_t)(h / cam.n_tiles) * upv + (int64_t)(h % cam.n_tiles) * WPT + (int)(t % WPT);
                 locate(u, v, r);
                 return;
@@ -622,56 +556,51 @@ k_blend(const float4 *__restrict__ rec, Layout L, const uint32_t *__restrict__ i
     }
 }
 
-// resident one-warp blocks per SM of a blend kernel on the current device
-template <typename K>
-static int resident_blocks(K kernel)
+// One-warp blocks of a blend kernel that fit on the current device at once; kept
+// per kernel (every k_blend has the same function type: one cache for that type
+// gave the scoring launches the export launches' 28 blocks per SM in a process
+// that had rendered first).
+template <int TW, int TH, int RPL, bool DA>
+static int blend_resident()
 {
-    static int cached[64] = {};
+    static std::atomic<int> cached[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (!cached[dev]) {
+    int c = cached[dev].load();
+    if (!c) {
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, 0) != cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blend<TW, TH, RPL, DA>, 32, 0) != cudaSuccess)
             return 0;
-        cached[dev] = sms * (per_sm > 0 ? per_sm : 1);
+        c = sms * (per_sm > 0 ? per_sm : 1);
+        cached[dev].store(c);
     }
-    return cached[dev];
+    return c;
 }
 
 template <int TW, int TH, int RPL>
 static cudaError_t blend_t(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                            const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
-                           const int *view_sel, int n_sel, const int *overflow, int *queue, cudaStream_t st)
+                           const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st)
 {
     const int nv = view_sel ? n_sel : L.V;
     const int64_t units = (int64_t)cam.n_tiles * (TW * TH / 64) * nv;
-    cudaError_t e = cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    if (blend_launches(nv) > 1) {
+    if (view_sel && blend_heavy_first(nv)) {
         const int64_t nt = (int64_t)nv * cam.n_tiles;
-        k_blend_heavy<<<(unsigned)ceil_div(nt, 256), 256, 0, st>>>(ranges, view_sel, nv, cam.n_tiles, overflow,
-                                                                   queue);
+        const cudaError_t e = launch_chained(k_blend_heavy, dim3((unsigned)ceil_div(nt, 256)), dim3(256), 0, st, 1, ranges,
+                                             view_sel, nv, cam.n_tiles, overflow, queue);
+        if (e != cudaSuccess) return e;
     }
-    if (depth || alpha) {
-        const int g = resident_blocks(k_blend<TW, TH, RPL, true>);
-        if (g <= 0) return cudaErrorInvalidValue;
-        k_blend<TW, TH, RPL, true><<<(unsigned)min64(units, g), 32, 0, st>>>(rec, L, inst_gauss, ranges, cam, partials,
-                                                                             rgb, depth, alpha, view_sel, nv, overflow,
-                                                                             queue);
-    } else {
-        const int g = resident_blocks(k_blend<TW, TH, RPL, false>);
-        if (g <= 0) return cudaErrorInvalidValue;
-        k_blend<TW, TH, RPL, false><<<(unsigned)min64(units, g), 32, 0, st>>>(rec, L, inst_gauss, ranges, cam,
-                                                                              partials, rgb, depth, alpha, view_sel, nv,
-                                                                              overflow, queue);
-    }
-    return cudaGetLastError();
+    auto kernel = depth || alpha ? k_blend<TW, TH, RPL, true> : k_blend<TW, TH, RPL, false>;
+    const int g = depth || alpha ? blend_resident<TW, TH, RPL, true>() : blend_resident<TW, TH, RPL, false>();
+    if (g <= 0) return cudaErrorInvalidValue;
+    return launch_chained(kernel, dim3((unsigned)min64(units, g)), dim3(32), 0, st, 1, rec, L, inst_gauss, ranges, cam,
+                          partials, rgb, depth, alpha, view_sel, nv, overflow, queue);
 }
 
 cudaError_t launch_blend(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                          const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
-                         const int *view_sel, int n_sel, const int *overflow, int *queue, cudaStream_t st)
+                         const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st)
 {
     if ((view_sel ? n_sel : L.V) <= 0) return cudaSuccess;
 #define RELOC_BLEND_CASE(W_, H_, R_)                                                                             \
@@ -701,11 +630,13 @@ cudaError_t launch_blend(const float4 *rec, const Layout &L, const uint32_t *ins
 constexpr int NCC_THREADS = 256;
 
 __global__ void __launch_bounds__(NCC_THREADS)
-k_ncc_finalize(const double *__restrict__ partials, const double *__restrict__ qstats, Layout L, int n_units,
+k_ncc_finalize(const double *__restrict__ partials, const double *__restrict__ qpart, Layout L, int n_units,
                int64_t n, double *__restrict__ scores, int *__restrict__ degenerate, double *__restrict__ coef)
 {
-    __shared__ double s[3][NCC_THREADS / 32];
+    __shared__ double s[5][NCC_THREADS / 32];
+    chain_wait();
     const int v = blockIdx.x;
+    const int q = L.view_q[v];
     const double *p = partials + (int64_t)v * n_units * 3;
     double a = 0, b = 0, c = 0;
     for (int t = threadIdx.x; t < n_units; t += NCC_THREADS) {
@@ -716,14 +647,25 @@ k_ncc_finalize(const double *__restrict__ partials, const double *__restrict__ q
     a = warp_sum_d(a);
     b = warp_sum_d(b);
     c = warp_sum_d(c);
-    if ((threadIdx.x & 31) == 0) { s[0][threadIdx.x >> 5] = a; s[1][threadIdx.x >> 5] = b; s[2][threadIdx.x >> 5] = c; }
+    // the query's partial sums
+    double d = 0, e = 0;
+    for (int t = threadIdx.x; t < QS_BLOCKS; t += NCC_THREADS) {
+        d += qpart[2 * ((int64_t)q * QS_BLOCKS + t)];
+        e += qpart[2 * ((int64_t)q * QS_BLOCKS + t) + 1];
+    }
+    d = warp_sum_d(d);
+    e = warp_sum_d(e);
+    if ((threadIdx.x & 31) == 0) {
+        const int w = threadIdx.x >> 5;
+        s[0][w] = a; s[1][w] = b; s[2][w] = c; s[3][w] = d; s[4][w] = e;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double Sr = 0, Srr = 0, Srq = 0;
-        for (int w = 0; w < NCC_THREADS / 32; ++w) { Sr += s[0][w]; Srr += s[1][w]; Srq += s[2][w]; }
+        double Sr = 0, Srr = 0, Srq = 0, Sq = 0, Sqq = 0;
+        for (int w = 0; w < NCC_THREADS / 32; ++w) {
+            Sr += s[0][w]; Srr += s[1][w]; Srq += s[2][w]; Sq += s[3][w]; Sqq += s[4][w];
+        }
         const double nn = (double)n;
-        const int q = L.view_q[v];
-        const double Sq = qstats[2 * q], Sqq = qstats[2 * q + 1];
         const double cov = Srq - Sr * Sq / nn;
         const double vr = Srr - Sr * Sr / nn;
         const double vq = Sqq - Sq * Sq / nn;
@@ -741,12 +683,12 @@ k_ncc_finalize(const double *__restrict__ partials, const double *__restrict__ q
     }
 }
 
-cudaError_t launch_ncc_finalize(const double *partials, const double *qstats, const Layout &L, int n_units,
+cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, const Layout &L, int n_units,
                                 int64_t n_samples, double *scores, int *degenerate, double *coef, cudaStream_t st)
 {
     if (L.V <= 0) return cudaSuccess;
-    k_ncc_finalize<<<L.V, NCC_THREADS, 0, st>>>(partials, qstats, L, n_units, n_samples, scores, degenerate, coef);
-    return cudaGetLastError();
+    return launch_chained(k_ncc_finalize, dim3(L.V), dim3(NCC_THREADS), 0, st, 1, partials, qpart, L, n_units, n_samples,
+                          scores, degenerate, coef);
 }
 
 // ------------------------------------------------------- K6 backward ------
@@ -1113,6 +1055,7 @@ k_argmax(const double *__restrict__ scores, Layout L, int *best, double *best_sc
 {
     __shared__ double s_s[256];
     __shared__ int s_i[256];
+    chain_wait();
     const int q = blockIdx.x;
     const int v0 = L.q_view[q], V = L.q_view[q + 1] - v0;
     double bs = -INFINITY;
@@ -1141,8 +1084,7 @@ cudaError_t launch_argmax(const double *scores, const Layout &L, int *best, doub
                           cudaStream_t st)
 {
     if (L.Q <= 0) return cudaSuccess;
-    k_argmax<<<L.Q, 256, 0, st>>>(scores, L, best, best_score, view_sel);
-    return cudaGetLastError();
+    return launch_chained(k_argmax, dim3(L.Q), dim3(256), 0, st, 1, scores, L, best, best_score, view_sel);
 }
 
 }  // namespace reloc

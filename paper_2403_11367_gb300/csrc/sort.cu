@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 16 ? 2 : 1)
 k_depth_sort(const uint32_t *__restrict__ dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, Layout L, uint32_t *n_vis)
 {
     __shared__ DepthSortShared<NW> sm;
+    chain_wait();
     const int C = (int)cooperative_groups::this_cluster().num_blocks();
     const int v = blockIdx.x / C;
     const int64_t off = L.vd_off[v];
@@ -251,19 +252,10 @@ cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, ui
     const int most = L.V <= 32 ? DS_MAX_CLUSTER : DS_MAX_CLUSTER / 2;
     int C = 1;
     while (C < most && (int64_t)C * 2048 < longest) C *= 2;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(C * L.V));
-    const bool wide = L.V <= DS_WIDE_VIEWS;
-    cfg.blockDim = dim3(wide ? 1024 : 512);
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return wide ? cudaLaunchKernelEx(&cfg, k_depth_sort<32>, dkey, bufA, bufB, out, L, n_vis)
-                : cudaLaunchKernelEx(&cfg, k_depth_sort<16>, dkey, bufA, bufB, out, L, n_vis);
+    const dim3 grid((unsigned)(C * L.V));
+    return L.V <= DS_WIDE_VIEWS
+               ? launch_chained(k_depth_sort<32>, grid, dim3(1024), 0, st, C, dkey, bufA, bufB, out, L, n_vis)
+               : launch_chained(k_depth_sort<16>, grid, dim3(512), 0, st, C, dkey, bufA, bufB, out, L, n_vis);
 }
 
 // --------------------------------------- depth sort, launches per pass -----
@@ -487,6 +479,7 @@ k_tile_count(const uint32_t *__restrict__ sorted_g, const uint32_t *__restrict__
              uint32_t *__restrict__ bhist)
 {
     extern __shared__ uint32_t s_d[];   // (band_rows + 1) x (ntx + 1)
+    chain_wait();
     const int c = blockIdx.x;
     const int v = find_segment(L.cb_base, L.V, c);
     const int k = c - L.cb_base[v];
@@ -556,23 +549,29 @@ k_tile_count(const uint32_t *__restrict__ sorted_g, const uint32_t *__restrict__
 
 // Per view: bhist[chunk][tile] becomes the exclusive prefix over the view's
 // chunks (each chunk's first slot inside a tile's list, relative to the
-// tile's start), totals -> ranges[v][tile].y; then a block per view scans
-// the totals in tile order into ranges[v][tile] = [begin, end) (empty tiles
-// [0, 0)) and n_inst[v].  The chunk prefix: a block per (view, 32 tiles),
-// SEGS threads per tile, each holding up to TCOL_SEG of the tile's chunks in
-// registers (all its loads in flight at once), so a view's ~80 chunks are
-// scanned as eight short runs plus a prefix over the eight run totals, and the
-// hundreds of smaller chunks of a call of few views as 32 runs.
+// tile's start), totals -> ranges[v][tile].y; then the view's last block to
+// finish scans the totals in tile order into ranges[v][tile] = [begin, end)
+// (empty tiles [0, 0)) and n_inst[v], and lists the heavy tiles for the blend
+// (two launches less than with kernels of their own).  The chunk prefix: a block
+// per (view, 32 tiles), SEGS threads per tile, each holding up to TCOL_SEG of the
+// tile's chunks in registers (all its loads in flight at once), so a view's ~80
+// chunks are scanned as eight short runs plus a prefix over the eight run totals,
+// and the hundreds of smaller chunks of a call of few views as 32 runs.
 constexpr int TCOL_TILES = 32;
 constexpr int TCOL_SEG = 16;                         // chunks per run in registers
-constexpr int TSCAN_THREADS = 1024;
+constexpr int TSCAN_PER = 4;                         // tiles per thread and round of the final scan
 
 template <int SEGS>
 __global__ void __launch_bounds__(TCOL_TILES * SEGS, SEGS > 8 ? 1 : 4)
 k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, uint32_t *__restrict__ bhist,
-                  int2 *__restrict__ ranges)
+                  int2 *ranges, uint32_t *__restrict__ n_inst, int *__restrict__ done, int *__restrict__ overflow,
+                  BlendQueue queue)
 {
+    constexpr int NT = TCOL_TILES * SEGS;
     __shared__ uint32_t s_run[SEGS][TCOL_TILES];
+    __shared__ uint32_t s_tmp[33];
+    __shared__ int s_last;
+    chain_wait();
     const int v = blockIdx.y;
     const int tl = threadIdx.x % TCOL_TILES, sg = threadIdx.x / TCOL_TILES;
     const int t = blockIdx.x * TCOL_TILES + tl;
@@ -581,62 +580,63 @@ k_tile_chunk_scan(const uint32_t *__restrict__ n_vis, Layout L, CamParams cp, ui
     const int64_t nv = min64(n_vis[v], S);
     const int nch = (int)ceil_div(nv, cp.bin_chunk);
     uint32_t *h = bhist + (int64_t)nt * L.cb_base[v] + t;
-    const int per = (int)ceil_div(nch, SEGS);      // chunks of this thread's run
-    const int c0 = sg * per, c1 = min(nch, c0 + per);
-    uint32_t sum = 0;
+    int2 *const R = ranges + (int64_t)v * nt;
+    const int per = (int)ceil_div(nch, SEGS);           // chunks of this thread's run
+    const int c0 = min(nch, sg * per), c1 = min(nch, c0 + per);
+    const int m = t < nt ? c1 - c0 : 0;
+    uint32_t *hp = h + (int64_t)c0 * nt;
+    uint32_t sum = 0, x[TCOL_SEG];
     if (per <= TCOL_SEG) {                              // uniform over the block
-        uint32_t x[TCOL_SEG];
-        uint32_t *hp = h + (int64_t)c0 * nt;
-        const int m = t < nt ? c1 - c0 : 0;
 #pragma unroll
         for (int j = 0; j < TCOL_SEG; ++j) x[j] = j < m ? hp[(int64_t)j * nt] : 0u;
 #pragma unroll
         for (int j = 0; j < TCOL_SEG; ++j) sum += x[j];
-        s_run[sg][tl] = sum;
-        __syncthreads();
-        if (t >= nt) return;
-        uint32_t run = 0;
-        for (int k = 0; k < sg; ++k) run += s_run[k][tl];
+    } else {                                            // views of more than SEGS * TCOL_SEG chunks
+        for (int j = 0; j < m; ++j) sum += hp[(int64_t)j * nt];
+    }
+    s_run[sg][tl] = sum;
+    __syncthreads();
+    uint32_t run = 0;
+    for (int k = 0; k < sg; ++k) run += s_run[k][tl];
+    if (per <= TCOL_SEG) {
 #pragma unroll
         for (int j = 0; j < TCOL_SEG; ++j)
             if (j < m) {
                 hp[(int64_t)j * nt] = run;
                 run += x[j];
             }
-        if (sg == SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
-        return;
+    } else {
+        for (int j = 0; j < m; ++j) {
+            const uint32_t y = hp[(int64_t)j * nt];
+            hp[(int64_t)j * nt] = run;
+            run += y;
+        }
     }
-    // long views (more than SEGS * TCOL_SEG chunks) or tiles past the
-    // grid: runs summed first, then rewritten
-    if (t < nt)
-        for (int c = c0; c < c1; ++c) sum += h[(int64_t)c * nt];
-    s_run[sg][tl] = sum;
+    if (sg == SEGS - 1 && t < nt) __stcg(&R[t].y, (int)run);
+    // the view's last block scans the totals of all its tiles
+    __threadfence();
     __syncthreads();
-    if (t >= nt) return;
-    uint32_t run = 0;
-    for (int k = 0; k < sg; ++k) run += s_run[k][tl];
-    for (int c = c0; c < c1; ++c) {
-        const uint32_t x = h[(int64_t)c * nt];
-        h[(int64_t)c * nt] = run;
-        run += x;
-    }
-    if (sg == SEGS - 1) ranges[(int64_t)v * nt + t].y = (int)run;
-}
-
-__global__ void __launch_bounds__(TSCAN_THREADS)
-k_tile_scan(Layout L, CamParams cp, int2 *__restrict__ ranges, uint32_t *__restrict__ n_inst, int *overflow)
-{
-    __shared__ uint32_t s_tmp[33];
-    const int v = blockIdx.x;
-    const int nt = cp.n_tiles;
-    int2 *R = ranges + (int64_t)v * nt;
+    if (threadIdx.x == 0) s_last = atomicAdd(done + v, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     uint32_t carry = 0;
-    for (int t0 = 0; t0 < nt; t0 += TSCAN_THREADS) {
-        const int t = t0 + threadIdx.x;
-        const uint32_t x = t < nt ? (uint32_t)R[t].y : 0u;
-        uint32_t tot;
-        const uint32_t start = carry + block_excl_scan(x, s_tmp, &tot);
-        if (t < nt) R[t] = x ? make_int2((int)start, (int)(start + x)) : make_int2(0, 0);
+    for (int t0 = 0; t0 < nt; t0 += NT * TSCAN_PER) {
+        const int a = t0 + (int)threadIdx.x * TSCAN_PER;
+        uint32_t y[TSCAN_PER], mine = 0, tot;
+#pragma unroll
+        for (int j = 0; j < TSCAN_PER; ++j) {
+            y[j] = a + j < nt ? (uint32_t)__ldcg(&R[a + j].y) : 0u;
+            mine += y[j];
+        }
+        uint32_t at = carry + block_excl_scan(mine, s_tmp, &tot);
+#pragma unroll
+        for (int j = 0; j < TSCAN_PER; ++j) {
+            if (a + j >= nt) break;
+            R[a + j] = y[j] ? make_int2((int)at, (int)(at + y[j])) : make_int2(0, 0);
+            if (queue.count && y[j] >= (uint32_t)BLEND_HEAVY) queue.list[atomicAdd(queue.count + 1, 1)] = v * nt + a + j;
+            at += y[j];
+        }
         carry += tot;
     }
     if (threadIdx.x == 0) {
@@ -647,24 +647,27 @@ k_tile_scan(Layout L, CamParams cp, int2 *__restrict__ ranges, uint32_t *__restr
 
 cudaError_t launch_tile_count(const uint32_t *sorted_g, const uint32_t *n_vis, const uint2 *rect, const Layout &L,
                               const CamParams &cp, int n_chunks, int view_chunks, uint2 *srect, uint32_t *bhist,
-                              int2 *ranges, uint32_t *n_inst, int *overflow, cudaStream_t st)
+                              int2 *ranges, uint32_t *n_inst, int *done, int *overflow, BlendQueue queue,
+                              cudaStream_t st)
 {
     if (L.V <= 0) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
     if (n_chunks > 0) {
         const int W = cp.ntx + 1;
         const int band_rows = max(1, min(cp.nty, TILE_COUNT_SMEM / (4 * W) - 1));
         const size_t smem = 4 * (size_t)(band_rows + 1) * W;
-        k_tile_count<<<n_chunks, BIN_THREADS, smem, st>>>(sorted_g, n_vis, rect, L, cp, band_rows, srect, bhist);
+        e = launch_chained(k_tile_count, dim3(n_chunks), dim3(BIN_THREADS), smem, st, 1, sorted_g, n_vis, rect, L, cp,
+                           band_rows, srect, bhist);
+        if (e != cudaSuccess) return e;
     }
     const dim3 cgrid((unsigned)ceil_div(cp.n_tiles, TCOL_TILES), L.V);
     // by the chunks a view may have; about a third of them hold visible Gaussians,
     // and the wide form costs the 64 views of 157 chunks 48 us more (147 for 99 us)
     if (view_chunks <= 4 * 8 * TCOL_SEG)
-        k_tile_chunk_scan<8><<<cgrid, TCOL_TILES * 8, 0, st>>>(n_vis, L, cp, bhist, ranges);
-    else
-        k_tile_chunk_scan<32><<<cgrid, TCOL_TILES * 32, 0, st>>>(n_vis, L, cp, bhist, ranges);
-    k_tile_scan<<<L.V, TSCAN_THREADS, 0, st>>>(L, cp, ranges, n_inst, overflow);
-    return cudaGetLastError();
+        return launch_chained(k_tile_chunk_scan<8>, cgrid, dim3(TCOL_TILES * 8), 0, st, 1, n_vis, L, cp, bhist, ranges,
+                              n_inst, done, overflow, queue);
+    return launch_chained(k_tile_chunk_scan<32>, cgrid, dim3(TCOL_TILES * 32), 0, st, 1, n_vis, L, cp, bhist, ranges,
+                          n_inst, done, overflow, queue);
 }
 
 // ------------------------------------------------------ K4 tile emission ----
@@ -742,6 +745,7 @@ k_tile_emit_flat(const uint32_t *__restrict__ sorted_g, const uint2 *__restrict_
     __shared__ uint32_t s_load[32];                     // DYN: the chunk's instances per row
     __shared__ int s_order[32];                         // DYN: rows, heaviest first
     __shared__ int s_next;
+    chain_wait();
     const EmitChunk ch = emit_chunk(n_vis, n_inst, L, cp);
     if (ch.skip) return;
     const int v = ch.v, n = ch.n;
@@ -954,6 +958,7 @@ k_tile_emit_smem(const uint32_t *__restrict__ sorted_g, const uint2 *__restrict_
     __shared__ uint32_t s_g[EMIT_STAGE];
     __shared__ uint2 s_q[TILE_EMIT_WARPS][64];
     extern __shared__ uint32_t s_cnt[];                 // [TILE_EMIT_WARPS][ntx]
+    chain_wait();
     const EmitChunk ch = emit_chunk(n_vis, n_inst, L, cp);
     if (ch.skip) return;
     const int v = ch.v, n = ch.n;
@@ -1029,27 +1034,20 @@ cudaError_t launch_tile_emit(const uint32_t *sorted_g, const uint2 *srect, const
     // has ~80); fewer take a block per (chunk, eight rows)
     const bool rm = cp.nty <= 32, dyn = rm && cp.bin_chunk <= EMIT_STAGE && n_chunks >= EMIT_DYN_MIN_CHUNKS;
     const dim3 grid1(n_chunks, 1);
+    const dim3 block(TILE_EMIT_WARPS * 32);
 #define EMIT_FLAT(CPL_)                                                                                         \
-    if (dyn)                                                                                                    \
-        k_tile_emit_flat<CPL_, true, true><<<grid1, TILE_EMIT_WARPS * 32, 0, st>>>(                             \
-            sorted_g, srect, n_vis, n_inst, bhist, ranges, L, cp, inst_gauss);                                  \
-    else if (rm)                                                                                                \
-        k_tile_emit_flat<CPL_, true, false><<<grid, TILE_EMIT_WARPS * 32, 0, st>>>(                             \
-            sorted_g, srect, n_vis, n_inst, bhist, ranges, L, cp, inst_gauss);                                  \
-    else                                                                                                        \
-        k_tile_emit_flat<CPL_, false, false><<<grid, TILE_EMIT_WARPS * 32, 0, st>>>(                            \
-            sorted_g, srect, n_vis, n_inst, bhist, ranges, L, cp, inst_gauss)
-    if (cp.ntx <= 128) {
-        EMIT_FLAT(4);
-    } else if (cp.ntx <= EMIT_FLAT_MAX_NTX) {
-        EMIT_FLAT(8);
+    return dyn  ? launch_chained(k_tile_emit_flat<CPL_, true, true>, grid1, block, 0, st, 1, sorted_g, srect,    \
+                                 n_vis, n_inst, bhist, ranges, L, cp, inst_gauss)                               \
+           : rm ? launch_chained(k_tile_emit_flat<CPL_, true, false>, grid, block, 0, st, 1, sorted_g, srect,    \
+                                 n_vis, n_inst, bhist, ranges, L, cp, inst_gauss)                               \
+                : launch_chained(k_tile_emit_flat<CPL_, false, false>, grid, block, 0, st, 1, sorted_g, srect,   \
+                                 n_vis, n_inst, bhist, ranges, L, cp, inst_gauss)
+    if (cp.ntx <= 128) EMIT_FLAT(4);
+    if (cp.ntx <= EMIT_FLAT_MAX_NTX) EMIT_FLAT(8);
 #undef EMIT_FLAT
-    } else {
-        const size_t smem = 4 * (size_t)TILE_EMIT_WARPS * cp.ntx;
-        k_tile_emit_smem<<<grid, TILE_EMIT_WARPS * 32, smem, st>>>(sorted_g, srect, n_vis, n_inst, bhist, ranges,
-                                                                  L, cp, inst_gauss);
-    }
-    return cudaGetLastError();
+    const size_t smem = 4 * (size_t)TILE_EMIT_WARPS * cp.ntx;
+    return launch_chained(k_tile_emit_smem, grid, block, smem, st, 1, sorted_g, srect, n_vis, n_inst, bhist, ranges, L, cp,
+                          inst_gauss);
 }
 
 cudaError_t configure_sort_kernels()
