@@ -704,6 +704,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     const int64_t HW = (int64_t)cp.width * cp.height;
     const Layout &L = sb.L;
     const ResultBlock &R = ctx->res_at;
+    const Records rec{ctx->rec.as<float4>(), ctx->rec.as<float4>() + 2 * sb.VS};
     int *d_overflow = R.overflow;
     uint32_t *nvis = R.nvis + sb.v0;
     uint32_t *ninst = R.ninst + sb.v0;
@@ -713,7 +714,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     if (sb.pblk > 0 || o.score) {
         CK(launch_project(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n, ctx->mean.as<float>() + 2 * ctx->n,
                           ctx->attr.p, ctx->precision, ctx->sh_degree, ctx->n, sb.d_run_begin, sb.d_run_off, sb.n_runs,
-                          ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->rec.as<float4>(),
+                          ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, rec,
                           ctx->rect.as<uint2>(), ctx->dkey.as<uint32_t>(), o.score ? ctx->qpart.as<double>() : nullptr, st));
         launches += 1;
     }
@@ -782,7 +783,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     const bool rp = o.target && o.rel;
     float *dep_out = rp ? ctx->tdep.as<float>() : (o.depth ? o.depth + (int64_t)sb.v0 * HW : nullptr);
     float *alp_out = rp ? ctx->talp.as<float>() : (o.alpha ? o.alpha + (int64_t)sb.v0 * HW : nullptr);
-    CK(launch_blend(ctx->rec.as<float4>(), L, fgauss, ctx->ranges.as<int2>(), cp,
+    CK(launch_blend(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
                     o.score ? ctx->partials.as<double>() : nullptr, rgb_out, dep_out, alp_out,
                     nullptr, 0, d_overflow, queue, st));
     launches += blend_launches(L.V, false);
@@ -818,7 +819,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
             }
         }
         CK(cudaMemsetAsync(ctx->gbuf.p, 0, 40 * (size_t)sb.VS, st));
-        CK(launch_blend_grad(ctx->rec.as<float4>(), L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
+        CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
                              ctx->tgimg.as<float>(), rp ? ctx->tgda.as<float>() : nullptr, ctx->trgb.as<float>(),
                              rp ? ctx->tdep.as<float>() : nullptr, rp ? ctx->talp.as<float>() : nullptr,
                              ctx->gbuf.as<float>(), d_overflow, st));
@@ -835,7 +836,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         launches += 1;
         if (o.grad) {
             CK(cudaMemsetAsync(ctx->gbuf.p, 0, 20 * (size_t)sb.VS, st));
-            CK(launch_blend_grad(ctx->rec.as<float4>(), L, fgauss, ctx->ranges.as<int2>(), cp,
+            CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
                                  ctx->gcoef.as<double>(), nullptr, nullptr, nullptr, nullptr, nullptr,
                                  ctx->gbuf.as<float>(), d_overflow, st));
             CK(launch_pose_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
@@ -850,7 +851,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
             launches += 1;
             if (o.brgb || o.bdepth || o.balpha) {
                 const int nq = sb.q1 - sb.q0;
-                CK(launch_blend(ctx->rec.as<float4>(), L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
+                CK(launch_blend(rec, L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
                                 o.brgb ? o.brgb + (int64_t)sb.q0 * 3 * HW : nullptr,
                                 o.bdepth ? o.bdepth + (int64_t)sb.q0 * HW : nullptr,
                                 o.balpha ? o.balpha + (int64_t)sb.q0 * HW : nullptr, vsel, nq, d_overflow,
@@ -1743,8 +1744,11 @@ extern "C" reloc_status reloc_export_debug(reloc_ctx *ctx, float *records_dev, i
     CK(cudaSetDevice(ctx->device));
     const int64_t VS = (int64_t)ctx->last_V * ctx->last_S;
     const size_t VI = (size_t)ctx->last_io_off.back();
-    if (records_dev && VS > 0)
-        CK(cudaMemcpyAsync(records_dev, ctx->rec.p, 48 * (size_t)VS, cudaMemcpyDeviceToDevice, st));
+    if (records_dev && VS > 0) {
+        CK(cudaMemcpy2DAsync(records_dev, 48, ctx->rec.p, 32, 32, (size_t)VS, cudaMemcpyDeviceToDevice, st));
+        CK(cudaMemcpy2DAsync(records_dev + 8, 48, ctx->rec.as<float4>() + 2 * VS, 16, 16, (size_t)VS,
+                             cudaMemcpyDeviceToDevice, st));
+    }
     if (rects_dev && VS > 0) {
         k_unpack_rect<<<(unsigned)ceil_div(VS, 256), 256, 0, st>>>(ctx->rect.as<uint2>(), ctx->dkey.as<uint32_t>(), VS,
                                                                   rects_dev);

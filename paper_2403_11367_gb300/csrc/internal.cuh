@@ -96,6 +96,22 @@ __device__ __forceinline__ int find_segment(const int32_t *base, int n, int x)
 
 constexpr int PROJ_THREADS = 128;
 
+// ---- projected records ----------------------------------------------------------
+// Per (view, Gaussian), 48 bytes in two arrays: geom[2 i] = (u, v, depth, log2 o),
+// geom[2 i + 1] = the principal axes, 32 bytes on a 32-byte boundary, so that a
+// lane fetches them with one 256-bit load; col[i] = (red, green, blue, 0), which
+// only the records that a block keeps need.
+struct Records {
+    float4 *geom, *col;
+};
+// One record's geometry.
+__device__ __forceinline__ void load_geom(const float4 *geom, int64_t i, float4 &a, float4 &b)
+{
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(geom + 2 * i));
+}
+
 // ---- launch chaining ----------------------------------------------------------
 // The kernels of a call form one chain on its stream.  A kernel launched by
 // launch_chained is set up while the one before still runs (programmatic
@@ -141,7 +157,7 @@ cudaError_t launch_project(const float *mx, const float *my, const float *mz, co
                            int precision, int sh_degree, int64_t n_map, const int64_t *run_begin,
                            const int64_t *run_off, int n_runs, uint32_t *gidx,
                            const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
-                           float4 *rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st);
+                           Records rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st);
 
 // Depth sort of every view's visible Gaussians in one launch: out[vd_off[v] + k]
 // = index of the k-th nearest (ties by index), n_vis[v] their number.  dkey:
@@ -227,7 +243,7 @@ cudaError_t launch_fill_tiles(const int2 *ranges_view, int n_tiles, uint32_t *ti
 // slot k for view_sel[k].  queue: a work queue of blend_list_ints(cam, n) entries
 // for n views, with the heavy tiles listed by launch_tile_count or, for selected
 // views, here.  blend_launches(n, selected) launches.
-cudaError_t launch_blend(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+cudaError_t launch_blend(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                          const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
                          const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st);
 
@@ -257,7 +273,7 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // gout[vd_off[v] + i][10] (u, v, a, b, c, r, g, b, opacity, z); cimg (may be
 // null) [V][3][H][W] the views' forward render (cdep, calp [V][H][W] its depth
 // and alpha, needed with gda) so the colour need not be composited again.
-cudaError_t launch_blend_grad(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
                               const int *overflow, cudaStream_t st);

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(PROJ_THREADS)
 k_project(const float *__restrict__ mx, const float *__restrict__ my, const float *__restrict__ mz,
           const T *__restrict__ attr, int64_t n_map, const int64_t *__restrict__ run_begin,
           const int64_t *__restrict__ run_off, int n_runs, uint32_t *__restrict__ gidx, Layout L, int n_blocks,
-          const ViewParams *__restrict__ views, CamParams cam, float4 *__restrict__ rec,
+          const ViewParams *__restrict__ views, CamParams cam, Records rec,
           uint2 *__restrict__ rect, uint32_t *__restrict__ dkey, double *__restrict__ qpart)
 {
     constexpr int K = (DEG + 1) * (DEG + 1);
@@ -314,10 +314,9 @@ k_project(const float *__restrict__ mx, const float *__restrict__ my, const floa
                         // sqrt(log2(e) / 2), so that the base-2 exponent is
                         // log2(o) - (alpha' . d)^2 - (beta' . d)^2
                         constexpr float KAPPA = 0.8493218002880191f;
-                        float4 *rp = rec + 3 * o;
-                        rp[0] = make_float4(u, vpx, tz, lopac);
-                        rp[1] = make_float4(KAPPA * ab[0], KAPPA * ab[1], KAPPA * ab[2], KAPPA * ab[3]);
-                        rp[2] = make_float4(cr, cg, cbl, 0.f);
+                        rec.geom[2 * o] = make_float4(u, vpx, tz, lopac);
+                        rec.geom[2 * o + 1] = make_float4(KAPPA * ab[0], KAPPA * ab[1], KAPPA * ab[2], KAPPA * ab[3]);
+                        rec.col[o] = make_float4(cr, cg, cbl, 0.f);
                     }
                 }
             }
@@ -332,7 +331,7 @@ k_project(const float *__restrict__ mx, const float *__restrict__ my, const floa
 cudaError_t launch_project(const float *mx, const float *my, const float *mz, const void *attr, int precision,
                            int sh_degree, int64_t n_map, const int64_t *run_begin, const int64_t *run_off, int n_runs,
                            uint32_t *gidx, const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
-                           float4 *rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st)
+                           Records rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st)
 {
     const int64_t grid = n_blocks + (qpart ? (int64_t)QS_BLOCKS * L.Q : 0);
     if (grid <= 0) return cudaSuccess;

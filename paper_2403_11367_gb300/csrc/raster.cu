@@ -140,7 +140,7 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
     return d;
 }
 
-// Records carry (u, v, depth, log2 o | a1, a2, b1, b2 | r, g, b, -): the
+// Records carry (u, v, depth, log2 o | a1, a2, b1, b2) and (r, g, b, -): the
 // footprint in principal-axis form, scaled for base 2: with d the offset of a
 // pixel centre from the projected mean, U = a1 dx + a2 dy and V = b1 dx + b2 dy,
 // the exponent is p' = log2(o) + power log2(e) = log2(o) - (U^2 + V^2), so
@@ -254,7 +254,7 @@ __device__ __forceinline__ float step_lt(float a, float b)
 // One 64-pixel warp block (unit `unit` of view v, its list range r): the
 // blend and the epilogue (image export to slot out_v, NCC partials).
 template <int TW, int TH, int RPL, bool DA>
-__device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const Layout &L,
+__device__ __forceinline__ void blend_unit(const Records &rec, const Layout &L,
                                            const uint32_t *__restrict__ inst_gauss, const CamParams &cam,
                                            double *__restrict__ partials, float *__restrict__ rgb,
                                            float *__restrict__ depth, float *__restrict__ alpha, int v, int out_v,
@@ -263,8 +263,11 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
     using GM = BlockGeom<TW, TH>;
     constexpr int BW = GM::BW, BH = GM::BH, WPT = GM::WPT;
     constexpr int CH = 32 * RPL;             // records per warp step
-    // kept records compacted in s_rec: (-qa, Gx, -2 qb, Gy) (-qc, -qc, P0, thr)
-    // (r, r, g, g) (b, b, z, z)
+    // kept records compacted in s_rec: (-qa, Gx, -2 qb, Gy) (-qc, P0, thr, b)
+    // (r, r, g, g) and for DA (z).  The pixel loop reads them back by broadcast,
+    // and the shared-memory pipe hands out eight bytes a cycle: with the gather
+    // it was 88% busy at 56 bytes a record (the issue slots 73%), so what costs no
+    // instruction to duplicate is stored once, 48 bytes.
     const int tile = unit / WPT, warp = unit - tile * WPT;
     const int tx = tile % cam.ntx, ty = tile / cam.ntx;
     const int lane = threadIdx.x;
@@ -277,10 +280,9 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
     // centre of the block's pixel centres and this lane's offsets from it (exact)
     const float ocx = (float)bx0p + 0.5f * BW, ocy = (float)by0p + 0.5f * BH;
     const float DX = (float)(lane % BW) + 0.5f - 0.5f * BW;
-    const float dy0 = (float)(2 * (lane / BW)) + 0.5f - 0.5f * BH;
-    const f32x2 DY2 = pk(dy0, dy0 + 1.f);
+    const float dy0 = (float)(2 * (lane / BW)) + 0.5f - 0.5f * BH, dy1 = dy0 + 1.f;
     const uint32_t *list = inst_gauss + L.io_off[v];
-    const float4 *vrec = rec + L.vd_off[v] * 3;
+    const float4 *geom = rec.geom + 2 * L.vd_off[v], *col = rec.col + L.vd_off[v];
     constexpr float L2E = 1.4426950408889634f;
     const float limL = -0.5f * cam.cut * cam.cut * L2E;
     const float l2amin = log2f(cam.alpha_min);
@@ -293,15 +295,16 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
     f32x2 R2 = 0ull, G2 = 0ull, B2 = 0ull, Z2 = 0ull, S2 = 0ull;
     const f32x2 NEG1 = pk(-1.f, -1.f);
 
-    // software pipeline: list indices two steps ahead, records one step ahead
+    // software pipeline: list indices two steps ahead, geometry one step ahead
     uint32_t gnext[RPL];
     float4 qa[RPL], qb[RPL], qc[RPL];
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
         const int j0 = r.x + q * 32 + lane, j1 = j0 + CH;
         if (j0 < r.y) {
-            const float4 *p = vrec + 3 * (int64_t)__ldg(list + j0);
-            qa[q] = __ldg(p); qb[q] = __ldg(p + 1); qc[q] = __ldg(p + 2);
+            const uint32_t g = __ldg(list + j0);
+            load_geom(geom, g, qa[q], qb[q]);
+            qc[q] = __ldg(col + g);
         }
         gnext[q] = j1 < r.y ? __ldg(list + j1) : 0u;
     }
@@ -331,11 +334,11 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
             // issue the next step's loads before working on this one
             const int jn = j + CH, jnn = j + 2 * CH;
             if (jn < r.y) {
-                const float4 *p = vrec + 3 * (int64_t)gnext[q];
-                qa[q] = __ldg(p); qb[q] = __ldg(p + 1); qc[q] = __ldg(p + 2);
+                load_geom(geom, gnext[q], qa[q], qb[q]);
+                qc[q] = __ldg(col + gnext[q]);
             }
             gnext[q] = jnn < r.y ? __ldg(list + jnn) : 0u;
-            // pa: u v z log2(o) | pb: scaled axes | pc: rgb.  A pixel counts iff
+            // pa: u v z log2(o) | pb: scaled axes.  A pixel counts iff
             // q <= min(-limL, log2 o - log2 alpha_min); keep the record iff the
             // ellipse at that bound (plus a margin for the float arithmetic,
             // widened 1%) meets the box
@@ -351,9 +354,9 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
                 float4 t0, t1;
                 block_stage(pa, pb, cq, fmaxf(limL + pa.w, l2amin), ocx, ocy, t0, t1);
                 sw[0][k] = t0;
-                sw[1][k] = t1;
+                sw[1][k] = make_float4(t1.x, t1.z, t1.w, pc.z);
                 sw[2][k] = make_float4(pc.x, pc.x, pc.y, pc.y);
-                sw[3][k] = DA ? make_float4(pc.z, pc.z, pa.z, pa.z) : make_float4(pc.z, pc.z, 0.f, 0.f);
+                if (DA) sw[3][k].x = pa.z;
             }
             nk += __popc(keep);
         }
@@ -361,12 +364,11 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
 #pragma unroll 4
         for (int k = 0; k < nk; ++k) {
             const float4 s0 = sw[0][k], s1 = sw[1][k];
-            const float k1 = fmaf(s0.z, DX, s0.w), k0 = fmaf(fmaf(s0.x, DX, s0.y), DX, s1.z);
-            const f32x2 P2 = fma2(DY2, fma2(pk(s1.x, s1.y), DY2, pk(k1, k1)), pk(k0, k0));
-            float p0, p1;
-            upk(P2, p0, p1);
+            // column terms shared by the lane's two pixels, then each pixel's row terms
+            const float k1 = fmaf(s0.z, DX, s0.w), k0 = fmaf(fmaf(s0.x, DX, s0.y), DX, s1.y);
+            const float p0 = fmaf(dy0, fmaf(s1.x, dy0, k1), k0), p1 = fmaf(dy1, fmaf(s1.x, dy1, k1), k0);
             // p' >= threshold
-            const f32x2 IN2 = pk(step_ge(p0, s1.w), step_ge(p1, s1.w));
+            const f32x2 IN2 = pk(step_ge(p0, s1.z), step_ge(p1, s1.z));
             // -alpha = max(-alpha_max, -2^p') (exact negation of the clamp)
             const float na0 = fmaxf(-cam.alpha_max, -ex2_approx(p0));
             const float na1 = fmaxf(-cam.alpha_max, -ex2_approx(p1));
@@ -383,12 +385,13 @@ __device__ __forceinline__ void blend_unit(const float4 *__restrict__ rec, const
             // minus the weight: the sums below accumulate negated
             const f32x2 NWF = mul2(mul2(T2, NAIN), GO2);
             T2 = TN2;
-            const float4 c0 = sw[2][k], c1 = sw[3][k];
+            const float4 c0 = sw[2][k];
             R2 = fma2(pk(c0.x, c0.y), NWF, R2);
             G2 = fma2(pk(c0.z, c0.w), NWF, G2);
-            B2 = fma2(pk(c1.x, c1.y), NWF, B2);
+            B2 = fma2(pk(s1.w, s1.w), NWF, B2);
             if (DA) {
-                Z2 = fma2(pk(c1.z, c1.w), NWF, Z2);
+                const float z = sw[3][k].x;
+                Z2 = fma2(pk(z, z), NWF, Z2);
                 S2 = add2(S2, NWF);
             }
         }
@@ -493,7 +496,7 @@ __global__ void k_blend_heavy(const int2 *__restrict__ ranges, const int *__rest
 
 template <int TW, int TH, int RPL, bool DA>
 __global__ void __launch_bounds__(32, RPL == 1 ? (DA ? 28 : 32) : 24)
-k_blend(const float4 *__restrict__ rec, Layout L, const uint32_t *__restrict__ inst_gauss,
+k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
         const int2 *__restrict__ ranges, CamParams cam, double *__restrict__ partials, float *__restrict__ rgb,
         float *__restrict__ depth, float *__restrict__ alpha, const int *__restrict__ view_sel, int n_views,
         const int *__restrict__ overflow, BlendQueue queue)
@@ -579,7 +582,7 @@ static int blend_resident()
 }
 
 template <int TW, int TH, int RPL>
-static cudaError_t blend_t(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+static cudaError_t blend_t(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                            const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
                            const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st)
 {
@@ -598,7 +601,7 @@ static cudaError_t blend_t(const float4 *rec, const Layout &L, const uint32_t *i
                           partials, rgb, depth, alpha, view_sel, nv, overflow, queue);
 }
 
-cudaError_t launch_blend(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+cudaError_t launch_blend(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                          const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
                          const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st)
 {
@@ -725,7 +728,7 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // first walk.
 template <int TW, int TH, bool IMG>
 __global__ void __launch_bounds__(32, IMG ? 24 : 32)
-k_blend_grad(const float4 *__restrict__ rec, Layout L, const uint32_t *__restrict__ inst_gauss,
+k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
              const int2 *__restrict__ ranges, CamParams cam, const double *__restrict__ coef,
              const float *__restrict__ gimg, const float *__restrict__ gda, const float *__restrict__ cimg,
              const float *__restrict__ cdep, const float *__restrict__ calp, float *__restrict__ gout,
@@ -758,7 +761,7 @@ k_blend_grad(const float4 *__restrict__ rec, Layout L, const uint32_t *__restric
     if (*overflow) return;
     const int2 r = ranges[(int64_t)v * cam.n_tiles + tile];
     const uint32_t *list = inst_gauss + L.io_off[v];
-    const float4 *vrec = rec + L.vd_off[v] * 3;
+    const float4 *geom = rec.geom + 2 * L.vd_off[v], *col = rec.col + L.vd_off[v];
     const float limL = -0.5f * cam.cut * cam.cut * L2E;
     const float l2amin = log2f(cam.alpha_min);
     const float amax = cam.alpha_max;
@@ -781,13 +784,12 @@ k_blend_grad(const float4 *__restrict__ rec, Layout L, const uint32_t *__restric
         const float by0 = (float)rlo + 0.5f, by1 = (float)rhi + 0.5f;
         const int j = b + lane;
         bool hit = false;
-        float4 pa = make_float4(0, 0, 0, 0), pb = pa, pc = pa;
+        float4 pa = make_float4(0, 0, 0, 0), pb = pa;
         Conic cq = {0.f, 0.f, 0.f};
         uint32_t gi = 0;
         if (j < r.y) {
             gi = __ldg(list + j);
-            const float4 *p = vrec + 3 * (int64_t)gi;
-            pa = __ldg(p); pb = __ldg(p + 1); pc = __ldg(p + 2);
+            load_geom(geom, gi, pa, pb);
             cq = conic_of(pb);
             const float qbound = fminf(-limL, pa.w - l2amin + 1.5e-3f);
             if (qbound > 0.f) {
@@ -798,6 +800,7 @@ k_blend_grad(const float4 *__restrict__ rec, Layout L, const uint32_t *__restric
         const unsigned keep = __ballot_sync(0xffffffffu, hit);
         if (hit) {
             const int k = __popc(keep & lt);
+            const float4 pc = __ldg(col + gi);
             float4 t0, t1;
             block_stage(pa, pb, cq, fmaxf(limL + pa.w, l2amin), ocx, ocy, t0, t1);
             s_rec[0][k] = t0;
@@ -1007,7 +1010,7 @@ k_blend_grad(const float4 *__restrict__ rec, Layout L, const uint32_t *__restric
 }
 
 template <int TW, int TH>
-static cudaError_t blend_grad_t(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+static cudaError_t blend_grad_t(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                                 const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                                 const float *cimg, const float *cdep, const float *calp, float *gout,
                                 const int *overflow, cudaStream_t st)
@@ -1022,7 +1025,7 @@ static cudaError_t blend_grad_t(const float4 *rec, const Layout &L, const uint32
     return cudaGetLastError();
 }
 
-cudaError_t launch_blend_grad(const float4 *rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
+cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
                               const int *overflow, cudaStream_t st)
