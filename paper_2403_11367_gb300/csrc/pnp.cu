@@ -11,10 +11,10 @@
 //
 // The problem is small (thousands of pairs, a 6 x 6 system per iteration) but
 // FP64, whose rate is about two operations a clock and SM on this GPU: a warp's
-// FP64 instruction holds the SM's pipe for some 15 clocks.  So the pairs are
-// spread two warps to an SM over one cooperative launch, and what counts is the
-// number of passes over the pairs, the barriers between them and the FP64
-// instructions of a reduction:
+// FP64 instruction holds its scheduler's pipe for some 60 clocks, however many of
+// its lanes work.  So the pairs are spread over all SMs in one cooperative launch,
+// and what counts is the number of passes over the pairs, the barriers between
+// them and the length of every chain of FP64 instructions:
 //   - one pass per iteration: the trial pose is evaluated with its normal
 //     equations, so an accepted step has them already (and the final pose its
 //     cost and squared error);
@@ -23,11 +23,17 @@
 //     back from a leading block;
 //   - when the full step does not lower the cost (every solve ends there: the
 //     cost is flat to rounding at the minimum) the ten halved steps are
-//     evaluated in one pass, not one by one;
+//     evaluated in one pass, half of them by each half of the block;
 //   - a warp sums its 32 accumulators by recursive halving (31 additions, lane
-//     j left with total j) instead of 28 butterflies of five.
-// Some 7,000 pairs on the driving street: 529 us a call with one block per 256
-// pairs, five barriers and two passes an iteration, 241 us so.
+//     j left with total j) instead of 28 butterflies of five;
+//   - the system is solved by Gauss-Jordan elimination with a row per lane and the
+//     update formed with an entry per lane; reciprocals and inverse square roots
+//     take an FP32 seed and Newton's iteration to FP64, the rotation its power
+//     series for angles below half a radian.
+// Some 7,000 pairs on the driving street: 641 us a call with one block per 256
+// pairs, five barriers and two passes an iteration, 196 us so; 6,124 pairs 201 us
+// with one pass, one barrier and a thread's serial solve, 167 us so (15 us an
+// iteration, 13 of them with a single block: the chain, not the pairs).
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -36,7 +42,7 @@
 
 namespace reloc {
 
-constexpr int PNP_MAX_THREADS = 128;
+constexpr int PNP_THREADS = 128;                    // four warps, one to each of the SM's schedulers
 constexpr int PNP_HALVINGS = 10;         // backtracking: the step is halved at most this often
 // accumulators of a pass: upper H (21), g (6), Huber cost, pairs with a point,
 // squared error and count of the pairs in front of the camera
@@ -76,7 +82,36 @@ __device__ __forceinline__ double warp_sums(double (&v)[N], int lane)
     return x;
 }
 
-__device__ __forceinline__ double huber_rho(double e, double k) { return e <= k ? 0.5 * e * e : k * (e - 0.5 * k); }
+// Whether x lies where its FP32 value can seed Newton's iteration (NaN: no).
+__device__ __forceinline__ bool seeds(double x) { return x > 1e-36 && x < 1e36; }
+
+// 1 / x for x > 0: FP32 seed (relative error 2^-23), two Newton steps.
+__device__ __forceinline__ double recip(double x)
+{
+    if (!seeds(x)) return 1.0 / x;
+    double r = (double)__frcp_rn((float)x);
+    r = fma(fma(-x, r, 1.0), r, r);
+    return fma(fma(-x, r, 1.0), r, r);
+}
+
+// 1 / sqrt(x) for x > 0: FP32 seed, two Newton steps.
+__device__ __forceinline__ double rsqrt_newton(double x)
+{
+    if (!seeds(x)) return 1.0 / sqrt(x);
+    double r = (double)rsqrtf((float)x);
+    r = fma(fma(-x * r, r, 1.0), 0.5 * r, r);
+    return fma(fma(-x * r, r, 1.0), 0.5 * r, r);
+}
+
+// Huber cost of a squared residual and its weight (1, or k / e beyond k).
+__device__ __forceinline__ double huber(double e2, double k, double &w)
+{
+    w = 1.0;
+    if (e2 <= k * k) return 0.5 * e2;
+    const double ie = rsqrt_newton(e2);
+    w = k * ie;
+    return k * fma(e2, ie, -0.5 * k);
+}
 
 // One pair's residual at pose W (R row-major, then t): false behind the camera.
 __device__ __forceinline__ bool pnp_residual(const PnpArgs &a, const double *W, const double4 &X, const float4 &q,
@@ -86,7 +121,7 @@ __device__ __forceinline__ bool pnp_residual(const PnpArgs &a, const double *W, 
     py = W[3] * X.x + W[4] * X.y + W[5] * X.z + W[10];
     const double pz = W[6] * X.x + W[7] * X.y + W[8] * X.z + W[11];
     if (pz <= 1e-6) return false;
-    iz = 1.0 / pz;
+    iz = recip(pz);
     ru = a.fx * px * iz + a.cx - (double)q.z;
     rv = a.fy * py * iz + a.cy - (double)q.w;
     e2 = ru * ru + rv * rv;
@@ -102,11 +137,10 @@ __device__ __forceinline__ void pnp_add(const PnpArgs &a, const double *W, const
     acc[PA_USED] += 1.0;
     double px, py, iz, ru, rv, e2;
     if (!pnp_residual(a, W, X, q, px, py, iz, ru, rv, e2)) return;
-    const double e = sqrt(e2);
-    acc[PA_COST] += huber_rho(e, a.huber);
-    acc[PA_SQ] += e * e;
+    double w;
+    acc[PA_COST] += huber(e2, a.huber, w);
+    acc[PA_SQ] += e2;
     acc[PA_CNT] += 1.0;
-    const double w = e <= a.huber ? 1.0 : a.huber / e;
     const double u0 = a.fx * iz, v1 = a.fy * iz;
     const double nx = px * iz, ny = py * iz;            // -u2 / u0, -v2 / v1
     const double u2 = -u0 * nx, u3 = u2 * py, u4 = a.fx - u2 * px, u5 = -u0 * py;
@@ -127,101 +161,102 @@ __device__ __forceinline__ void pnp_add(const PnpArgs &a, const double *W, const
     acc[25] += wu4 * ru + wv4 * rv; acc[26] += wu5 * ru + wv5 * rv;
 }
 
-// W' = [Exp(phi) R | Exp(phi) t + rho] for delta = (rho, phi) scaled by s.
-__device__ void apply_update(const double *W, const double *delta, double s, double *Wn)
+// A = sin(th) / th and B = (1 - cos(th)) / th^2 from th^2: Exp = I + A K + B K^2,
+// K = [phi]x.  Power series in th^2 up to a quarter (the last term kept is below
+// 2^-60 there), the functions beyond.
+__device__ __forceinline__ void exp_factors(double th2, double &A, double &B)
 {
-    const double rho[3] = {s * delta[0], s * delta[1], s * delta[2]};
-    const double ph[3] = {s * delta[3], s * delta[4], s * delta[5]};
-    const double th2 = ph[0] * ph[0] + ph[1] * ph[1] + ph[2] * ph[2], th = sqrt(th2);
-    double A, B;                                   // Exp = I + A K + B K^2, K = [phi]x
-    if (th < 1e-8) {
-        A = 1.0 - th2 / 6.0;
-        B = 0.5 - th2 / 24.0;
+    if (th2 <= 0.25) {
+        // 1 / (2 k + 1)! and 1 / (2 k + 2)!, alternating, k = 8 .. 0
+        const double ca[9] = {1.0 / 355687428096000.0, -1.0 / 1307674368000.0, 1.0 / 6227020800.0, -1.0 / 39916800.0,
+                              1.0 / 362880.0, -1.0 / 5040.0, 1.0 / 120.0, -1.0 / 6.0, 1.0};
+        const double cb[9] = {1.0 / 6402373705728000.0, -1.0 / 20922789888000.0, 1.0 / 87178291200.0, -1.0 / 479001600.0,
+                              1.0 / 3628800.0, -1.0 / 40320.0, 1.0 / 720.0, -1.0 / 24.0, 0.5};
+        A = ca[0];
+        B = cb[0];
+#pragma unroll
+        for (int k = 1; k < 9; ++k) {
+            A = fma(A, th2, ca[k]);
+            B = fma(B, th2, cb[k]);
+        }
     } else {
+        const double th = sqrt(th2);
         double sn, cs;
         sincos(th, &sn, &cs);
         A = sn / th;
         B = (1.0 - cs) / th2;
     }
-    const double K[9] = {0.0, -ph[2], ph[1], ph[2], 0.0, -ph[0], -ph[1], ph[0], 0.0};
-    double E[9];
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) {
-            double k2 = 0.0;
-            for (int m = 0; m < 3; ++m) k2 += K[3 * r + m] * K[3 * m + c];
-            E[3 * r + c] = (r == c ? 1.0 : 0.0) + A * K[3 * r + c] + B * k2;
-        }
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c)
-            Wn[3 * r + c] = E[3 * r] * W[c] + E[3 * r + 1] * W[3 + c] + E[3 * r + 2] * W[6 + c];
-        Wn[9 + r] = E[3 * r] * W[9] + E[3 * r + 1] * W[10] + E[3 * r + 2] * W[11] + rho[r];
-    }
 }
 
-// Solve (H + 1e-9 tr(H)/6 I) x = -g by Cholesky; H given as 21 upper entries.
-// Unrolled into registers, with one reciprocal per pivot.
-__device__ __forceinline__ bool solve6(const double *Hu, const double *g, double (&x)[6])
+// W' = [Exp(phi) R | Exp(phi) t + rho] for delta = (rho, phi) scaled by s, an entry
+// per lane of 12 lanes (q): row q / 3 and column q % 3 of R, then t; with K^2 =
+// phi phi^T - th^2 I, row r of Exp is (1 - B th^2) e_r + A [phi]x_r + B phi_r phi^T.
+__device__ __forceinline__ double update_entry(const double *W, const double *delta, double s, int q)
 {
-    double H[6][6];
-    {
-        int k = 0;
+    const double p0 = s * delta[3], p1 = s * delta[4], p2 = s * delta[5];
+    const double th2 = p0 * p0 + p1 * p1 + p2 * p2;
+    double A, B;
+    exp_factors(th2, A, B);
+    const int r = q < 9 ? q / 3 : q - 9;
+    const double pr = r == 0 ? p0 : r == 1 ? p1 : p2, d = fma(-B, th2, 1.0), bp = B * pr;
+    const double k0 = r == 0 ? 0.0 : r == 1 ? p2 : -p1, k1 = r == 0 ? -p2 : r == 1 ? 0.0 : p0;
+    const double k2 = r == 0 ? p1 : r == 1 ? -p0 : 0.0;
+    const double e0 = fma(bp, p0, fma(A, k0, r == 0 ? d : 0.0)), e1 = fma(bp, p1, fma(A, k1, r == 1 ? d : 0.0));
+    const double e2 = fma(bp, p2, fma(A, k2, r == 2 ? d : 0.0));
+    const int o = q < 9 ? q % 3 : 9, step = q < 9 ? 3 : 1;
+    return fma(e0, W[o], fma(e1, W[o + step], fma(e2, W[o + 2 * step], q < 9 ? 0.0 : s * delta[r])));
+}
+
+// Solve (H + 1e-9 tr(H)/6 I) x = -g, H given as 21 upper entries, by a warp: lane r
+// < 6 holds row r of [H | -g] and ends with x_r (Gauss-Jordan; H is symmetric
+// positive definite, so its pivots need no exchange and are all positive: false
+// otherwise).
+__device__ __forceinline__ bool solve6(const double *Hu, const double *g, int lane, double &x)
+{
+    const int r = lane < 6 ? lane : 5;
+    double m[7];
 #pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-            for (int c = r; c < 6; ++c) H[c][r] = Hu[k++];
+    for (int c = 0; c < 6; ++c) {
+        const int i = r < c ? r : c, j = r < c ? c : r;
+        m[c] = Hu[6 * i - i * (i - 1) / 2 + (j - i)];
     }
-    const double ridge = 1e-9 * (H[0][0] + H[1][1] + H[2][2] + H[3][3] + H[4][4] + H[5][5]) / 6.0;
-    double il[6];
+    m[6] = -g[r];
+    const double ridge = 1e-9 / 6.0 * (Hu[0] + Hu[6] + Hu[11] + Hu[15] + Hu[18] + Hu[20]);
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+        if (r == c) m[c] += ridge;
     bool ok = true;
+    x = 0.0;
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-        double d = H[j][j] + ridge;
+        double row[7];
 #pragma unroll
-        for (int m = 0; m < 6; ++m)
-            if (m < j) d -= H[j][m] * H[j][m];
-        ok = ok && d > 0.0;
-        il[j] = 1.0 / sqrt(d);
+        for (int c = 0; c < 7; ++c)
+            if (c >= j) row[c] = __shfl_sync(0xffffffffu, m[c], j);
+        ok = ok && row[j] > 0.0 && row[j] < INFINITY;
+        const double inv = recip(row[j]);
+        const double f = r == j ? 0.0 : m[j] * inv;
+        if (r == j) x = inv;
 #pragma unroll
-        for (int i = 0; i < 6; ++i)
-            if (i > j) {
-                double s = H[i][j];
-#pragma unroll
-                for (int m = 0; m < 6; ++m)
-                    if (m < j) s -= H[i][m] * H[j][m];
-                H[i][j] = s * il[j];
-            }
+        for (int c = 0; c < 7; ++c)
+            if (c > j) m[c] = fma(-f, row[c], m[c]);
     }
-    double y[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        double s = -g[i];
-#pragma unroll
-        for (int m = 0; m < 6; ++m)
-            if (m < i) s -= H[i][m] * y[m];
-        y[i] = s * il[i];
-    }
-#pragma unroll
-    for (int i = 5; i >= 0; --i) {
-        double s = y[i];
-#pragma unroll
-        for (int m = 0; m < 6; ++m)
-            if (m > i) s -= H[m][i] * x[m];
-        x[i] = s * il[i];
-    }
+    x *= m[6];
     return ok;
 }
 
-__global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
+__global__ void __launch_bounds__(PNP_THREADS) k_refine_pnp(PnpArgs a)
 {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
-    constexpr int MAX_WARPS = PNP_MAX_THREADS / 32;
-    __shared__ double s_red[MAX_WARPS][PNP_ACC];
+    constexpr int NW = PNP_THREADS / 32;
+    __shared__ double s_red[NW][PNP_ACC];
     __shared__ double s_tot[PNP_ACC];                    // the last pass's totals
     __shared__ double s_pose[12], s_trial[PNP_HALVINGS][12], s_delta[6];
     __shared__ int s_ok;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // pairs go round the blocks, so that a block's first warps hold its share
+    const int first = blockIdx.x + gridDim.x * threadIdx.x, stride = gridDim.x * PNP_THREADS;
     int turn = 0;                                        // which half of the partial sums a pass writes
 
     // back-projection of every pair with the rendered depth
@@ -250,7 +285,7 @@ __global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
                 }
             }
         }
-        a.X[i] = X;                                      // read back by this thread only
+        a.X[i] = X;                                      // read back by this block only
     }
 
     // The grid's totals of this lane's warp sum v (lane j: entry j) into s_tot,
@@ -261,28 +296,24 @@ __global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
         double *part = a.part + (int64_t)turn * gridDim.x * PNP_ACC;
         turn ^= 1;                                       // a block may still read these while the next pass writes
         if (warp == 0) {
-            double t = s_red[0][lane];
-            for (int w = 1; w < n_warps; ++w) t += s_red[w][lane];
+            const double t = (s_red[0][lane] + s_red[1][lane]) + (s_red[2][lane] + s_red[3][lane]);
             __stcg(part + (int64_t)blockIdx.x * PNP_ACC + lane, t);
         }
         grid.sync();
-        double t = 0.0;
-        int b = warp;
-        for (; b + 7 * n_warps < (int)gridDim.x; b += 8 * n_warps) {
+        // four running sums of the warp's quarter of the blocks, all loads of a round in flight
+        double t4[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = warp; b < (int)gridDim.x; b += 8 * NW) {
             double x[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = __ldcg(part + (int64_t)(b + k * n_warps) * PNP_ACC + lane);
+            for (int k = 0; k < 8; ++k)
+                x[k] = b + k * NW < (int)gridDim.x ? __ldcg(part + (int64_t)(b + k * NW) * PNP_ACC + lane) : 0.0;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) t += x[k];
+            for (int k = 0; k < 8; ++k) t4[k & 3] += x[k];
         }
-        for (; b < (int)gridDim.x; b += n_warps) t += __ldcg(part + (int64_t)b * PNP_ACC + lane);
-        s_red[warp][lane] = t;
+        s_red[warp][lane] = (t4[0] + t4[1]) + (t4[2] + t4[3]);
         __syncthreads();
-        if (warp == 0) {
-            t = s_red[0][lane];
-            for (int w = 1; w < n_warps; ++w) t += s_red[w][lane];
-            s_tot[lane] = t;
-        }
+        static_assert(NW == 4, "sums of four warps");
+        if (warp == 0) s_tot[lane] = (s_red[0][lane] + s_red[1][lane]) + (s_red[2][lane] + s_red[3][lane]);
         __syncthreads();
     };
     // normal equations, cost and squared error at pose W (shared memory)
@@ -290,8 +321,13 @@ __global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
         double acc[PNP_ACC];
 #pragma unroll
         for (int j = 0; j < PNP_ACC; ++j) acc[j] = 0.0;
-        for (int i = first; i < a.n; i += stride) pnp_add(a, W, a.X[i], a.pairs[i], acc);
-        grid_totals(warp_sums<PNP_ACC>(acc, lane));
+        // a warp without pairs adds nothing (its FP64 instructions would take the same time)
+        double v = 0.0;
+        if (__any_sync(0xffffffffu, first < a.n)) {
+            for (int i = first; i < a.n; i += stride) pnp_add(a, W, a.X[i], a.pairs[i], acc);
+            v = warp_sums<PNP_ACC>(acc, lane);
+        }
+        grid_totals(v);
     };
 
     if (threadIdx.x < 12) s_pose[threadIdx.x] = a.W0[threadIdx.x];
@@ -302,11 +338,13 @@ __global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
     int it = 0;
     if (n_used >= 3.0) {
         for (; it < a.max_iters; ++it) {
-            if (threadIdx.x == 0) {
-                double d[6];
-                s_ok = solve6(s_tot, s_tot + PA_G, d);
-                for (int j = 0; j < 6; ++j) s_delta[j] = d[j];
-                apply_update(s_pose, d, 1.0, s_trial[0]);
+            if (warp == 0) {
+                double x;
+                const bool ok = solve6(s_tot, s_tot + PA_G, lane, x);
+                if (lane < 6) s_delta[lane] = x;
+                if (lane == 0) s_ok = ok;
+                __syncwarp();
+                if (lane < 12) s_trial[0][lane] = update_entry(s_pose, s_delta, 1.0, lane);
             }
             __syncthreads();
             if (!s_ok) break;
@@ -315,24 +353,32 @@ __global__ void __launch_bounds__(PNP_MAX_THREADS) k_refine_pnp(PnpArgs a)
             int take = 0;
             if (!(s_tot[PA_COST] < cost)) {
                 // the halved steps, all in one pass
-                if (threadIdx.x < PNP_HALVINGS)
-                    apply_update(s_pose, s_delta, 1.0 / (double)(2 << threadIdx.x), s_trial[threadIdx.x]);
+                for (int k = threadIdx.x; k < 12 * PNP_HALVINGS; k += PNP_THREADS) {
+                    const int h = k / 12;
+                    s_trial[h][k - 12 * h] = update_entry(s_pose, s_delta, 1.0 / (double)(2 << h), k - 12 * h);
+                }
                 __syncthreads();
-                double c[16];
+                // threads 0..63 evaluate the first five, threads 64..127 the others, on the same pairs
+                constexpr int HALF = PNP_HALVINGS / 2;
+                const int h0 = threadIdx.x < PNP_THREADS / 2 ? 0 : HALF;
+                double c[8];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) c[k] = 0.0;
-                for (int i = first; i < a.n; i += stride) {
+                for (int k = 0; k < 8; ++k) c[k] = 0.0;
+                for (int i = blockIdx.x + gridDim.x * (threadIdx.x & (PNP_THREADS / 2 - 1)); i < a.n; i += stride / 2) {
                     const double4 X = a.X[i];
                     const float4 q = a.pairs[i];
                     if (X.w == 0.0) continue;
 #pragma unroll
-                    for (int k = 0; k < PNP_HALVINGS; ++k) {
-                        double px, py, iz, ru, rv, e2;
-                        if (pnp_residual(a, s_trial[k], X, q, px, py, iz, ru, rv, e2)) c[k] += huber_rho(sqrt(e2), a.huber);
+                    for (int k = 0; k < HALF; ++k) {
+                        double px, py, iz, ru, rv, e2, w;
+                        if (pnp_residual(a, s_trial[h0 + k], X, q, px, py, iz, ru, rv, e2)) c[k] += huber(e2, a.huber, w);
                     }
                 }
-                grid_totals(warp_sums<16>(c, lane));     // lanes 2 k and 2 k + 1: step k
-                for (take = 0; take < PNP_HALVINGS && !(s_tot[2 * take] < cost); ++take) {}
+                // lanes 4 k .. 4 k + 3 of a warp hold its sum k; entry 8 half + k of the pass
+                const double cs = __shfl_sync(0xffffffffu, warp_sums<8>(c, lane), (4 * lane) & 31);
+                grid_totals(lane >= 8 && lane < 16 ? (h0 ? cs : 0.0) : lane < 8 ? (h0 ? 0.0 : cs) : 0.0);
+                auto cost_of = [&](int h) { return s_tot[h < HALF ? h : 8 + h - HALF]; };
+                for (take = 0; take < PNP_HALVINGS && !(cost_of(take) < cost); ++take) {}
                 if (take == PNP_HALVINGS) break;         // no step lowers the cost: converged
                 step = 1.0 / (double)(2 << take);
                 __syncthreads();                         // s_tot is read before the pass below writes it
@@ -387,17 +433,16 @@ cudaError_t launch_refine_pnp(const double *pose_render, const double *pose_init
     a.pairs = reinterpret_cast<const float4 *>(pairs);
     a.X = reinterpret_cast<double4 *>(X_scratch);
     a.out = out;
-    // at most one block per SM (all resident: the launch is cooperative), of two
-    // warps while that covers the pairs one each, of four beyond
+    // at most one block per SM (all resident: the launch is cooperative), of a warp's
+    // worth of pairs or more
     int dev = 0, n_sm = 1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int nt = n <= 64 * n_sm ? 64 : PNP_MAX_THREADS;
-    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(n_sm, ceil_div(n, nt)));
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(n_sm, ceil_div(n, 32)));
     a.part = X_scratch + 4 * (int64_t)n;
     void *args[] = {&a};
-    e = cudaLaunchCooperativeKernel((const void *)k_refine_pnp, dim3(nb), dim3(nt), args, 0, st);
+    e = cudaLaunchCooperativeKernel((const void *)k_refine_pnp, dim3(nb), dim3(PNP_THREADS), args, 0, st);
     return e;
 }
 
