@@ -539,6 +539,7 @@ struct CallOut {
     bool argmax = false;                                        // per query argmax
     float *brgb = nullptr, *bdepth = nullptr, *balpha = nullptr; // winners [Q][...]
     double *grad = nullptr;                                     // NCC pose gradients [V][6] (device)
+    bool keep_rgb = false;                                      // their forward's render is kept (set by run_batch)
     const float *target = nullptr;  // training: target images [V][3][H][W] (device)
     double l1_scale = 0.0;          // training: weight of sum |C - I| in the loss
     double ssim_scale = 0.0;        // training: weight of sum (1 - SSIM) in the loss
@@ -692,6 +693,9 @@ static void stage_tables(SubBatch &sb, char *host, char *dev)
     sb.d_views = (const ViewParams *)put(sb.views.data(), sizeof(ViewParams) * (size_t)nv);
 }
 
+// A sub-batch's renders kept for its pose gradients, up to a bound on the memory.
+constexpr int64_t GRAD_IMAGE_MAX = (int64_t)1 << 30;
+
 static void stage_mark(reloc_ctx *ctx, int sbi, int s, cudaStream_t st, bool capturing)
 {
     if (ctx->prof && !capturing) cudaEventRecord(ctx->ev[(size_t)sbi * (RELOC_STAGE_COUNT + 1) + s], st);
@@ -779,7 +783,8 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     }
     const uint32_t *fgauss = ctx->inst.as<uint32_t>();
     stage_mark(ctx, sbi, RELOC_STAGE_BLEND, st, capturing);
-    float *rgb_out = o.target ? ctx->trgb.as<float>() : (o.rgb ? o.rgb + (int64_t)sb.v0 * 3 * HW : nullptr);
+    // the pose gradients' forward writes its render too, so that the backward pass need not composite again
+    float *rgb_out = o.target || o.keep_rgb ? ctx->trgb.as<float>() : (o.rgb ? o.rgb + (int64_t)sb.v0 * 3 * HW : nullptr);
     const bool rp = o.target && o.rel;
     float *dep_out = rp ? ctx->tdep.as<float>() : (o.depth ? o.depth + (int64_t)sb.v0 * HW : nullptr);
     float *alp_out = rp ? ctx->talp.as<float>() : (o.alpha ? o.alpha + (int64_t)sb.v0 * HW : nullptr);
@@ -837,7 +842,8 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         if (o.grad) {
             CK(cudaMemsetAsync(ctx->gbuf.p, 0, 20 * (size_t)sb.VS, st));
             CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
-                                 ctx->gcoef.as<double>(), nullptr, nullptr, nullptr, nullptr, nullptr,
+                                 ctx->gcoef.as<double>(), nullptr, nullptr,
+                                 o.keep_rgb ? ctx->trgb.as<float>() : nullptr, nullptr, nullptr,
                                  ctx->gbuf.as<float>(), d_overflow, st));
             CK(launch_pose_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
                                  ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.p, ctx->precision, ctx->n,
@@ -956,6 +962,8 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             for (auto &sb : sbs) pb = std::max<int64_t>(pb, (int64_t)sb.pblk * (sb.v1 - sb.v0));
             CKS(ctx->gbuf.ensure(20 * (size_t)VS));
             CKS(ctx->gcoef.ensure(32 * (size_t)V));
+            o.keep_rgb = 12 * V * HW <= GRAD_IMAGE_MAX;
+            if (o.keep_rgb) CKS(ctx->trgb.ensure(12 * (size_t)V * HW));
             CKS(ctx->gpart.ensure(48 * (size_t)pb));
         }
         CKS(ctx->qpart.ensure(16 * QS_BLOCKS * (size_t)Qm));
