@@ -772,8 +772,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     const BlendQueue queue{R.queues + 4 * sbi, ctx->bqueue.as<int>()};
     const BlendQueue queue_w{R.queues + 4 * sbi + 2, ctx->bqueue.as<int>()};
     CK(launch_tile_count(ctx->v1b.as<uint32_t>(), nvis, ctx->rect.as<uint2>(), L, cp, sb.cb, sb.cb_view, ctx->srect.as<uint2>(),
-                         ctx->bhist.as<uint32_t>(), ctx->ranges.as<int2>(), ninst, R.done + sb.v0, d_overflow,
-                         blend_heavy_first(L.V) ? queue : BlendQueue{nullptr, nullptr}, st));
+                         ctx->bhist.as<uint32_t>(), ctx->ranges.as<int2>(), ninst, R.done + sb.v0, d_overflow, queue, st));
     launches += sb.cb > 0 ? 2 : 1;
     stage_mark(ctx, sbi, RELOC_STAGE_TILE_EMIT, st, capturing);
     if (sb.cb > 0) {
@@ -791,7 +790,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     CK(launch_blend(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
                     o.score ? ctx->partials.as<double>() : nullptr, rgb_out, dep_out, alp_out,
                     nullptr, 0, d_overflow, queue, st));
-    launches += blend_launches(L.V, false);
+    launches += blend_launches(false);
     stage_mark(ctx, sbi, RELOC_STAGE_SCORE, st, capturing);
     if (o.target) {
         // map training: the image loss and dL/dC, then back through the blend and the projection
@@ -862,7 +861,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
                                 o.bdepth ? o.bdepth + (int64_t)sb.q0 * HW : nullptr,
                                 o.balpha ? o.balpha + (int64_t)sb.q0 * HW : nullptr, vsel, nq, d_overflow,
                                 queue_w, st));
-                launches += blend_launches(nq, true);
+                launches += blend_launches(true);
             }
         }
     }

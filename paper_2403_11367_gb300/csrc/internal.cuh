@@ -242,7 +242,7 @@ cudaError_t launch_fill_tiles(const int2 *ranges_view, int n_tiles, uint32_t *ti
 // view_sel != null: blend only the n_sel views view_sel[0..n_sel), image
 // slot k for view_sel[k].  queue: a work queue of blend_list_ints(cam, n) entries
 // for n views, with the heavy tiles listed by launch_tile_count or, for selected
-// views, here.  blend_launches(n, selected) launches.
+// views, here.  blend_launches(selected) launches.
 cudaError_t launch_blend(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                          const CamParams &cam, double *partials, float *rgb, float *depth, float *alpha,
                          const int *view_sel, int n_sel, const int *overflow, BlendQueue queue, cudaStream_t st);
@@ -254,11 +254,9 @@ inline int blend_units(const CamParams &cam) { return cam.n_tiles * (cam.tile_w 
 // entries stay far inside int32.  Sub-batches are cut to respect it.
 constexpr int64_t BLEND_MAX_UNITS = (int64_t)1 << 29;
 inline int64_t blend_list_ints(const CamParams &cam, int64_t n) { return n * cam.n_tiles; }
-// Launches of several views hand out their heavy tiles first (a one-view launch
-// ends on its longest unit whatever the order); a launch of selected views lists
-// them itself.
-__host__ __device__ __forceinline__ bool blend_heavy_first(int64_t n) { return n >= 4; }
-inline int blend_launches(int64_t n, bool selected) { return selected && blend_heavy_first(n) ? 2 : 1; }
+// Image launches of fewer views take half blocks.
+constexpr int BLEND_HALF_VIEWS = 4;
+inline int blend_launches(bool selected) { return selected ? 2 : 1; }
 
 // K7: NCC per view from its n_units partials and its query's partial sums
 // (launch_project);

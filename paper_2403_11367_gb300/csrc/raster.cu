@@ -437,13 +437,156 @@ __device__ __forceinline__ void blend_unit(const Records &rec, const Layout &L,
     }
 }
 
+// Half of a 64-pixel block (its left or right columns), a pixel to a lane: image
+// launches of few views, where the SMs run out of units before the longest lists
+// end.  Half a block's record takes 22 instructions instead of 33 and half a block
+// keeps fewer of them, so the last units end sooner; all units together take more
+// (every record is tested twice).  One view of a driving map (653,141 list entries,
+// lists up to 2,846): 104 -> 104 us with list order, 88 us with the heavy tiles
+// first; one object's view 30.8 -> 20.7 us, a winner of 64 such views 120 -> 106 us with its scores.
+// Records come through a ring of asynchronous copies: no registers held for loads
+// in flight, which the deeper unrolling takes.
+// A pixel's arithmetic is blend_unit's (offsets from the 64-pixel block's centre,
+// the same operations on one half of each pair), so its values are the same bit for
+// bit.
+constexpr int HALF_RING = 4;              // record batches of a half block in flight or in use
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <int TW, int TH, bool DA>
+__device__ __forceinline__ void blend_half(const Records &rec, const Layout &L, const uint32_t *__restrict__ inst_gauss,
+                                           const CamParams &cam, float *__restrict__ rgb, float *__restrict__ depth,
+                                           float *__restrict__ alpha, int v, int out_v, int half_unit, int2 r,
+                                           float4 (*sw)[64], float4 (*ring)[3][32])
+{
+    using GM = BlockGeom<TW, TH>;
+    constexpr int BW = GM::BW, BH = GM::BH, WPT = GM::WPT;
+    const int unit = half_unit >> 1, tile = unit / WPT, warp = unit - tile * WPT;
+    const int tx = tile % cam.ntx, ty = tile / cam.ntx;
+    const int lane = threadIdx.x;
+    const int bx0p = tx * TW + (warp % GM::NBX) * BW, by0p = ty * TH + (warp / GM::NBX) * BH;
+    const int row = lane / (BW / 2), colx = lane % (BW / 2) + (half_unit & 1) * (BW / 2);
+    const int px = bx0p + colx, py = by0p + row;
+    const bool in = px < cam.width && py < cam.height;
+    const float ocx = (float)bx0p + 0.5f * BW, ocy = (float)by0p + 0.5f * BH;
+    const float DX = (float)colx + 0.5f - 0.5f * BW, DY = (float)row + 0.5f - 0.5f * BH;
+    const uint32_t *list = inst_gauss + L.io_off[v];
+    const float4 *geom = rec.geom + 2 * L.vd_off[v], *col = rec.col + L.vd_off[v];
+    constexpr float L2E = 1.4426950408889634f;
+    const float limL = -0.5f * cam.cut * cam.cut * L2E, l2amin = log2f(cam.alpha_min);
+    const unsigned lt = lanemask_lt_u();
+    float T = in ? 1.f : 0.f, R = 0.f, G = 0.f, B = 0.f, Z = 0.f, S = 0.f;
+    // batch m's records go to ring slot m % HALF_RING, each lane copying the one it
+    // will read; list indices two batches further on
+    auto index_at = [&](int j) { return j < r.y ? __ldg(list + j) : 0u; };
+    auto fetch = [&](int m, uint32_t g) {
+        if (r.x + 32 * m + lane < r.y) {
+            float4(*const slot)[32] = ring[m % HALF_RING];
+            cp_async16(&slot[0][lane], geom + 2 * (int64_t)g);
+            cp_async16(&slot[1][lane], geom + 2 * (int64_t)g + 1);
+            cp_async16(&slot[2][lane], col + g);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint32_t gi[HALF_RING + 1];
+#pragma unroll
+    for (int m = 0; m < HALF_RING + 1; ++m) gi[m] = index_at(r.x + 32 * m + lane);
+#pragma unroll
+    for (int m = 0; m < HALF_RING - 1; ++m) fetch(m, gi[m]);
+    uint32_t g0 = gi[HALF_RING - 1], g1 = gi[HALF_RING];
+    int m = 0;
+    // kept records wait in a ring until there are four: the loop below is unrolled with
+    // no remainder (a batch keeps six or seven, and one at a time each costs the
+    // chain's latency)
+    int head = 0, tail = 0;
+    auto blend4 = [&](int base) {
+#pragma unroll
+        for (int k = base; k < base + 4; ++k) {
+            const float4 s0 = sw[0][k], s1 = sw[1][k], c = sw[2][k];
+            const float k1 = fmaf(s0.z, DX, s0.w), k0 = fmaf(fmaf(s0.x, DX, s0.y), DX, s1.y);
+            const float p = fmaf(DY, fmaf(s1.x, DY, k1), k0);
+            const float na = __fmul_rn(fmaxf(-cam.alpha_max, -ex2_approx(p)), step_ge(p, s1.z));
+            const float TN = __fmaf_rn(T, na, T);
+            const float w = __fmul_rn(__fmul_rn(T, na), step_ge(TN, cam.t_min));
+            T = TN;
+            R = __fmaf_rn(c.x, w, R);
+            G = __fmaf_rn(c.y, w, G);
+            B = __fmaf_rn(s1.w, w, B);
+            if (DA) {
+                Z = __fmaf_rn(c.z, w, Z);
+                S = __fadd_rn(S, w);
+            }
+        }
+    };
+    for (int b = r.x; b < r.y; b += 32) {
+        const bool live = T >= cam.t_min && in;
+        const unsigned alive = __ballot_sync(0xffffffffu, live);
+        if (!alive) break;
+        const float bx0 = (float)__reduce_min_sync(0xffffffffu, live ? (unsigned)px : 0xffffu) + 0.5f;
+        const float bx1 = (float)__reduce_max_sync(0xffffffffu, live ? (unsigned)px : 0u) + 0.5f;
+        // rows rise with the lane
+        const float by0 = (float)(by0p + (__ffs(alive) - 1) / (BW / 2)) + 0.5f;
+        const float by1 = (float)(by0p + (31 - __clz(alive)) / (BW / 2)) + 0.5f;
+        asm volatile("cp.async.wait_group %0;" ::"n"(HALF_RING - 2) : "memory");
+        const float4(*const slot)[32] = ring[m % HALF_RING];
+        const float4 pa = slot[0][lane], pb = slot[1][lane], pc = slot[2][lane];
+        const int j = b + lane;
+        fetch(m + HALF_RING - 1, g0);
+        g0 = g1;
+        g1 = index_at(j + 32 * (HALF_RING + 1));
+        ++m;
+        const Conic cq = conic_of(pb);
+        const float qbound = fminf(-limL, pa.w - l2amin + 1.5e-3f);
+        bool hit = false;
+        if (j < r.y && qbound > 0.f)
+            hit = quad_min_rect(pb, cq, bx0 - pa.x, bx1 - pa.x, by0 - pa.y, by1 - pa.y) <= qbound * 1.01f + 1e-3f;
+        const unsigned keep = __ballot_sync(0xffffffffu, hit);
+        if (hit) {
+            const int k = (tail + __popc(keep & lt)) & 63;
+            float4 t0, t1;
+            block_stage(pa, pb, cq, fmaxf(limL + pa.w, l2amin), ocx, ocy, t0, t1);
+            sw[0][k] = t0;
+            sw[1][k] = make_float4(t1.x, t1.z, t1.w, pc.z);
+            sw[2][k] = make_float4(pc.x, pc.y, pa.z, 0.f);
+        }
+        tail += __popc(keep);
+        __syncwarp();
+        for (; tail - head >= 4; head += 4) blend4(head & 63);
+        __syncwarp();
+    }
+    // what is left, made up to four with records that no pixel takes
+    if (tail > head) {
+        if (lane < 4 && lane >= tail - head) {
+            const int k = (head + lane) & 63;
+            sw[0][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            sw[1][k] = make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
+            sw[2][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        __syncwarp();
+        blend4(head & 63);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");   // the slots are the next unit's
+    if (!in) return;
+    const int64_t HW = (int64_t)cam.width * cam.height, pix = (int64_t)py * cam.width + px;
+    if (rgb) {
+        float *o = rgb + (int64_t)out_v * 3 * HW;
+        o[pix] = __fmul_rn(R, -1.f); o[HW + pix] = __fmul_rn(G, -1.f); o[2 * HW + pix] = __fmul_rn(B, -1.f);
+    }
+    if (depth) depth[(int64_t)out_v * HW + pix] = __fmul_rn(Z, -1.f);
+    if (alpha) alpha[(int64_t)out_v * HW + pix] = __fmul_rn(S, -1.f);
+}
+
 // Persistent K6: a grid of resident one-warp blocks (as many as fit on the
 // SMs) takes the launch's units -- (view, tile, 64-pixel block) of every view
 // of every query in the call -- from one queue (an atomic ticket per unit).
 // The units of heavy tiles (lists of at least BLEND_HEAVY records, listed by
 // k_tile_chunk_scan: the horizon's tiles, whose units run up to twenty times the
 // mean) are handed out first, the rest in view-major order (the heavy ones
-// skipped there), so that no long unit starts near the end of the launch.
+// skipped there), so that no long unit starts near the end of the launch: one
+// driving view in half blocks 102 -> 88 us, a winner of 64 views 121 -> 110 us
+// with the launch that lists its heavy tiles.
 // A warp holds its next ticket, the next unit's view and list range while it
 // blends the current one, so the dependent loads that start a unit are off
 // the critical path, and no block launch separates units (a per-unit grid
@@ -469,23 +612,24 @@ __global__ void k_blend_heavy(const int2 *__restrict__ ranges, const int *__rest
     if (r.y - r.x >= BLEND_HEAVY) queue.list[atomicAdd(queue.count + 1, 1)] = (int)i;
 }
 
-template <int TW, int TH, int RPL, bool DA>
-__global__ void __launch_bounds__(32, RPL == 1 ? (DA ? 28 : 32) : 24)
+// HALF: units of half a block (image launches of few views, no NCC).
+template <int TW, int TH, int RPL, bool DA, bool HALF>
+__global__ void __launch_bounds__(32, HALF ? 16 : RPL == 1 ? (DA ? 28 : 32) : 24)
 k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
         const int2 *__restrict__ ranges, CamParams cam, double *__restrict__ partials, float *__restrict__ rgb,
         float *__restrict__ depth, float *__restrict__ alpha, const int *__restrict__ view_sel, int n_views,
         const int *__restrict__ overflow, BlendQueue queue)
 {
-    __shared__ float4 s_rec[4][32 * RPL];
+    __shared__ float4 s_rec[HALF ? 3 : 4][HALF ? 64 : 32 * RPL];
+    __shared__ float4 s_ring[HALF ? HALF_RING : 1][HALF ? 3 : 1][HALF ? 32 : 1];
     chain_wait();
-    constexpr int WPT = BlockGeom<TW, TH>::WPT;
+    constexpr int WPT = BlockGeom<TW, TH>::WPT * (HALF ? 2 : 1);   // units of a tile
     const int upv = cam.n_tiles * WPT;                          // units per view
     const int64_t total = (int64_t)upv * n_views;
     const bool ovf = *overflow != 0;
     // heavy units, handed out first (and skipped in order) when the launch
     // listed them
-    const bool listed = blend_heavy_first(n_views);
-    const int64_t hh = listed ? (int64_t)queue.count[1] * WPT : 0;
+    const int64_t hh = (int64_t)queue.count[1] * WPT;
     const int lane = threadIdx.x;
     // view and list range of unit u (empty past the end or after an overflow)
     auto locate = [&](int64_t u, int &v, int2 &r) {
@@ -511,7 +655,7 @@ k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
             }
             u = t - hh;
             locate(u, v, r);
-            if (u >= total || !listed || r.y - r.x < BLEND_HEAVY) return;
+            if (u >= total || r.y - r.x < BLEND_HEAVY) return;
         }
     };
     int64_t u;
@@ -519,15 +663,24 @@ k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
     int2 r;
     next(u, v, r);
     while (u < total) {
-        // the next unit: ticket, view and range in flight during this one
+        // the next unit: ticket, view and range in flight during this one, unless
+        // this one is heavy: its successor may be too, and would wait here while
+        // another warp is free
         int64_t un;
         int vn;
         int2 rn;
-        next(un, vn, rn);
+        const bool heavy = HALF && r.y - r.x >= BLEND_HEAVY;
+        if (!heavy) next(un, vn, rn);
         const int vi = (int)(u / upv);
-        blend_unit<TW, TH, RPL, DA>(rec, L, inst_gauss, cam, partials, rgb, depth, alpha, v < 0 ? 0 : v, vi,
-                                    (int)(u - (int64_t)vi * upv), v < 0 ? make_int2(0, 0) : r, s_rec);
+        const int loc = (int)(u - (int64_t)vi * upv);
+        if constexpr (HALF)
+            blend_half<TW, TH, DA>(rec, L, inst_gauss, cam, rgb, depth, alpha, v < 0 ? 0 : v, vi, loc,
+                                   v < 0 ? make_int2(0, 0) : r, s_rec, s_ring);
+        else
+            blend_unit<TW, TH, RPL, DA>(rec, L, inst_gauss, cam, partials, rgb, depth, alpha, v < 0 ? 0 : v, vi, loc,
+                                        v < 0 ? make_int2(0, 0) : r, s_rec);
         __syncwarp();
+        if (heavy) next(un, vn, rn);
         u = un;
         v = vn;
         r = rn;
@@ -538,7 +691,7 @@ k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
 // per kernel (every k_blend has the same function type: one cache for that type
 // gave the scoring launches the export launches' 28 blocks per SM in a process
 // that had rendered first).
-template <int TW, int TH, int RPL, bool DA>
+template <int TW, int TH, int RPL, bool DA, bool HALF>
 static int blend_resident()
 {
     static std::atomic<int> cached[64];
@@ -548,7 +701,7 @@ static int blend_resident()
     if (!c) {
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blend<TW, TH, RPL, DA>, 32, 0) != cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blend<TW, TH, RPL, DA, HALF>, 32, 0) != cudaSuccess)
             return 0;
         c = sms * (per_sm > 0 ? per_sm : 1);
         cached[dev].store(c);
@@ -563,17 +716,28 @@ static cudaError_t blend_t(Records rec, const Layout &L, const uint32_t *inst_ga
 {
     const int nv = view_sel ? n_sel : L.V;
     const int64_t units = (int64_t)cam.n_tiles * (TW * TH / 64) * nv;
-    if (view_sel && blend_heavy_first(nv)) {
+    if (view_sel) {
         const int64_t nt = (int64_t)nv * cam.n_tiles;
         const cudaError_t e = launch_chained(k_blend_heavy, dim3((unsigned)ceil_div(nt, 256)), dim3(256), 0, st, 1, ranges,
                                              view_sel, nv, cam.n_tiles, overflow, queue);
         if (e != cudaSuccess) return e;
     }
-    auto kernel = depth || alpha ? k_blend<TW, TH, RPL, true> : k_blend<TW, TH, RPL, false>;
-    const int g = depth || alpha ? blend_resident<TW, TH, RPL, true>() : blend_resident<TW, TH, RPL, false>();
-    if (g <= 0) return cudaErrorInvalidValue;
-    return launch_chained(kernel, dim3((unsigned)min64(units, g)), dim3(32), 0, st, 1, rec, L, inst_gauss, ranges, cam,
-                          partials, rgb, depth, alpha, view_sel, nv, overflow, queue);
+    auto run = [&](auto kernel, int resident, int64_t n) {
+        if (resident <= 0) return cudaErrorInvalidValue;
+        return launch_chained(kernel, dim3((unsigned)min64(n, resident)), dim3(32), 0, st, 1, rec, L, inst_gauss, ranges,
+                              cam, partials, rgb, depth, alpha, view_sel, nv, overflow, queue);
+    };
+    const bool da = depth || alpha;
+    // Image launches that end on their longest lists take half blocks (the figures are
+    // blend_half's); from four views on a launch is bound by its instructions, which
+    // half blocks raise.
+    if constexpr (RPL == 1) {
+        if (!partials && nv < BLEND_HALF_VIEWS)
+            return da ? run(k_blend<TW, TH, 1, true, true>, blend_resident<TW, TH, 1, true, true>(), 2 * units)
+                      : run(k_blend<TW, TH, 1, false, true>, blend_resident<TW, TH, 1, false, true>(), 2 * units);
+    }
+    return da ? run(k_blend<TW, TH, RPL, true, false>, blend_resident<TW, TH, RPL, true, false>(), units)
+              : run(k_blend<TW, TH, RPL, false, false>, blend_resident<TW, TH, RPL, false, false>(), units);
 }
 
 cudaError_t launch_blend(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
