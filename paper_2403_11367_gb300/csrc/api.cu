@@ -794,29 +794,29 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     stage_mark(ctx, sbi, RELOC_STAGE_SCORE, st, capturing);
     if (o.target) {
         // map training: the image loss and dL/dC, then back through the blend and the projection
-        CK(launch_photo_l1(ctx->trgb.as<float>(), o.target + (int64_t)sb.v0 * 3 * HW, (int64_t)L.V * 3 * HW,
-                           o.l1_scale, ctx->tgimg.as<float>(), false, ctx->tloss.as<double>(), st));
-        if (o.ssim_scale > 0) {
-            CK(launch_ssim(ctx->trgb.as<float>(), o.target + (int64_t)sb.v0 * 3 * HW, 3 * L.V, cp.height, cp.width,
-                           o.ssim_scale, ctx->tabc.as<float>(), ctx->tgimg.as<float>(), ctx->tloss.as<double>(), st));
-            launches += 2;
-        }
+        const float *tgt = o.target + (int64_t)sb.v0 * 3 * HW;
+        if (o.ssim_scale > 0)
+            CK(launch_ssim(ctx->trgb.as<float>(), tgt, 3 * L.V, cp.height, cp.width, o.l1_scale, o.ssim_scale,
+                           ctx->tabc.as<float>(), ctx->tgimg.as<float>(), ctx->tloss.as<double>(), st));
+        else
+            CK(launch_photo_l1(ctx->trgb.as<float>(), tgt, (int64_t)L.V * 3 * HW, o.l1_scale,
+                               ctx->tgimg.as<float>(), ctx->tloss.as<double>(), st));
+        launches += o.ssim_scale > 0 ? 2 : 1;
         if (rp) {
             // re-projection loss over the pairs (t, t+1) whose first view is in this sub-batch
             const int np = std::max(0, std::min(L.V, o.n_views_total - 1 - sb.v0));
-            const float *tg = o.target + (int64_t)sb.v0 * 3 * HW;
             CK(cudaMemsetAsync(ctx->tgda.p, 0, 8 * (size_t)L.V * HW, st));
             if (np > 0) {
-                CK(launch_reproj_warp(ctx->tdep.as<float>(), ctx->talp.as<float>(), tg, o.rel + 12 * (int64_t)sb.v0,
+                CK(launch_reproj_warp(ctx->tdep.as<float>(), ctx->talp.as<float>(), tgt, o.rel + 12 * (int64_t)sb.v0,
                                       np, cp, o.rp_alpha_min, ctx->twarp.as<float>(), ctx->tjac.as<float>(), st));
-                CK(launch_photo_l1(ctx->twarp.as<float>(), tg, (int64_t)np * 3 * HW, o.rp_l1_scale,
-                                   ctx->tgw.as<float>(), false, ctx->tloss.as<double>(), st));
-                launches += 2;
-                if (o.rp_ssim_scale > 0) {
-                    CK(launch_ssim(ctx->twarp.as<float>(), tg, 3 * np, cp.height, cp.width, o.rp_ssim_scale,
-                                   ctx->tabc.as<float>(), ctx->tgw.as<float>(), ctx->tloss.as<double>(), st));
-                    launches += 2;
-                }
+                if (o.rp_ssim_scale > 0)
+                    CK(launch_ssim(ctx->twarp.as<float>(), tgt, 3 * np, cp.height, cp.width, o.rp_l1_scale,
+                                   o.rp_ssim_scale, ctx->tabc.as<float>(), ctx->tgw.as<float>(),
+                                   ctx->tloss.as<double>(), st));
+                else
+                    CK(launch_photo_l1(ctx->twarp.as<float>(), tgt, (int64_t)np * 3 * HW, o.rp_l1_scale,
+                                       ctx->tgw.as<float>(), ctx->tloss.as<double>(), st));
+                launches += o.rp_ssim_scale > 0 ? 3 : 2;
                 CK(launch_reproj_back(ctx->tgw.as<float>(), ctx->tjac.as<float>(), ctx->tdep.as<float>(),
                                       ctx->talp.as<float>(), np, HW, o.rp_alpha_min, ctx->tgda.as<float>(), st));
                 launches += 1;
@@ -831,7 +831,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
                               ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.as<float>(), ctx->n,
                               ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(), o.tgrad,
                               st));
-        launches += 3;
+        launches += 2;
     }
     if (o.score) {
         CK(launch_ncc_finalize(ctx->partials.as<double>(), ctx->qpart.as<double>(), L, blend_units(cp),

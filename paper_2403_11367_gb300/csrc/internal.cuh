@@ -284,13 +284,14 @@ cudaError_t launch_pose_chain(const float *mx, const float *my, const float *mz,
                               double *out, cudaStream_t st);
 
 // ---- map training (train.cu) -------------------------------------------------
-// L1 samples: loss += scale * sum |rgb - target|, gimg (=|+=) scale * sign.
-cudaError_t launch_photo_l1(const float *rgb, const float *target, int64_t n, double scale, float *gimg,
-                            bool accumulate, double *loss, cudaStream_t st);
-// D-SSIM over planes channel planes [H][W]: loss += scale * sum (1 - SSIM),
-// gimg += its gradient; abc: 3 * planes * H * W floats of scratch.
-cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H, int W, double scale, float *abc,
-                        float *gimg, double *loss, cudaStream_t st);
+// L1 samples: loss += scale * sum |rgb - target|, gimg = scale * sign.
+cudaError_t launch_photo_l1(const float *rgb, const float *target, int64_t n, double scale, float *gimg, double *loss,
+                            cudaStream_t st);
+// L1 and D-SSIM over planes channel planes [H][W]: loss += l1_scale * sum
+// |rgb - target| + scale * sum (1 - SSIM), gimg = their gradient; abc: 3 * planes *
+// H * W floats of scratch.
+cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H, int W, double l1_scale, double scale,
+                        float *abc, float *gimg, double *loss, cudaStream_t st);
 // Re-projection of Eq. 5 for n_views consecutive pairs: targets holds views
 // 0 .. n_views (n_views + 1 images), rel [n_views][12] the relative poses;
 // warped, jac [n_views][3][H][W]; then gda [n_views][2][H][W] = dL/d(D, A).

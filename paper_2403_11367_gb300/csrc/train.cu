@@ -8,38 +8,96 @@
 
 namespace reloc {
 
-// ------------------------------------------------------------------ L1 -----
-// L1 part of L_rgb (Eq. 3) over n samples: loss += scale * sum |C - I| and
-// dL/dC = scale * sign(C - I) (sign(0) = +1, the right derivative), written
-// or added (accumulate) to gimg.  One FP64 atomic per block.
-__global__ void __launch_bounds__(256)
-k_photo_l1(const float *__restrict__ rgb, const float *__restrict__ target, int64_t n, float scale, double dscale,
-           float *__restrict__ gimg, int accumulate, double *__restrict__ loss)
+// Sums of FP32 samples in pairs hi + lo: TwoSum (Knuth, The Art of Computer
+// Programming, volume 2, section 4.2.2) gives the exact rounding error of each
+// addition, and the errors are summed in lo.  A block's sum is then within 2^-47 of
+// itself, as many bits as the FP64 sum of FP32 samples can use here (the losses add
+// 10^4 such sums in FP64), at six FP32 instructions a sample instead of two on the
+// FP64 pipe, each of which holds a scheduler's share of it for about 60 cycles.
+struct PairSum {
+    float hi, lo;
+};
+__device__ __forceinline__ void pair_add(PairSum &a, float x)
 {
-    __shared__ double s_red[8];
-    double acc = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
-        const float d = rgb[i] - target[i];
-        acc += (double)fabsf(d);
-        const float g = d >= 0.f ? scale : -scale;
-        gimg[i] = accumulate ? gimg[i] + g : g;
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += s_red[w];
-        atomicAdd(loss, s * dscale);
+    const float s = __fadd_rn(a.hi, x), b = __fsub_rn(s, a.hi);
+    a.lo = __fadd_rn(a.lo, __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    a.hi = s;
+}
+template <int LANES>
+__device__ __forceinline__ void pair_butterfly(PairSum &a)
+{
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
+        pair_add(a, h);
+        a.lo = __fadd_rn(a.lo, l);
     }
 }
+// an infinite or NaN sum is hi's alone (its error term is inf - inf)
+__device__ __forceinline__ double pair_value(PairSum a) { return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi; }
+// Total over a block of 256 threads, in thread 0.  s_pair: 8 entries; ends with
+// every thread past the barrier, so s_pair may be used again after another one.
+__device__ __forceinline__ double pair_block_total(PairSum a, PairSum *s_pair)
+{
+    pair_butterfly<32>(a);
+    if ((threadIdx.x & 31) == 0) s_pair[threadIdx.x >> 5] = a;
+    __syncthreads();
+    if (threadIdx.x >= 32) return 0.0;
+    a = s_pair[threadIdx.x & 7];
+    pair_butterfly<8>(a);
+    return threadIdx.x == 0 ? pair_value(a) : 0.0;
+}
 
-cudaError_t launch_photo_l1(const float *rgb, const float *target, int64_t n, double scale, float *gimg,
-                            bool accumulate, double *loss, cudaStream_t st)
+// ------------------------------------------------------------------ L1 -----
+// L1 part of L_rgb (Eq. 3) over n samples: loss += scale * sum |C - I| and
+// dL/dC = scale * sign(C - I) (sign(0) = +1, the right derivative), written to
+// gimg.  One FP64 atomic per block.  Bound by memory: 12 bytes a sample.  With the
+// D-SSIM term on, k_ssim_bwd forms both instead.
+__device__ __forceinline__ float l1_slope(float d, float scale) { return d >= 0.f ? scale : -scale; }
+// loss += scale * sum |d| of a block of 256 threads, N differences each.  Magnitudes
+// that could leave FP32's range when summed, infinities and NaN go the FP64 way.
+template <int N>
+__device__ __forceinline__ void l1_block_add(const float (&d)[N], double scale, PairSum *s_pair, double *loss)
+{
+    PairSum acc = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < N; ++k) pair_add(acc, fabsf(d[k]));
+    if (__syncthreads_or(!(acc.hi < 1e30f))) {
+        double t = 0.0;
+        for (int k = 0; k < N; ++k) t += fabs((double)d[k]);
+        atomicAdd(loss, t * scale);
+        return;
+    }
+    const double t = pair_block_total(acc, s_pair);
+    if (threadIdx.x == 0) atomicAdd(loss, t * scale);
+}
+
+constexpr int L1_PER = 8;            // samples of a thread, all loads in flight
+__global__ void __launch_bounds__(256)
+k_photo_l1(const float *__restrict__ rgb, const float *__restrict__ target, int64_t n, float scale, double dscale,
+           float *__restrict__ gimg, double *__restrict__ loss)
+{
+    __shared__ PairSum s_pair[8];
+    const int64_t base = (int64_t)blockIdx.x * (256 * L1_PER) + threadIdx.x;
+    float d[L1_PER];
+#pragma unroll
+    for (int k = 0; k < L1_PER; ++k) {
+        const int64_t i = base + 256 * k;
+        d[k] = i < n ? rgb[i] - target[i] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < L1_PER; ++k) {
+        const int64_t i = base + 256 * k;
+        if (i < n) gimg[i] = l1_slope(d[k], scale);
+    }
+    l1_block_add(d, dscale, s_pair, loss);
+}
+
+cudaError_t launch_photo_l1(const float *rgb, const float *target, int64_t n, double scale, float *gimg, double *loss,
+                            cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>(ceil_div(n, 256 * 8), 152 * 16);
-    k_photo_l1<<<(int)blocks, 256, 0, st>>>(rgb, target, n, (float)scale, scale, gimg, accumulate ? 1 : 0, loss);
+    k_photo_l1<<<(unsigned)ceil_div(n, 256 * L1_PER), 256, 0, st>>>(rgb, target, n, (float)scale, scale, gimg, loss);
     return cudaGetLastError();
 }
 
@@ -118,7 +176,7 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
 {
     __shared__ float sin_[2][SS_H * SS_IN_STRIDE];
     __shared__ float hsum[5][SS_H * SS_H_STRIDE];
-    __shared__ double s_red[SS_THREADS / 32];
+    __shared__ PairSum s_pair[SS_THREADS / 32];
     const int64_t HW = (int64_t)H * W;
     const int plane = blockIdx.z;
     const int x0 = blockIdx.x * SS_T, y0 = blockIdx.y * SS_T;
@@ -168,7 +226,7 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
             q[m][o] = acc;
         }
     }
-    double contrib = 0.0;
+    PairSum contrib = {0.f, 0.f};
     const int gx = x0 + col;
 #pragma unroll
     for (int o = 0; o < SS_OUT; ++o) {
@@ -186,26 +244,23 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
             po[0] = -scale * d_m;
             po[HW] = -scale * d_xx;
             po[2 * HW] = -scale * d_xy;
-            contrib += 1.0 - (double)s;
+            pair_add(contrib, 1.f);                     // 1 - s, exactly
+            pair_add(contrib, -s);
         }
     }
-    for (int off = 16; off > 0; off >>= 1) contrib += __shfl_xor_sync(0xffffffffu, contrib, off);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = contrib;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < SS_THREADS / 32; ++w) t += s_red[w];
-        atomicAdd(loss, t * dscale);
-    }
+    const double t = pair_block_total(contrib, s_pair);
+    if (threadIdx.x == 0) atomicAdd(loss, t * dscale);
 }
 
 // Backward: dL/dx(q) = sum_p w(p - q) (a(p) + 2 x(q) b(p) + y(q) c(p)) over
 // the image's pixels p (the window is symmetric, so the same separable
-// passes), added to gimg.
+// passes), plus the L1 part (its loss too): gimg is written once, and rgb and target
+// are at hand, which a pass of its own would read again.
 __global__ void __launch_bounds__(SS_THREADS)
 k_ssim_bwd(const float *__restrict__ abc, const float *__restrict__ x_img, const float *__restrict__ y_img, int H,
-           int W, SsimWin win, float *__restrict__ gimg)
+           int W, SsimWin win, float l1_scale, double l1_dscale, float *__restrict__ gimg, double *__restrict__ loss)
 {
+    __shared__ PairSum s_pair[SS_THREADS / 32];
     __shared__ float sin_[3][SS_H * SS_IN_STRIDE];
     __shared__ float hsum[3][SS_H * SS_H_STRIDE];
     const int64_t HW = (int64_t)H * W;
@@ -247,19 +302,23 @@ k_ssim_bwd(const float *__restrict__ abc, const float *__restrict__ x_img, const
             q[m][o] = acc;
         }
     }
+    float dif[SS_OUT] = {};
     const int gx = x0 + col;
 #pragma unroll
     for (int o = 0; o < SS_OUT; ++o) {
         const int gy = y0 + r0 + o;
         if (gx < W && gy < H) {
             const int64_t pix = plane * HW + (int64_t)gy * W + gx;
-            gimg[pix] += q[0][o] + 2.f * x_img[pix] * q[1][o] + y_img[pix] * q[2][o];
+            const float x = x_img[pix], y = y_img[pix];
+            dif[o] = x - y;
+            gimg[pix] = l1_slope(dif[o], l1_scale) + (q[0][o] + 2.f * x * q[1][o] + y * q[2][o]);
         }
     }
+    l1_block_add(dif, l1_dscale, s_pair, loss);
 }
 
-cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H, int W, double scale, float *abc,
-                        float *gimg, double *loss, cudaStream_t st)
+cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H, int W, double l1_scale, double scale,
+                        float *abc, float *gimg, double *loss, cudaStream_t st)
 {
     if (planes <= 0) return cudaSuccess;
     const SsimWin win = ssim_window();
@@ -267,7 +326,7 @@ cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H
     k_ssim_fwd<<<grid, SS_THREADS, 0, st>>>(rgb, target, H, W, win, (float)scale, scale, abc, loss);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_ssim_bwd<<<grid, SS_THREADS, 0, st>>>(abc, rgb, target, H, W, win, gimg);
+    k_ssim_bwd<<<grid, SS_THREADS, 0, st>>>(abc, rgb, target, H, W, win, (float)l1_scale, l1_scale, gimg, loss);
     return cudaGetLastError();
 }
 
