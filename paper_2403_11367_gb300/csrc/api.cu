@@ -127,10 +127,10 @@ struct ResultBlock {
     int *degen = nullptr;               // [V]
     int *best = nullptr;                // [Q]
     int *done = nullptr;                // [V] tile scan: finished blocks
-    int *queues = nullptr;              // [sub-batches][4] blend queue counters
+    int *queues = nullptr;              // [sub-batches][5] blend queue counters
 };
 
-size_t result_scratch_bytes(int64_t V, int64_t n_sb) { return 4 * (size_t)(V + 4 * n_sb); }
+size_t result_scratch_bytes(int64_t V, int64_t n_sb) { return 4 * (size_t)(V + 5 * n_sb); }
 
 // Places a block at base (null: only its size).  Returns its bytes.
 size_t result_block(char *base, int64_t V, int64_t Q, int64_t n_sb, ResultBlock *out)
@@ -769,8 +769,9 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
     }
     stage_mark(ctx, sbi, RELOC_STAGE_TILE_COUNT, st, capturing);
     // work queues of the sub-batch's blend and of its winners'
-    const BlendQueue queue{R.queues + 4 * sbi, ctx->bqueue.as<int>()};
-    const BlendQueue queue_w{R.queues + 4 * sbi + 2, ctx->bqueue.as<int>()};
+    const BlendQueue queue{R.queues + 5 * sbi, ctx->bqueue.as<int>()};
+    int *const ticket_g = R.queues + 5 * sbi + 4;          // the backward blend's
+    const BlendQueue queue_w{R.queues + 5 * sbi + 2, ctx->bqueue.as<int>()};
     CK(launch_tile_count(ctx->v1b.as<uint32_t>(), nvis, ctx->rect.as<uint2>(), L, cp, sb.cb, sb.cb_view, ctx->srect.as<uint2>(),
                          ctx->bhist.as<uint32_t>(), ctx->ranges.as<int2>(), ninst, R.done + sb.v0, d_overflow, queue, st));
     launches += sb.cb > 0 ? 2 : 1;
@@ -826,7 +827,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
                              ctx->tgimg.as<float>(), rp ? ctx->tgda.as<float>() : nullptr, ctx->trgb.as<float>(),
                              rp ? ctx->tdep.as<float>() : nullptr, rp ? ctx->talp.as<float>() : nullptr,
-                             ctx->gbuf.as<float>(), d_overflow, st));
+                             ctx->gbuf.as<float>(), d_overflow, queue, ticket_g, st));
         CK(launch_param_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
                               ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.as<float>(), ctx->n,
                               ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(), o.tgrad,
@@ -843,7 +844,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
             CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
                                  ctx->gcoef.as<double>(), nullptr, nullptr,
                                  o.keep_rgb ? ctx->trgb.as<float>() : nullptr, nullptr, nullptr,
-                                 ctx->gbuf.as<float>(), d_overflow, st));
+                                 ctx->gbuf.as<float>(), d_overflow, queue, ticket_g, st));
             CK(launch_pose_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
                                  ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.p, ctx->precision, ctx->n,
                                  ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(),

@@ -271,10 +271,11 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // gout[vd_off[v] + i][10] (u, v, a, b, c, r, g, b, opacity, z).  cimg (may be
 // null) [V][3][H][W]: the views' forward render (cdep, calp [V][H][W] its depth
 // and alpha, needed with gda), so the colour need not be composited again.
+// queue: the heavy tiles (launch_tile_count); ticket: zeroed before the call.
 cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
-                              const int *overflow, cudaStream_t st);
+                              const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st);
 
 // Chain of gin to each view's left pose update: out[V][6] (rho, phi);
 // part: n_blocks * V * 6 doubles of scratch.

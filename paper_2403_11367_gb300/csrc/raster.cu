@@ -669,7 +669,7 @@ k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
         int64_t un;
         int vn;
         int2 rn;
-        const bool heavy = HALF && r.y - r.x >= BLEND_HEAVY;
+        const bool heavy = r.y - r.x >= BLEND_HEAVY;
         if (!heavy) next(un, vn, rn);
         const int vi = (int)(u / upv);
         const int loc = (int)(u - (int64_t)vi * upv);
@@ -691,7 +691,7 @@ k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
 // per kernel (every k_blend has the same function type: one cache for that type
 // gave the scoring launches the export launches' 28 blocks per SM in a process
 // that had rendered first).
-template <int TW, int TH, int RPL, bool DA, bool HALF>
+template <auto KERNEL>
 static int blend_resident()
 {
     static std::atomic<int> cached[64];
@@ -701,7 +701,7 @@ static int blend_resident()
     if (!c) {
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_blend<TW, TH, RPL, DA, HALF>, 32, 0) != cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, 32, 0) != cudaSuccess)
             return 0;
         c = sms * (per_sm > 0 ? per_sm : 1);
         cached[dev].store(c);
@@ -733,11 +733,11 @@ static cudaError_t blend_t(Records rec, const Layout &L, const uint32_t *inst_ga
     // half blocks raise.
     if constexpr (RPL == 1) {
         if (!partials && nv < BLEND_HALF_VIEWS)
-            return da ? run(k_blend<TW, TH, 1, true, true>, blend_resident<TW, TH, 1, true, true>(), 2 * units)
-                      : run(k_blend<TW, TH, 1, false, true>, blend_resident<TW, TH, 1, false, true>(), 2 * units);
+            return da ? run(k_blend<TW, TH, 1, true, true>, blend_resident<k_blend<TW, TH, 1, true, true>>(), 2 * units)
+                      : run(k_blend<TW, TH, 1, false, true>, blend_resident<k_blend<TW, TH, 1, false, true>>(), 2 * units);
     }
-    return da ? run(k_blend<TW, TH, RPL, true, false>, blend_resident<TW, TH, RPL, true, false>(), units)
-              : run(k_blend<TW, TH, RPL, false, false>, blend_resident<TW, TH, RPL, false, false>(), units);
+    return da ? run(k_blend<TW, TH, RPL, true, false>, blend_resident<k_blend<TW, TH, RPL, true, false>>(), units)
+              : run(k_blend<TW, TH, RPL, false, false>, blend_resident<k_blend<TW, TH, RPL, false, false>>(), units);
 }
 
 cudaError_t launch_blend(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
@@ -861,6 +861,10 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // instructions a record where a reduce-scatter by shuffles takes 62, a third of the
 // whole walk, and one atomic instruction a group: 16 driving views 5.93 ms a step for
 // 6.61, and at 64 registers (the reduction's own array is gone) 5.91.
+// IMG = true (training: many views): resident warps take their units from a queue,
+// the heavy tiles' first, so that no long list starts near the end: 2.90 -> 2.66 ms
+// of the 16 views' step.  IMG = false: a block per unit, which one view's gradient
+// (the usual call) is faster with, 305 us against 337 from the queue.
 // IMG = false: L is the view's NCC (G from coef), five outputs (u, v, a, b, c).
 // IMG = true: G is given per pixel (gimg [V][3][H][W], an image loss's
 // gradient), and optionally G_D, G_A (gda [V][2][H][W]); ten outputs: also
@@ -868,12 +872,12 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // cimg (may be null): the forward's render of the views ([V][3][H][W], in image
 // mode with cdep, calp [V][H][W] when gda is given) replaces the first walk.
 template <int TW, int TH, bool IMG>
-__global__ void __launch_bounds__(32, 32)
-k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
-             const int2 *__restrict__ ranges, CamParams cam, const double *__restrict__ coef,
-             const float *__restrict__ gimg, const float *__restrict__ gda, const float *__restrict__ cimg,
-             const float *__restrict__ cdep, const float *__restrict__ calp, float *__restrict__ gout,
-             const int *__restrict__ overflow)
+__device__ __forceinline__ void blend_grad_unit(const Records &rec, const Layout &L,
+                                                const uint32_t *__restrict__ inst_gauss, const CamParams &cam,
+                                                const double *__restrict__ coef, const float *__restrict__ gimg,
+                                                const float *__restrict__ gda, const float *__restrict__ cimg,
+                                                const float *__restrict__ cdep, const float *__restrict__ calp,
+                                                float *__restrict__ gout, int v, int unit, int2 r)
 {
     constexpr int NOUT = IMG ? 10 : 5;
     constexpr int GRP = 30 / NOUT;              // records summed together
@@ -889,11 +893,9 @@ k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
     // record; rows 36 apart: 16-byte rows, no bank conflict along or across them
     __shared__ __align__(16) float s_t[30][36];
     __shared__ uint32_t s_tg[GRP];              // the group's Gaussians
-    const int unit = blockIdx.x;
-    const int tile = unit / WPT, warp = unit - tile * WPT;
-    const int v = blockIdx.y;
-    const int tx = tile % cam.ntx, ty = tile / cam.ntx;
     const int lane = threadIdx.x;
+    const int tile = unit / WPT, warp = unit - tile * WPT;
+    const int tx = tile % cam.ntx, ty = tile / cam.ntx;
     const int bx0p = tx * TW + (warp % GM::NBX) * BW, by0p = ty * TH + (warp / GM::NBX) * BH;
     const int px = bx0p + lane % BW;
     const int py0 = by0p + 2 * (lane / BW);
@@ -902,8 +904,6 @@ k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
     const float DX = (float)(lane % BW) + 0.5f - 0.5f * BW;
     const float dy0 = (float)(2 * (lane / BW)) + 0.5f - 0.5f * BH;
     const f32x2 DY2 = pk(dy0, dy0 + 1.f);
-    if (*overflow) return;
-    const int2 r = ranges[(int64_t)v * cam.n_tiles + tile];
     const uint32_t *list = inst_gauss + L.io_off[v];
     const float4 *geom = rec.geom + 2 * L.vd_off[v], *col = rec.col + L.vd_off[v];
     const float limL = -0.5f * cam.cut * cam.cut * L2E;
@@ -1168,32 +1168,74 @@ k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
     if (held) flush();
 }
 
+template <int TW, int TH, bool IMG>
+__global__ void __launch_bounds__(32, IMG ? 27 : 32)
+k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
+             const int2 *__restrict__ ranges, CamParams cam, const double *__restrict__ coef,
+             const float *__restrict__ gimg, const float *__restrict__ gda, const float *__restrict__ cimg,
+             const float *__restrict__ cdep, const float *__restrict__ calp, float *__restrict__ gout,
+             const int *__restrict__ overflow, BlendQueue queue, int *__restrict__ ticket)
+{
+    constexpr int WPT = BlockGeom<TW, TH>::WPT;
+    if (*overflow) return;
+    if (!IMG) {
+        const int2 r = ranges[(int64_t)blockIdx.y * cam.n_tiles + blockIdx.x / WPT];
+        if (r.x < r.y)
+            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, blockIdx.y,
+                                         blockIdx.x, r);
+        return;
+    }
+    const int upv = cam.n_tiles * WPT;                          // units per view
+    const int64_t total = (int64_t)upv * L.V, hh = (int64_t)queue.count[1] * WPT;
+    while (true) {
+        // the next unit of the queue: the heavy tiles', then the others in order
+        int64_t u = 0;
+        if (threadIdx.x == 0) u = atomicAdd(ticket, 1);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        const bool listed = u < hh;
+        if (listed) {
+            const int t = queue.list[(int)(u / WPT)];
+            u = (int64_t)(t / cam.n_tiles) * upv + (int64_t)(t % cam.n_tiles) * WPT + u % WPT;
+        } else {
+            u -= hh;
+        }
+        if (u >= total) break;
+        const int v = (int)(u / upv), unit = (int)(u - (int64_t)v * upv);
+        const int2 r = ranges[(int64_t)v * cam.n_tiles + unit / WPT];
+        if (r.x < r.y && (listed || r.y - r.x < BLEND_HEAVY))
+            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, v, unit, r);
+        __syncwarp();
+    }
+}
+
 template <int TW, int TH>
 static cudaError_t blend_grad_t(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                                 const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                                 const float *cimg, const float *cdep, const float *calp, float *gout,
-                                const int *overflow, cudaStream_t st)
+                                const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
 {
-    dim3 grid(cam.n_tiles * (TW * TH / 64), L.V);
-    if (gimg)
-        k_blend_grad<TW, TH, true><<<grid, 32, 0, st>>>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep,
-                                                        calp, gout, overflow);
-    else
-        k_blend_grad<TW, TH, false><<<grid, 32, 0, st>>>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg,
-                                                         nullptr, nullptr, gout, overflow);
+    const int units = cam.n_tiles * (TW * TH / 64);             // per view
+    if (gimg) {
+        const int resident = blend_resident<k_blend_grad<TW, TH, true>>();
+        if (resident <= 0) return cudaErrorInvalidValue;
+        k_blend_grad<TW, TH, true><<<(unsigned)min64((int64_t)units * L.V, resident), 32, 0, st>>>(
+            rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep, calp, gout, overflow, queue, ticket);
+    } else {
+        k_blend_grad<TW, TH, false><<<dim3(units, L.V), 32, 0, st>>>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg,
+                                                                     nullptr, nullptr, gout, overflow, queue, ticket);
+    }
     return cudaGetLastError();
 }
-
 cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
-                              const int *overflow, cudaStream_t st)
+                              const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
 {
     if (L.V <= 0) return cudaSuccess;
 #define RELOC_GRAD_CASE(W_, H_) \
     if (cam.tile_w == W_ && cam.tile_h == H_) \
         return blend_grad_t<W_, H_>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep, calp, gout, \
-                                    overflow, st);
+                                    overflow, queue, ticket, st);
     RELOC_GRAD_CASE(16, 16)
     RELOC_GRAD_CASE(8, 8)
     RELOC_GRAD_CASE(32, 8)
