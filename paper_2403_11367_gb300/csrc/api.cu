@@ -1220,9 +1220,9 @@ static reloc_status apply_proposal(reloc_ctx *ctx, std::vector<QuerySpec> &qs, c
     CKS(run_batch(ctx, seeds, cam, st, ro, false));
     // (b) inputs, (c) logits and top-k
     __nv_bfloat16 *in = ctx->prop_in.as<__nv_bfloat16>();
-    for (int j = 0; j < Ql; ++j)
-        CK(proposal_make_input(qs[sel[j]].img, ctx->prop_seed.as<float>() + (int64_t)j * 3 * HW, H, W,
-                               in + (int64_t)j * PROPOSAL_H * PROPOSAL_W * 2, st));
+    std::vector<const float *> imgs(Ql);
+    for (int j = 0; j < Ql; ++j) imgs[j] = qs[sel[j]].img;
+    CK(proposal_make_inputs(imgs.data(), ctx->prop_seed.as<float>(), Ql, H, W, in, st));
     CK(proposal_forward(ctx->prop, in, Ql, ctx->prop_logits.as<float>(), st));
     CK(launch_topk(ctx->prop_logits.as<float>(), Ql, PROPOSAL_CLASSES, ctx->prop_k, ctx->prop_idx.as<int32_t>(),
                    ctx->prop_mrg.as<float>(), st));
@@ -1498,8 +1498,8 @@ extern "C" reloc_status reloc_proposal_make_input(reloc_ctx *ctx, const float *q
     if (cam->height % PROPOSAL_H || cam->width % PROPOSAL_W || cam->height / PROPOSAL_H != cam->width / PROPOSAL_W)
         return fail(RELOC_EINVAL, "the proposal needs H = 47 f and W = 176 f");
     CK(cudaSetDevice(ctx->device));
-    CK(proposal_make_input(query_dev, coarse_rgb_dev, cam->height, cam->width, (__nv_bfloat16 *)input_dev,
-                           (cudaStream_t)stream));
+    CK(proposal_make_inputs(&query_dev, coarse_rgb_dev, 1, cam->height, cam->width, (__nv_bfloat16 *)input_dev,
+                            (cudaStream_t)stream));
     return RELOC_OK;
 }
 

@@ -11,29 +11,58 @@
 
 namespace reloc {
 
-// 8x box average of the RGB mean (gray) of a planar [3][H][W] image into
-// channel `ch` of an NHWC [Ho][Wo][2] BF16 input, Ho = H / f, Wo = W / f.
-__global__ void k_downsample_gray(const float *__restrict__ img, int H, int W, int f, int ch,
-                                  __nv_bfloat16 *__restrict__ out)
+// f x f box average of the RGB mean (gray) of planar [3][H][W] images into NHWC
+// [n][H / f][W / f][2] BF16 inputs: channel 0 from query j, channel 1 from render j.
+// A thread sums one output in a fixed order (rows, columns, r + g + b).  One launch
+// for GRAY_PAIRS queries and renders; bound by reading them (406 MB for 32 driving
+// queries, 60 us).  An image a launch and a value a load kept 33 blocks of 256
+// threads waiting for one row after the other: 64 launches of 11 us, 62 us
+// now.  VEC: f a multiple of 4 and rows on 16 bytes, so four columns a load.
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+k_downsample_gray(GrayQueries q, const float *__restrict__ render, int H, int W, int f, __nv_bfloat16 *__restrict__ out)
 {
     const int Ho = H / f, Wo = W / f;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= Ho * Wo) return;
+    const int j = blockIdx.y >> 1, ch = blockIdx.y & 1;
     const int oy = i / Wo, ox = i % Wo;
     const int64_t HW = (int64_t)H * W;
+    const float *img = ch ? render + 3 * HW * j : q.img[j];
     float s = 0.f;
-    for (int y = oy * f; y < oy * f + f; ++y)
-        for (int x = ox * f; x < ox * f + f; ++x) {
-            const int64_t p = (int64_t)y * W + x;
-            s += img[p] + img[HW + p] + img[2 * HW + p];
-        }
-    out[(int64_t)i * 2 + ch] = __float2bfloat16_rn(s / (3.f * f * f));
+    if (VEC) {
+#pragma unroll 2
+        for (int y = oy * f; y < oy * f + f; ++y)
+#pragma unroll 2
+            for (int x = ox * f; x < ox * f + f; x += 4) {
+                const float *p = img + (int64_t)y * W + x;
+                const float4 r = *reinterpret_cast<const float4 *>(p), g = *reinterpret_cast<const float4 *>(p + HW),
+                             b = *reinterpret_cast<const float4 *>(p + 2 * HW);
+                s += r.x + g.x + b.x;
+                s += r.y + g.y + b.y;
+                s += r.z + g.z + b.z;
+                s += r.w + g.w + b.w;
+            }
+    } else {
+        for (int y = oy * f; y < oy * f + f; ++y)
+            for (int x = ox * f; x < ox * f + f; ++x) {
+                const int64_t p = (int64_t)y * W + x;
+                s += img[p] + img[HW + p] + img[2 * HW + p];
+            }
+    }
+    out[((int64_t)j * Ho * Wo + i) * 2 + ch] = __float2bfloat16_rn(s / (3.f * f * f));
 }
 
-cudaError_t launch_downsample_gray(const float *img, int H, int W, int f, int ch, __nv_bfloat16 *out, cudaStream_t st)
+cudaError_t launch_downsample_gray(const GrayQueries &q, const float *render, int n, int H, int W, int f,
+                                   __nv_bfloat16 *out, cudaStream_t st)
 {
-    const int n = (H / f) * (W / f);
-    k_downsample_gray<<<(n + 255) / 256, 256, 0, st>>>(img, H, W, f, ch, out);
+    bool vec = f % 4 == 0 && W % 4 == 0 && ((uintptr_t)render & 15) == 0;
+    for (int j = 0; j < n; ++j) vec = vec && ((uintptr_t)q.img[j] & 15) == 0;
+    const dim3 grid((unsigned)(((H / f) * (W / f) + 255) / 256), (unsigned)(2 * n));
+    if (vec)
+        k_downsample_gray<true><<<grid, 256, 0, st>>>(q, render, H, W, f, out);
+    else
+        k_downsample_gray<false><<<grid, 256, 0, st>>>(q, render, H, W, f, out);
     return cudaGetLastError();
 }
 

@@ -334,8 +334,13 @@ cudaError_t proposal_train_step(ProposalNet *P, const __nv_bfloat16 *in, const i
 const float *proposal_logits(const ProposalNet *P);
 // != 0 once a tensor-core wait of a finished launch gave up
 int proposal_status(const ProposalNet *P);
-cudaError_t proposal_make_input(const float *query, const float *seed_rgb, int H, int W, __nv_bfloat16 *out,
-                                cudaStream_t st);
+constexpr int GRAY_PAIRS = 64;
+struct GrayQueries {
+    const float *img[GRAY_PAIRS];
+};
+// Network inputs of n queries and their coarse-pose renders (renders [n][3][H][W]).
+cudaError_t proposal_make_inputs(const float *const *queries, const float *renders, int n, int H, int W,
+                                 __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t launch_gemm_bf16(const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *bias, float *Cf,
                              __nv_bfloat16 *Cb, int M, int N, int K, int lda, int ldb, int ldc, int relu, int split_k,
                              float *partials, int *status, cudaStream_t st, int inject = 0);

@@ -12,6 +12,7 @@
 // Flat parameter layout (FP32, used for save/load and for checks): for each
 // conv layer W[C_out][3][3][C_in] then b[C_out]; then FC1 W[1024][1536],
 // b[1024]; FC2 W[64][1024], b[64] -- 1,916,960 values.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -20,7 +21,8 @@
 
 namespace reloc {
 
-cudaError_t launch_downsample_gray(const float *img, int H, int W, int f, int ch, __nv_bfloat16 *out, cudaStream_t st);
+cudaError_t launch_downsample_gray(const GrayQueries &q, const float *render, int n, int H, int W, int f,
+                                   __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t launch_im2col(const __nv_bfloat16 *x, int B, int H, int W, int C, int Ho, int Wo, int Kp,
                           __nv_bfloat16 *col, cudaStream_t st);
 cudaError_t launch_relu_back(const float *d, int H, int W, int Ho, int Wo, int Kp, const __nv_bfloat16 *y, int M, int N,
@@ -384,12 +386,17 @@ cudaError_t proposal_train_step(ProposalNet *P, const __nv_bfloat16 *in, const i
 const float *proposal_logits(const ProposalNet *P) { return P->logits.as<float>(); }
 int proposal_status(const ProposalNet *P) { return *(volatile int *)P->status.p; }
 
-cudaError_t proposal_make_input(const float *query, const float *seed_rgb, int H, int W, __nv_bfloat16 *out,
-                                cudaStream_t st)
+cudaError_t proposal_make_inputs(const float *const *queries, const float *renders, int n, int H, int W,
+                                 __nv_bfloat16 *out, cudaStream_t st)
 {
-    const int f = H / IN_H;
-    PK(launch_downsample_gray(query, H, W, f, 0, out, st));
-    return launch_downsample_gray(seed_rgb, H, W, f, 1, out, st);
+    for (int j0 = 0; j0 < n; j0 += GRAY_PAIRS) {
+        const int m = std::min(GRAY_PAIRS, n - j0);
+        GrayQueries q = {};
+        for (int j = 0; j < m; ++j) q.img[j] = queries[j0 + j];
+        PK(launch_downsample_gray(q, renders + (int64_t)j0 * 3 * H * W, m, H, W, H / IN_H,
+                                  out + (int64_t)j0 * IN_H * IN_W * IN_C, st));
+    }
+    return cudaSuccess;
 }
 
 }  // namespace reloc
