@@ -121,7 +121,7 @@ typedef struct reloc_counts {
 
 /* Stage indices of reloc_stage_times(). */
 enum {
-    RELOC_STAGE_CULL = 0,      /* block subset gather (K1)                              */
+    RELOC_STAGE_CULL = 0,      /* nothing: the subset gather (K1) runs in K2's launch    */
     RELOC_STAGE_PROJECT,       /* EWA projection + SH (K2)                              */
     RELOC_STAGE_DEPTH_SORT,    /* visibility compaction + depth radix sort             */
     RELOC_STAGE_TILE_COUNT,    /* per-chunk tile counts, scan into tile ranges (K3)     */

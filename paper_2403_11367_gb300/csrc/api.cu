@@ -1,6 +1,6 @@
 // api.cu -- the C ABI of reloc.h: context, map load, block selection,
 // candidate grid, and the per-call orchestration of the kernels
-// (K1 gather -> K2 project -> depth sort -> K3 tile counts + ranges ->
+// (K1 + K2 gather and project -> depth sort -> K3 tile counts + ranges ->
 //  K4 tile emission -> K6 blend + NCC partials -> K7 NCC -> K8 argmax -> export).
 //
 // All stages run on the caller's stream with device-resident counts, so a

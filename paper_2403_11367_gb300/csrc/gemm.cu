@@ -189,7 +189,7 @@ struct GemmSmem {
     static constexpr uint32_t B_BYTES = BN * GEMM_BK * 2;
     static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
     // four stages of the widest tile fill the SM's shared memory; narrower
-    // tiles take the loads' latency on four stages too, two CTAs to an SM
+    // tiles need four for the loads' latency too
     static constexpr int STAGES = 4;
     static constexpr size_t EPI = (size_t)GEMM_EPI_WARPS * 32 * GEMM_EPI_LD * 4;
     static constexpr size_t TOTAL = (size_t)STAGES * STAGE + EPI + 1024;   // + alignment slack
