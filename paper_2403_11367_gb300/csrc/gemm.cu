@@ -30,7 +30,8 @@
 //     shared memory so that a row's 32 values leave as one 128-byte store (a
 //     lane's own row written straight from its registers put every lane of a
 //     store on another line, and the write took several times as long as the
-//     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us).  Bias and
+//     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us, and 53 with the
+//     waits below; 8192 x 8192 x 8192, where the write is a fortieth, 1060 and 1102).  Bias and
 //     ReLU are applied there.
 // An MN-major operand's tile is loaded as boxes of 64 columns (128 bytes) by the
 // 64 rows of the K step, in the canonical MN-major SWIZZLE_128B layout; its
@@ -59,6 +60,12 @@ constexpr int GEMM_BM = 128;
 constexpr int GEMM_BK = 64;
 constexpr int GEMM_EPI_LD = 36;                     // floats per staged row: 16-byte rows, no bank conflict
 constexpr unsigned long long GEMM_WAIT_NS = 1000000000ull;   // 1 s per wait
+// Tries between two looks at the timer.  A timer read before the first try and after
+// every further one stood in the chain from a stage's MMAs over its refill to its
+// next MMAs: 8192 x 8192 x 8192 1360 us, 1135 so (one try that sleeps up to 20 us in
+// hardware: 1178); 8192 x 1024 x 1536 57.5 -> 53.
+constexpr int GEMM_TRIES = 64;
+constexpr int GEMM_BAND = 16;                       // row tiles of a band of the tile order
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -106,19 +113,26 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N, bool a_mn, 
 }
 
 // Wait until the phase of the given parity has completed, or GEMM_WAIT_NS.
+__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done)
+                 : "r"(mbar), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
 {
-    const unsigned long long deadline = global_ns() + GEMM_WAIT_NS;
+    unsigned long long deadline = 0;
     for (;;) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(mbar), "r"(parity)
-                     : "memory");
-        if (done) return true;
-        if (global_ns() > deadline) return false;
+        for (int k = 0; k < GEMM_TRIES; ++k)
+            if (mbar_try(mbar, parity)) return true;
+        const unsigned long long now = global_ns();
+        if (deadline == 0) deadline = now + GEMM_WAIT_NS;
+        if (now > deadline) return false;
     }
 }
 
@@ -196,6 +210,16 @@ struct GemmSmem {
     static constexpr uint32_t TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;       // two accumulators, power of two >= 32
 };
 
+// Row and column tile of tile mn: bands of 16 row tiles, columns after one another
+// within a band, so that the tiles in flight share their operands in both directions
+// (one row of tiles after the other reads all of B again for every five rows of A).
+// 8192 x 8192 x 8192: 1135 -> 1102 us; bands of 8 1140, of 32 1120, one band 1170.
+__device__ __forceinline__ int2 gemm_tile(int mn, int n_tm, int n_tn)
+{
+    const int per = GEMM_BAND * n_tn, band = mn / per, r = mn - band * per, rows = min(GEMM_BAND, n_tm - GEMM_BAND * band);
+    return make_int2(GEMM_BAND * band + r % rows, r / rows);
+}
+
 template <int BN, bool AMN, bool BMN>
 __global__ void __launch_bounds__(GEMM_THREADS)
 k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs g)
@@ -243,6 +267,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const uint32_t sbase = smem_u32(smem);
     // a bounded wait that gave up stops every role of the CTA
     auto wait = [&](uint64_t &bar, uint32_t parity) -> bool {
+        if (mbar_try(smem_u32(&bar), parity)) return true;
         if (abort_s) return false;
         if (mbar_wait(smem_u32(&bar), parity)) return true;
         abort_s = 1;
@@ -256,13 +281,13 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         bool ok = true;
         for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
             const int z = t / n_mn, mn = t - z * n_mn;
-            const int m0 = mn / g.n_tn * GEMM_BM, n0 = mn % g.n_tn * BN, kbeg = z * k_per;
+            const int2 tile = gemm_tile(mn, n_mn / g.n_tn, g.n_tn);
+            const int m0 = tile.x * GEMM_BM, n0 = tile.y * BN, kbeg = z * k_per;
             for (int k = 0; k < n_k; ++k, ++it) {
                 const int s = it % STAGES;
                 const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
                 // the stage is free once the MMAs of K step it - STAGES have read it
                 if (it >= STAGES && !wait(bar_empty[s], ph ^ 1u)) { ok = false; break; }
-                if (abort_s) { ok = false; break; }
                 const uint32_t sa = sbase + s * SM::STAGE, sb = sa + SM::A_BYTES;
                 const uint32_t fb = smem_u32(&bar_full[s]);
                 mbar_expect_tx(fb, SM::STAGE);
@@ -336,7 +361,8 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         int i = 0;
         for (int t = blockIdx.x; t < g.n_tiles; t += gridDim.x, ++i) {
             const int z = t / n_mn, mn = t - z * n_mn;
-            const int row0 = mn / g.n_tn * GEMM_BM + quad * 32, n0 = mn % g.n_tn * BN;
+            const int2 tile = gemm_tile(mn, n_mn / g.n_tn, g.n_tn);
+            const int row0 = tile.x * GEMM_BM + quad * 32, n0 = tile.y * BN;
             // every lane waits for itself; one that gave up takes the warp out
             if (!__all_sync(0xffffffffu, wait(bar_tfull[i & 1], (uint32_t)(i >> 1) & 1u))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
