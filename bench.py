@@ -43,7 +43,8 @@ N_QUERIES = 4
 # particular kernel's instruction mix
 FLOPS_PER_EVAL = 22
 # dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of this
-# workload's 64-view scoring k_blend launch of query 0 (1559.56 MB + 18.85 MB); to be re-taken whenever that kernel changes (None: not taken)
+# workload's 64-view scoring k_blend launch of query 0 (1559.56 MB +
+# 18.85 MB); to be re-taken whenever that kernel changes (None: not taken)
 BLEND_DRAM_BYTES_PER_LAUNCH = 1_578_414_592
 WORKLOAD = ("driving street: 2M Gaussians SH3 FP32, 20 m blocks, 40 m radius (~280k-320k/query), "
             "1408x376 fx=fy=552, 64 candidates (4x4x4 grid 0.5 m / 2 deg), 16x16 tiles")

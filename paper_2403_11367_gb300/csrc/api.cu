@@ -494,8 +494,8 @@ static reloc_status make_cam(const reloc_ctx *ctx, const reloc_camera *cam, CamP
 // by one warp in depth order, and the row through the horizon meets nearly all
 // of a chunk: a driving view's 51 chunks of 2048 left 113 us to that row's warps
 // on an idle GPU, 409 chunks of 256 take 29 us; 16 views (6.4 M pairs) emit in
-// 146 us at 1024 to a chunk, 169 at 2048, 192 at 256; 64 views gain nothing below
-// 2048, and every chunk costs a row of per-tile counts.
+// 133 us at 1024 to a chunk, 138 at 512 (and count in 87 for 62 us); 64 views gain 4 us
+// at 1024 and count 28 us longer: every chunk costs a row of per-tile counts.
 static void set_bin_chunk(CamParams &cp, int64_t pairs)
 {
     int chunk = BIN_CHUNK_MAX;

@@ -61,9 +61,9 @@ __device__ __forceinline__ double cs_warp_total(CSum c)
 }
 
 // ------------------------------------------------------------------ K6 -----
-// One CTA per (view, tile).  Each thread owns two vertically adjacent pixels,
-// so a warp covers a TW x (64/TW) pixel block, and the warps of a tile run
-// independently (no barrier until the NCC epilogue).  A warp walks the tile's
+// A warp per 64-pixel block of a (view, tile), a TW x (64/TW) strip (16 x 4 for
+// wider tiles), each lane owning two vertically adjacent pixels; blocks are
+// independent.  A warp walks the tile's
 // sorted list RPL*32 records at a time: each lane loads its records (the
 // tile's warps read the same records, so after the first they hit L1),
 // derives the power threshold below which a record cannot contribute --
