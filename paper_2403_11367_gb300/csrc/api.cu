@@ -174,6 +174,7 @@ struct reloc_ctx {
     DevBuf gbuf, gcoef, gpart, gpose;    // NCC pose gradients
     // map training: render and dL/dC scratch, loss, parameter gradients, Adam moments
     DevBuf trgb, tgimg, tabc, tloss, tgrad, adam_m, adam_v;
+    DevBuf tconic;                       // the conics' gradients of a sub-batch
     DevBuf tdep, talp, twarp, tjac, tgw, tgda, trel;     // re-projection loss
     int64_t adam_t = 0;
     PinBuf pin, gemm_status, pnp_out, prop_loss;
@@ -289,7 +290,7 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
                       &ctx->qpart, &ctx->res, &ctx->view_sel, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
                       &ctx->hdepth, &ctx->prop_in, &ctx->prop_seed, &ctx->prop_logits, &ctx->prop_idx,
                       &ctx->prop_mrg, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
-                      &ctx->gpart, &ctx->gpose};
+                      &ctx->gpart, &ctx->gpose, &ctx->tconic};
     for (DevBuf *b : bufs) b->release();
     if (ctx->prop) proposal_destroy(ctx->prop);
     ctx->pin.release();
@@ -581,17 +582,18 @@ static int64_t inst_cap(const reloc_ctx *ctx, int64_t S, int64_t override_cap)
 // Workspace bytes of one query: per view, the per-Gaussian arrays (records,
 // rectangle, depth key, a key/value sort buffer, the depth order, depth-ordered
 // rectangle, radix histograms), the instance list, ranges, NCC partials per
-// warp block and the per-chunk tile counts; plus the gathered subset.
-static int64_t query_bytes(int64_t S, int V, int64_t cap, const CamParams &cp)
+// warp block and the per-chunk tile counts; plus the gathered subset.  grad_bytes:
+// those of one (view, Gaussian)'s gradients, for calls that form them.
+static int64_t query_bytes(int64_t S, int V, int64_t cap, const CamParams &cp, int grad_bytes)
 {
-    const int64_t per_view = S * 85 + cap * 4 + (int64_t)cp.n_tiles * 8 + (int64_t)blend_units(cp) * 24 +
+    const int64_t per_view = S * (85 + grad_bytes) + cap * 4 + (int64_t)cp.n_tiles * 8 + (int64_t)blend_units(cp) * 24 +
                              4 * (int64_t)cp.n_tiles * ceil_div(S, cp.bin_chunk) + 1024;
     return (int64_t)V * per_view + S * 4 + 4096;
 }
 
 // Split the call into sub-batches and build each one's host tables.
 static void plan_batches(const reloc_ctx *ctx, const std::vector<QuerySpec> &qs, const std::vector<int64_t> &caps,
-                         const CamParams &cp, std::vector<SubBatch> &out)
+                         const CamParams &cp, int grad_bytes, std::vector<SubBatch> &out)
 {
     out.clear();
     const int Q = (int)qs.size();
@@ -602,7 +604,7 @@ static void plan_batches(const reloc_ctx *ctx, const std::vector<QuerySpec> &qs,
         sb.v0 = vglob;
         int64_t bytes = 0, units = 0;
         while (q < Q) {
-            const int64_t b = query_bytes(qs[q].S, qs[q].V, caps[q], cp);
+            const int64_t b = query_bytes(qs[q].S, qs[q].V, caps[q], cp, grad_bytes);
             const int64_t un = (int64_t)qs[q].V * blend_units(cp);
             if (q > sb.q0 && (bytes + b > ctx->mem_budget || units + un > BLEND_MAX_UNITS)) break;
             bytes += b;
@@ -823,15 +825,16 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
                 launches += 1;
             }
         }
-        CK(cudaMemsetAsync(ctx->gbuf.p, 0, 40 * (size_t)sb.VS, st));
+        CK(cudaMemsetAsync(ctx->gbuf.p, 0, 28 * (size_t)sb.VS, st));
+        CK(cudaMemsetAsync(ctx->tconic.p, 0, 24 * (size_t)sb.VS, st));
         CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp, nullptr,
                              ctx->tgimg.as<float>(), rp ? ctx->tgda.as<float>() : nullptr, ctx->trgb.as<float>(),
                              rp ? ctx->tdep.as<float>() : nullptr, rp ? ctx->talp.as<float>() : nullptr,
-                             ctx->gbuf.as<float>(), d_overflow, queue, ticket_g, st));
+                             ctx->gbuf.as<float>(), ctx->tconic.as<double>(), d_overflow, queue, ticket_g, st));
         CK(launch_param_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
                               ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.as<float>(), ctx->n,
-                              ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(), o.tgrad,
-                              st));
+                              ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(),
+                              ctx->tconic.as<double>(), o.tgrad, st));
         launches += 2;
     }
     if (o.score) {
@@ -844,7 +847,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
             CK(launch_blend_grad(rec, L, fgauss, ctx->ranges.as<int2>(), cp,
                                  ctx->gcoef.as<double>(), nullptr, nullptr,
                                  o.keep_rgb ? ctx->trgb.as<float>() : nullptr, nullptr, nullptr,
-                                 ctx->gbuf.as<float>(), d_overflow, queue, ticket_g, st));
+                                 ctx->gbuf.as<float>(), nullptr, d_overflow, queue, ticket_g, st));
             CK(launch_pose_chain(ctx->mean.as<float>(), ctx->mean.as<float>() + ctx->n,
                                  ctx->mean.as<float>() + 2 * ctx->n, ctx->attr.p, ctx->precision, ctx->n,
                                  ctx->gidx.as<uint32_t>(), L, sb.pblk, sb.d_views, cp, ctx->gbuf.as<float>(),
@@ -911,7 +914,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
     std::vector<SubBatch> sbs;
     int retries = 0, launches = 0;
     for (;;) {
-        plan_batches(ctx, qs, caps, cp, sbs);
+        plan_batches(ctx, qs, caps, cp, o.target ? 52 : o.grad ? 20 : 0, sbs);
         // ---- workspace: the largest sub-batch --------------------------------
         int64_t S_tot = 1, VS = 1, VI = 1, c1 = 1, cb = 1, V = 1, Qm = 1;
         size_t tab = 0;
@@ -946,7 +949,8 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         if (o.target) {
             CKS(ctx->trgb.ensure(12 * (size_t)V * HW));
             CKS(ctx->tgimg.ensure(12 * (size_t)V * HW));
-            CKS(ctx->gbuf.ensure(40 * (size_t)VS));
+            CKS(ctx->gbuf.ensure(28 * (size_t)VS));
+            CKS(ctx->tconic.ensure(24 * (size_t)VS));
             if (o.ssim_scale > 0 || o.rp_ssim_scale > 0) CKS(ctx->tabc.ensure(36 * (size_t)V * HW));
             if (o.rel) {
                 CKS(ctx->tdep.ensure(4 * (size_t)V * HW));

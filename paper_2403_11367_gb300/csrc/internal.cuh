@@ -268,14 +268,15 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // mean and conic.  gimg null: of the view's NCC (coef from K7), added into
 // gout[vd_off[v] + i][5] (u, v, a, b, c).  gimg [V][3][H][W] = dL/dC of an
 // image loss (gda [V][2][H][W] = dL/d(depth, alpha), may be null): added into
-// gout[vd_off[v] + i][10] (u, v, a, b, c, r, g, b, opacity, z).  cimg (may be
+// gconic[vd_off[v] + i][3] (a, b, c, FP64) and gout[vd_off[v] + i][7] (u, v, r, g, b,
+// opacity, z).  cimg (may be
 // null) [V][3][H][W]: the views' forward render (cdep, calp [V][H][W] its depth
 // and alpha, needed with gda), so the colour need not be composited again.
 // queue: the heavy tiles (launch_tile_count); ticket: zeroed before the call.
 cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
-                              const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st);
+                              double *gconic, const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st);
 
 // Chain of gin to each view's left pose update: out[V][6] (rho, phi);
 // part: n_blocks * V * 6 doubles of scratch.
@@ -301,11 +302,11 @@ cudaError_t launch_reproj_warp(const float *dep, const float *alp, const float *
                                cudaStream_t st);
 cudaError_t launch_reproj_back(const float *gw, const float *jac, const float *dep, const float *alp, int n_views,
                                int64_t HW, float alpha_min, float *gda, cudaStream_t st);
-// gin [VS][10] (launch_blend_grad, image mode) -> gmap [14][n_map] (added):
+// gin [VS][7], gconic [VS][3] (launch_blend_grad, image mode) -> gmap [14][n_map] (added):
 // mean xyz, scale xyz, quat wxyz, opacity, rgb.  FP32 attributes only.
 cudaError_t launch_param_chain(const float *mx, const float *my, const float *mz, const float *attr, int64_t n_map,
                                const uint32_t *gidx, const Layout &L, int n_blocks, const ViewParams *views,
-                               const CamParams &cam, const float *gin, float *gmap, cudaStream_t st);
+                               const CamParams &cam, const float *gin, const double *gconic, float *gmap, cudaStream_t st);
 struct AdamParams {
     float lr[5];          // mean, scale, quaternion, opacity, colour
     float beta1, beta2, eps, bc1, bc2, o_min;

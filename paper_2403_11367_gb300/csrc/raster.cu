@@ -869,6 +869,12 @@ cudaError_t launch_ncc_finalize(const double *partials, const double *qpart, con
 // IMG = true: G is given per pixel (gimg [V][3][H][W], an image loss's
 // gradient), and optionally G_D, G_A (gda [V][2][H][W]); ten outputs: also
 // dL/d colour = sum w G, dL/d opacity = dL/d power / o and dL/dz = sum w G_D.
+// There the conic's three sums over the warps go to FP64 entries (gconic): the chain
+// rule carries them through the inverse of Sigma', which multiplies the rounding of
+// FP32 sums, different in every order of the warps, by the condition number of a long
+// thin footprint.  Repeats of a 16-view driving gradient lay up to 4.6e-3 apart in
+// their worst element (2e-6 as a whole) with FP32 entries, 6e-6 so, for 5.38 -> 5.49
+// ms a step; all ten in FP64 took the same time and 28 bytes a record more.
 // cimg (may be null): the forward's render of the views ([V][3][H][W], in image
 // mode with cdep, calp [V][H][W] when gda is given) replaces the first walk.
 template <int TW, int TH, bool IMG>
@@ -877,7 +883,8 @@ __device__ __forceinline__ void blend_grad_unit(const Records &rec, const Layout
                                                 const double *__restrict__ coef, const float *__restrict__ gimg,
                                                 const float *__restrict__ gda, const float *__restrict__ cimg,
                                                 const float *__restrict__ cdep, const float *__restrict__ calp,
-                                                float *__restrict__ gout, int v, int unit, int2 r)
+                                                float *__restrict__ gout, double *__restrict__ gconic, int v, int unit,
+                                                int2 r)
 {
     constexpr int NOUT = IMG ? 10 : 5;
     constexpr int GRP = 30 / NOUT;              // records summed together
@@ -1066,24 +1073,39 @@ __device__ __forceinline__ void blend_grad_unit(const Records &rec, const Layout
     f32x2 K2 = pk(G[0][0] * C[0][0] + G[0][1] * C[0][1] + G[0][2] * C[0][2] + GDA[0][0] * DA[0][0] + GDA[0][1] * DA[0][1],
                   G[1][0] * C[1][0] + G[1][1] * C[1][1] + G[1][2] * C[1][2] + GDA[1][0] * DA[1][0] + GDA[1][1] * DA[1][1]);
 
-    // lane m adds up row m of the group and adds the total to its record's entry
+    // lane m adds up row m of the group and adds the total to its record's entry: a
+    // tree over the lanes' values (halves, quarters, ... of the row), whose rounding
+    // grows with five additions and not with the row's length
     int held = 0;                                // records in the group
-    float *const go = gout + NOUT * L.vd_off[v];
+    float *const go = gout + (IMG ? 7 : 5) * L.vd_off[v];
+    double *const gd = IMG ? gconic + 3 * L.vd_off[v] : nullptr;
     auto flush = [&]() {
         __syncwarp();
         if (lane < held * NOUT) {
-            f32x2 s0 = 0ull, s1 = 0ull;
+            f32x2 w[2][2];                       // lanes 4 h .. 4 h + 3 plus those 8, 16 and 24 on
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float4 t = *reinterpret_cast<const float4 *>(&s_t[lane][4 * q]);
-                s0 = add2(s0, pk(t.x, t.y));
-                s1 = add2(s1, pk(t.z, t.w));
+            for (int h = 0; h < 2; ++h) {
+                f32x2 e[2][2];
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const float4 a = *reinterpret_cast<const float4 *>(&s_t[lane][4 * h + 8 * k]);
+                    const float4 b = *reinterpret_cast<const float4 *>(&s_t[lane][4 * h + 8 * k + 16]);
+                    e[k][0] = add2(pk(a.x, a.y), pk(b.x, b.y));
+                    e[k][1] = add2(pk(a.z, a.w), pk(b.z, b.w));
+                }
+                w[h][0] = add2(e[0][0], e[1][0]);
+                w[h][1] = add2(e[0][1], e[1][1]);
             }
             float lo, hi;
-            upk(add2(s0, s1), lo, hi);
+            upk(add2(add2(w[0][0], w[1][0]), add2(w[0][1], w[1][1])), lo, hi);
             const float tot = lo + hi;
-            const int slot = lane / NOUT;
-            if (tot != 0.f) atomicAdd(go + NOUT * (int64_t)s_tg[slot] + (lane - NOUT * slot), tot);
+            const int slot = lane / NOUT, m = lane - NOUT * slot;
+            const int64_t g = s_tg[slot];
+            if (tot != 0.f) {
+                if (!IMG) atomicAdd(go + 5 * g + m, tot);
+                else if (m >= 2 && m < 5) atomicAdd(gd + 3 * g + (m - 2), (double)tot);
+                else atomicAdd(go + 7 * g + (m < 2 ? m : m - 3), tot);
+            }
         }
         __syncwarp();
         held = 0;
@@ -1174,14 +1196,14 @@ k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
              const int2 *__restrict__ ranges, CamParams cam, const double *__restrict__ coef,
              const float *__restrict__ gimg, const float *__restrict__ gda, const float *__restrict__ cimg,
              const float *__restrict__ cdep, const float *__restrict__ calp, float *__restrict__ gout,
-             const int *__restrict__ overflow, BlendQueue queue, int *__restrict__ ticket)
+             double *__restrict__ gconic, const int *__restrict__ overflow, BlendQueue queue, int *__restrict__ ticket)
 {
     constexpr int WPT = BlockGeom<TW, TH>::WPT;
     if (*overflow) return;
     if (!IMG) {
         const int2 r = ranges[(int64_t)blockIdx.y * cam.n_tiles + blockIdx.x / WPT];
         if (r.x < r.y)
-            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, blockIdx.y,
+            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, gconic, blockIdx.y,
                                          blockIdx.x, r);
         return;
     }
@@ -1203,7 +1225,7 @@ k_blend_grad(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
         const int v = (int)(u / upv), unit = (int)(u - (int64_t)v * upv);
         const int2 r = ranges[(int64_t)v * cam.n_tiles + unit / WPT];
         if (r.x < r.y && (listed || r.y - r.x < BLEND_HEAVY))
-            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, v, unit, r);
+            blend_grad_unit<TW, TH, IMG>(rec, L, inst_gauss, cam, coef, gimg, gda, cimg, cdep, calp, gout, gconic, v, unit, r);
         __syncwarp();
     }
 }
@@ -1212,30 +1234,31 @@ template <int TW, int TH>
 static cudaError_t blend_grad_t(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                                 const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                                 const float *cimg, const float *cdep, const float *calp, float *gout,
-                                const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
+                                double *gconic, const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
 {
     const int units = cam.n_tiles * (TW * TH / 64);             // per view
     if (gimg) {
         const int resident = blend_resident<k_blend_grad<TW, TH, true>>();
         if (resident <= 0) return cudaErrorInvalidValue;
         k_blend_grad<TW, TH, true><<<(unsigned)min64((int64_t)units * L.V, resident), 32, 0, st>>>(
-            rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep, calp, gout, overflow, queue, ticket);
+            rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep, calp, gout, gconic, overflow, queue, ticket);
     } else {
         k_blend_grad<TW, TH, false><<<dim3(units, L.V), 32, 0, st>>>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg,
-                                                                     nullptr, nullptr, gout, overflow, queue, ticket);
+                                                                     nullptr, nullptr, gout, nullptr, overflow, queue,
+                                                                     ticket);
     }
     return cudaGetLastError();
 }
 cudaError_t launch_blend_grad(Records rec, const Layout &L, const uint32_t *inst_gauss, const int2 *ranges,
                               const CamParams &cam, const double *coef, const float *gimg, const float *gda,
                               const float *cimg, const float *cdep, const float *calp, float *gout,
-                              const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
+                              double *gconic, const int *overflow, BlendQueue queue, int *ticket, cudaStream_t st)
 {
     if (L.V <= 0) return cudaSuccess;
 #define RELOC_GRAD_CASE(W_, H_) \
     if (cam.tile_w == W_ && cam.tile_h == H_) \
         return blend_grad_t<W_, H_>(rec, L, inst_gauss, ranges, cam, coef, gimg, gda, cimg, cdep, calp, gout, \
-                                    overflow, queue, ticket, st);
+                                    gconic, overflow, queue, ticket, st);
     RELOC_GRAD_CASE(16, 16)
     RELOC_GRAD_CASE(8, 8)
     RELOC_GRAD_CASE(32, 8)

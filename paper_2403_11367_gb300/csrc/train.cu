@@ -437,9 +437,9 @@ cudaError_t launch_reproj_back(const float *gw, const float *jac, const float *d
 }
 
 // --------------------------------------------------------- parameter chain --
-// gin holds, per (view, subset Gaussian), the gradients of the loss with
-// respect to the projected mean (u, v), the conic (a, b, c), the colour, the
-// opacity and the camera depth z = t_z (k_blend_grad, image mode).  A thread per subset Gaussian walks
+// gin and gconic hold, per (view, subset Gaussian), the gradients of the loss with
+// respect to the projected mean (u, v), the colour, the opacity and the camera
+// depth z = t_z, and to the conic (a, b, c) (k_blend_grad, image mode).  A thread per subset Gaussian walks
 // its query's views and carries them back through the projection (Sec. III-A:
 // Sigma' = J W Sigma W^T J^T + 0.3 I, conic = Sigma'^-1, t = W mu):
 //   dL/dSigma' = -A G_A A                       (G_A = [[ga, gb/2], [gb/2, gc]])
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(PROJ_THREADS)
 k_param_chain(const float *__restrict__ mx, const float *__restrict__ my, const float *__restrict__ mz,
               const float *__restrict__ attr, int64_t n_map, const uint32_t *__restrict__ gidx, Layout L,
               const ViewParams *__restrict__ views, CamParams cam, const float *__restrict__ gin,
-              float *__restrict__ gmap)
+              const double *__restrict__ gconic, float *__restrict__ gmap)
 {
     const int qi = find_segment(L.q_pblk, L.Q, (int)blockIdx.x);
     const int64_t S = L.q_gsub[qi + 1] - L.q_gsub[qi];
@@ -489,9 +489,10 @@ k_param_chain(const float *__restrict__ mx, const float *__restrict__ my, const 
     bool any = false;
     for (int vv = 0; vv < V; ++vv) {
         const int v = v_begin + vv;
-        const float *g10 = gin + 10 * (L.vd_off[v] + i);
-        const float gu = g10[0], gv = g10[1], ga = g10[2], gb = g10[3], gc = g10[4];
-        const float gr = g10[5], gg = g10[6], gbl = g10[7], go = g10[8], gz = g10[9];
+        const float *g7 = gin + 7 * (L.vd_off[v] + i);
+        const double *g3 = gconic + 3 * (L.vd_off[v] + i);
+        const float gu = g7[0], gv = g7[1], ga = (float)g3[0], gb = (float)g3[1], gc = (float)g3[2];
+        const float gr = g7[2], gg = g7[3], gbl = g7[4], go = g7[5], gz = g7[6];
         if (gu == 0.f && gv == 0.f && ga == 0.f && gb == 0.f && gc == 0.f && gr == 0.f && gg == 0.f &&
             gbl == 0.f && go == 0.f && gz == 0.f)
             continue;
@@ -597,10 +598,10 @@ k_param_chain(const float *__restrict__ mx, const float *__restrict__ my, const 
 
 cudaError_t launch_param_chain(const float *mx, const float *my, const float *mz, const float *attr, int64_t n_map,
                                const uint32_t *gidx, const Layout &L, int n_blocks, const ViewParams *views,
-                               const CamParams &cam, const float *gin, float *gmap, cudaStream_t st)
+                               const CamParams &cam, const float *gin, const double *gconic, float *gmap, cudaStream_t st)
 {
     if (n_blocks <= 0 || L.V <= 0) return cudaSuccess;
-    k_param_chain<<<n_blocks, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, gin, gmap);
+    k_param_chain<<<n_blocks, PROJ_THREADS, 0, st>>>(mx, my, mz, attr, n_map, gidx, L, views, cam, gin, gconic, gmap);
     return cudaGetLastError();
 }
 
