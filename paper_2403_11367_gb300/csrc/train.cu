@@ -8,44 +8,16 @@
 
 namespace reloc {
 
-// Sums of FP32 samples in pairs hi + lo: TwoSum (Knuth, The Art of Computer
-// Programming, volume 2, section 4.2.2) gives the exact rounding error of each
-// addition, and the errors are summed in lo.  A block's sum is then within 2^-47 of
-// itself, as many bits as the FP64 sum of FP32 samples can use here (the losses add
-// 10^4 such sums in FP64), at six FP32 instructions a sample instead of two on the
-// FP64 pipe, each of which holds a scheduler's share of it for about 60 cycles.
-struct PairSum {
-    float hi, lo;
-};
-__device__ __forceinline__ void pair_add(PairSum &a, float x)
-{
-    const float s = __fadd_rn(a.hi, x), b = __fsub_rn(s, a.hi);
-    a.lo = __fadd_rn(a.lo, __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    a.hi = s;
-}
-template <int LANES>
-__device__ __forceinline__ void pair_butterfly(PairSum &a)
+// FP64 total over a block of 256 threads, in thread 0.  s_sum: 8 entries.
+__device__ __forceinline__ double block_total(double a, double *s_sum)
 {
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) {
-        const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
-        pair_add(a, h);
-        a.lo = __fadd_rn(a.lo, l);
-    }
-}
-// an infinite or NaN sum is hi's alone (its error term is inf - inf)
-__device__ __forceinline__ double pair_value(PairSum a) { return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi; }
-// Total over a block of 256 threads, in thread 0.  s_pair: 8 entries; ends with
-// every thread past the barrier, so s_pair may be used again after another one.
-__device__ __forceinline__ double pair_block_total(PairSum a, PairSum *s_pair)
-{
-    pair_butterfly<32>(a);
-    if ((threadIdx.x & 31) == 0) s_pair[threadIdx.x >> 5] = a;
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = a;
     __syncthreads();
-    if (threadIdx.x >= 32) return 0.0;
-    a = s_pair[threadIdx.x & 7];
-    pair_butterfly<8>(a);
-    return threadIdx.x == 0 ? pair_value(a) : 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 1; w < 8; ++w) a += s_sum[w];
+    return a;
 }
 
 // ------------------------------------------------------------------ L1 -----
@@ -54,21 +26,14 @@ __device__ __forceinline__ double pair_block_total(PairSum a, PairSum *s_pair)
 // gimg.  One FP64 atomic per block.  Bound by memory: 12 bytes a sample.  With the
 // D-SSIM term on, k_ssim_bwd forms both instead.
 __device__ __forceinline__ float l1_slope(float d, float scale) { return d >= 0.f ? scale : -scale; }
-// loss += scale * sum |d| of a block of 256 threads, N differences each.  Magnitudes
-// that could leave FP32's range when summed, infinities and NaN go the FP64 way.
+// loss += scale * sum |d| of a block of 256 threads, N differences each, in FP64.
 template <int N>
-__device__ __forceinline__ void l1_block_add(const float (&d)[N], double scale, PairSum *s_pair, double *loss)
+__device__ __forceinline__ void l1_block_add(const float (&d)[N], double scale, double *s_sum, double *loss)
 {
-    PairSum acc = {0.f, 0.f};
+    double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < N; ++k) pair_add(acc, fabsf(d[k]));
-    if (__syncthreads_or(!(acc.hi < 1e30f))) {
-        double t = 0.0;
-        for (int k = 0; k < N; ++k) t += fabs((double)d[k]);
-        atomicAdd(loss, t * scale);
-        return;
-    }
-    const double t = pair_block_total(acc, s_pair);
+    for (int k = 0; k < N; ++k) acc += (double)fabsf(d[k]);
+    const double t = block_total(acc, s_sum);
     if (threadIdx.x == 0) atomicAdd(loss, t * scale);
 }
 
@@ -77,7 +42,7 @@ __global__ void __launch_bounds__(256)
 k_photo_l1(const float *__restrict__ rgb, const float *__restrict__ target, int64_t n, float scale, double dscale,
            float *__restrict__ gimg, double *__restrict__ loss)
 {
-    __shared__ PairSum s_pair[8];
+    __shared__ double s_sum[8];
     const int64_t base = (int64_t)blockIdx.x * (256 * L1_PER) + threadIdx.x;
     float d[L1_PER];
 #pragma unroll
@@ -90,7 +55,7 @@ k_photo_l1(const float *__restrict__ rgb, const float *__restrict__ target, int6
         const int64_t i = base + 256 * k;
         if (i < n) gimg[i] = l1_slope(d[k], scale);
     }
-    l1_block_add(d, dscale, s_pair, loss);
+    l1_block_add(d, dscale, s_sum, loss);
 }
 
 cudaError_t launch_photo_l1(const float *rgb, const float *target, int64_t n, double scale, float *gimg, double *loss,
@@ -176,7 +141,7 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
 {
     __shared__ float sin_[2][SS_H * SS_IN_STRIDE];
     __shared__ float hsum[5][SS_H * SS_H_STRIDE];
-    __shared__ PairSum s_pair[SS_THREADS / 32];
+    __shared__ double s_sum[SS_THREADS / 32];
     const int64_t HW = (int64_t)H * W;
     const int plane = blockIdx.z;
     const int x0 = blockIdx.x * SS_T, y0 = blockIdx.y * SS_T;
@@ -226,7 +191,7 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
             q[m][o] = acc;
         }
     }
-    PairSum contrib = {0.f, 0.f};
+    double contrib = 0.0;
     const int gx = x0 + col;
 #pragma unroll
     for (int o = 0; o < SS_OUT; ++o) {
@@ -244,11 +209,10 @@ k_ssim_fwd(const float *__restrict__ x_img, const float *__restrict__ y_img, int
             po[0] = -scale * d_m;
             po[HW] = -scale * d_xx;
             po[2 * HW] = -scale * d_xy;
-            pair_add(contrib, 1.f);                     // 1 - s, exactly
-            pair_add(contrib, -s);
+            contrib += 1.0 - (double)s;
         }
     }
-    const double t = pair_block_total(contrib, s_pair);
+    const double t = block_total(contrib, s_sum);
     if (threadIdx.x == 0) atomicAdd(loss, t * dscale);
 }
 
@@ -260,7 +224,7 @@ __global__ void __launch_bounds__(SS_THREADS)
 k_ssim_bwd(const float *__restrict__ abc, const float *__restrict__ x_img, const float *__restrict__ y_img, int H,
            int W, SsimWin win, float l1_scale, double l1_dscale, float *__restrict__ gimg, double *__restrict__ loss)
 {
-    __shared__ PairSum s_pair[SS_THREADS / 32];
+    __shared__ double s_sum[SS_THREADS / 32];
     __shared__ float sin_[3][SS_H * SS_IN_STRIDE];
     __shared__ float hsum[3][SS_H * SS_H_STRIDE];
     const int64_t HW = (int64_t)H * W;
@@ -314,7 +278,7 @@ k_ssim_bwd(const float *__restrict__ abc, const float *__restrict__ x_img, const
             gimg[pix] = l1_slope(dif[o], l1_scale) + (q[0][o] + 2.f * x * q[1][o] + y * q[2][o]);
         }
     }
-    l1_block_add(dif, l1_dscale, s_pair, loss);
+    l1_block_add(dif, l1_dscale, s_sum, loss);
 }
 
 cudaError_t launch_ssim(const float *rgb, const float *target, int planes, int H, int W, double l1_scale, double scale,
