@@ -388,9 +388,11 @@ __global__ void __launch_bounds__(PNP_THREADS) k_refine_pnp(PnpArgs a)
             sq = s_tot[PA_SQ];
             cnt = s_tot[PA_CNT];
             if (threadIdx.x < 12) s_pose[threadIdx.x] = s_trial[take][threadIdx.x];
-            __syncthreads();
+            // read before the barrier: after it the first warp may write the next step
+            // already, and a warp that judged by that one could leave alone
             double dmax = 0.0;
             for (int j = 0; j < 6; ++j) dmax = fmax(dmax, fabs(step * s_delta[j]));
+            __syncthreads();
             if (dmax < a.tol) {
                 ++it;
                 break;
