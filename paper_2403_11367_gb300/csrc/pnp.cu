@@ -39,6 +39,7 @@
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
+#include "newton.h"
 
 namespace reloc {
 
@@ -85,22 +86,18 @@ __device__ __forceinline__ double warp_sums(double (&v)[N], int lane)
 // Whether x lies where its FP32 value can seed Newton's iteration (NaN: no).
 __device__ __forceinline__ bool seeds(double x) { return x > 1e-36 && x < 1e36; }
 
-// 1 / x for x > 0: FP32 seed (relative error 2^-23), two Newton steps.
+// 1 / x for x > 0: FP32 seed (relative error 2^-23), two Newton steps; rounded once.
 __device__ __forceinline__ double recip(double x)
 {
     if (!seeds(x)) return 1.0 / x;
-    double r = (double)__frcp_rn((float)x);
-    r = fma(fma(-x, r, 1.0), r, r);
-    return fma(fma(-x, r, 1.0), r, r);
+    return newton_recip(x, (double)__frcp_rn((float)x));
 }
 
-// 1 / sqrt(x) for x > 0: FP32 seed, two Newton steps.
+// 1 / sqrt(x) for x > 0: FP32 seed, two Newton steps; rounded once.
 __device__ __forceinline__ double rsqrt_newton(double x)
 {
     if (!seeds(x)) return 1.0 / sqrt(x);
-    double r = (double)rsqrtf((float)x);
-    r = fma(fma(-x * r, r, 1.0), 0.5 * r, r);
-    return fma(fma(-x * r, r, 1.0), 0.5 * r, r);
+    return newton_rsqrt(x, (double)rsqrtf((float)x));
 }
 
 // Huber cost of a squared residual and its weight (1, or k / e beyond k).
