@@ -224,7 +224,7 @@ cudaError_t configure_sort_kernels();
 
 // Pose refinement by PnP on one view's depth (pnp.cu), one cooperative launch:
 // out[20] = pose[16], rms, cost, n_used, iterations (device or pinned host
-// memory); X_scratch: 4 doubles per pair, then per-block sums (under 256 KB).
+// memory); X_scratch: 6 doubles per pair, then per-block sums (under 256 KB).
 cudaError_t launch_refine_pnp(const double *pose_render, const double *pose_init, double fx, double fy, double cx,
                               double cy, int width, int height, const float *depth, const float *alpha,
                               const float *pairs, int n, int max_iters, double huber, double alpha_min, double tol,

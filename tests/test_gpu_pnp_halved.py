@@ -37,9 +37,9 @@ def cost(W, X, q, cam, k=2.0):
     return np.where(e <= k, 0.5 * e * e, k * (e - 0.5 * k)).sum(), P, r, e
 
 
-def gauss_newton(W, X, q, cam, k=2.0):
-    """(step, condition number of the system, cost at W)."""
-    c, P, r, e = cost(W, X, q, cam, k)
+def system(W, X, q, cam, k=2.0):
+    """Normal equations (H, g) of the Huber cost at W."""
+    _, P, r, e = cost(W, X, q, cam, k)
     x, y, z = P.T
     o = np.zeros_like(x)
     Jp = np.stack([np.stack([cam.fx / z, o, -cam.fx * x / z ** 2], 1), np.stack([o, cam.fy / z, -cam.fy * y / z ** 2], 1)], 1)
@@ -47,9 +47,18 @@ def gauss_newton(W, X, q, cam, k=2.0):
                   np.stack([o, o, o + 1, y, -x, o], 1)], 1)
     J = Jp @ M
     w = np.where(e <= k, 1.0, k / np.maximum(e, 1e-300))
-    H, g = np.einsum("n,nra,nrb->ab", w, J, J), np.einsum("n,nra,nr->a", w, J, r)
-    H += 1e-9 * np.trace(H) / 6 * np.eye(6)
-    return np.linalg.solve(H, -g), np.linalg.cond(H), c
+    return np.einsum("n,nra,nrb->ab", w, J, J), np.einsum("n,nra,nr->a", w, J, r)
+
+
+def gradient(W, X, q, cam):
+    return system(W, X, q, cam)[1]
+
+
+def gauss_newton(W, X, q, cam, k=2.0):
+    """(step, condition number of the system, cost at W)."""
+    H, g = system(W, X, q, cam, k)
+    H = H + 1e-9 * np.trace(H) / 6 * np.eye(6)
+    return np.linalg.solve(H, -g), np.linalg.cond(H), cost(W, X, q, cam, k)[0]
 
 
 def problem():
