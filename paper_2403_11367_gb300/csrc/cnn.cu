@@ -68,10 +68,12 @@ cudaError_t launch_downsample_gray(const GrayQueries &q, const float *render, in
 
 // im2col for a 3x3 / stride 2 / pad 1 convolution: X [B][H][W][C] ->
 // col [B*Ho*Wo][Kp], zero beyond K = 9 C.  A thread writes eight columns, 16
-// bytes: eight channels of one tap, or for the two-channel input four taps.
+// bytes: eight channels of one tap, or for the two-channel input four taps, each one
+// 4-byte load (PAIR) or, of a caller's buffer off 4 bytes, two 2-byte loads.
 // Bound by its writes (211 MB for the five layers at batch 256; one value a
 // thread took 650 us there).
 constexpr int COL_THREADS = 256;
+template <bool PAIR>
 __global__ void __launch_bounds__(COL_THREADS)
 k_im2col(const __nv_bfloat16 *__restrict__ x, int M, int H, int W, int C, int Ho, int Wo, int Kp,
          __nv_bfloat16 *__restrict__ col)
@@ -89,8 +91,11 @@ k_im2col(const __nv_bfloat16 *__restrict__ x, int M, int H, int W, int C, int Ho
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int tap = 4 * g + j, y = 2 * oy - 1 + tap / 3, xx = 2 * ox - 1 + tap % 3;
-            if (tap < 9 && y >= 0 && y < H && xx >= 0 && xx < W)
-                w[j] = *reinterpret_cast<const uint32_t *>(xb + ((int64_t)y * W + xx) * 2);
+            if (tap < 9 && y >= 0 && y < H && xx >= 0 && xx < W) {
+                const __nv_bfloat16 *p = xb + ((int64_t)y * W + xx) * 2;
+                w[j] = PAIR ? *reinterpret_cast<const uint32_t *>(p)
+                            : (uint32_t)__bfloat16_as_ushort(p[0]) | (uint32_t)__bfloat16_as_ushort(p[1]) << 16;
+            }
         }
         v = make_uint4(w[0], w[1], w[2], w[3]);
     } else {
@@ -102,13 +107,15 @@ k_im2col(const __nv_bfloat16 *__restrict__ x, int M, int H, int W, int C, int Ho
     *reinterpret_cast<uint4 *>(col + row64 * Kp + 8 * g) = v;
 }
 
-// C 2 or a multiple of 8; Kp a multiple of 8, at most 8 * 256; x on 4 (C = 2) or 16 bytes.
+// C 2 or a multiple of 8; Kp a multiple of 8, at most 8 * 256; x on 2 (C = 2) or 16 bytes.
 cudaError_t launch_im2col(const __nv_bfloat16 *x, int B, int H, int W, int C, int Ho, int Wo, int Kp,
                           __nv_bfloat16 *col, cudaStream_t st)
 {
-    if ((C != 2 && C % 8) || Kp % 8 || Kp / 8 > COL_THREADS) return cudaErrorInvalidValue;
+    if ((C != 2 && (C % 8 || ((uintptr_t)x & 15))) || Kp % 8 || Kp / 8 > COL_THREADS) return cudaErrorInvalidValue;
     const int M = B * Ho * Wo;
-    k_im2col<<<(unsigned)ceil_div(M, COL_THREADS / (Kp / 8)), COL_THREADS, 0, st>>>(x, M, H, W, C, Ho, Wo, Kp, col);
+    const unsigned grid = (unsigned)ceil_div(M, COL_THREADS / (Kp / 8));
+    if (((uintptr_t)x & 3) == 0) k_im2col<true><<<grid, COL_THREADS, 0, st>>>(x, M, H, W, C, Ho, Wo, Kp, col);
+    else k_im2col<false><<<grid, COL_THREADS, 0, st>>>(x, M, H, W, C, Ho, Wo, Kp, col);
     return cudaGetLastError();
 }
 
