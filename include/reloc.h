@@ -286,7 +286,7 @@ reloc_status reloc_localize_host(reloc_ctx *ctx, const float *query_host, const 
  * -> refine is the paper's refinement loop.
  *   depth_dev, alpha_dev  [H][W] float32, device: Eq. (depth) D and
  *                         1 - T of the view (caller-owned)
- *   pairs_dev             [n_pairs][4] float32, device: (u_r, v_r, u_q, v_q)
+ *   pairs_dev             [n_pairs][4] float32, device, 16-byte aligned: (u_r, v_r, u_q, v_q)
  *                         pixel coordinates, pixel (x, y) centred at
  *                         (x + 0.5, y + 0.5)
  *   pose_init             world-to-camera start (typically pose_render)
@@ -300,7 +300,7 @@ reloc_status reloc_localize_host(reloc_ctx *ctx, const float *query_host, const 
  * solves (H + 1e-9 tr(H)/6 I) delta = -g, W <- [Exp(phi) R | Exp(phi) t +
  * rho]; a step that does not lower the cost is halved up to 10 times, then
  * the solve stops; it also stops when max |delta| < tol or after max_iters.
- * Errors: EINVAL (NULL pointer, n_pairs < 1, bad options), ENUMERIC
+ * Errors: EINVAL (NULL pointer, n_pairs < 1, pairs_dev off 16 bytes, bad options), ENUMERIC
  * (non-finite pose or fewer than 3 usable pairs), ECUDA. */
 typedef struct reloc_pnp_options {
     int32_t max_iters;         /* default 30                                          */

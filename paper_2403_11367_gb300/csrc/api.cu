@@ -1819,6 +1819,7 @@ extern "C" reloc_status reloc_refine_pnp(reloc_ctx *ctx, const double *pose_rend
     if (!ctx || !pose_render || !pose_init || !cam || !depth_dev || !alpha_dev || !pairs_dev || !out)
         return fail(RELOC_EINVAL, "NULL argument");
     if (n_pairs < 1) return fail(RELOC_EINVAL, "n_pairs %d < 1", n_pairs);
+    if ((uintptr_t)pairs_dev & 15) return fail(RELOC_EINVAL, "pairs_dev needs 16-byte alignment");
     if (cam->width < 2 || cam->height < 2 || cam->width > 16383 || cam->height > 16383)
         return fail(RELOC_EINVAL, "image size %dx%d out of range", cam->width, cam->height);
     if (!(cam->fx > 0) || !(cam->fy > 0) || !std::isfinite(cam->cx) || !std::isfinite(cam->cy))
