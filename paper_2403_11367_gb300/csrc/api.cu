@@ -61,9 +61,13 @@ reloc_status fail(reloc_status st, const char *fmt, ...)
         if (s_ != RELOC_OK) return s_;                                                                  \
     } while (0)
 
+// Device memory that grows on demand and is released with its owner.
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    DevBuf() = default;
+    DevBuf(const DevBuf &) = delete;
+    ~DevBuf() { release(); }
     reloc_status ensure(size_t n)
     {
         if (n <= bytes && p) return RELOC_OK;
@@ -90,9 +94,13 @@ struct DevBuf {
     template <typename T> T *as() const { return (T *)p; }
 };
 
+// The same of pinned host memory.
 struct PinBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    PinBuf() = default;
+    PinBuf(const PinBuf &) = delete;
+    ~PinBuf() { release(); }
     reloc_status ensure(size_t n)
     {
         if (n <= bytes && p) return RELOC_OK;
@@ -284,19 +292,7 @@ extern "C" reloc_status reloc_destroy(reloc_ctx *ctx)
 {
     if (!ctx) return RELOC_OK;
     cudaSetDevice(ctx->device);
-    DevBuf *bufs[] = {&ctx->mean, &ctx->attr, &ctx->gidx, &ctx->tables, &ctx->rec, &ctx->rect,
-                      &ctx->dkey, &ctx->kva, &ctx->v1b, &ctx->hist1, &ctx->dtot, &ctx->chunk_sums,
-                      &ctx->srect, &ctx->bhist, &ctx->inst, &ctx->ranges, &ctx->partials,
-                      &ctx->qpart, &ctx->res, &ctx->view_sel, &ctx->bqueue, &ctx->hq, &ctx->hrgb,
-                      &ctx->hdepth, &ctx->prop_in, &ctx->prop_seed, &ctx->prop_logits, &ctx->prop_idx,
-                      &ctx->prop_mrg, &ctx->pnp_X, &ctx->gbuf, &ctx->gcoef,
-                      &ctx->gpart, &ctx->gpose, &ctx->tconic};
-    for (DevBuf *b : bufs) b->release();
     if (ctx->prop) proposal_destroy(ctx->prop);
-    ctx->pin.release();
-    ctx->gemm_status.release();
-    ctx->pnp_out.release();
-    ctx->prop_loss.release();
     for (auto &e : ctx->ev)
         if (e) cudaEventDestroy(e);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
