@@ -553,6 +553,7 @@ struct CallOut {
 // A run of consecutive queries whose workspace fits the memory budget.
 struct SubBatch {
     int q0 = 0, q1 = 0, v0 = 0, v1 = 0;
+    int64_t bytes = 0;                                  // workspace (query_bytes)
     int64_t S_tot = 0, S_max = 0, VS = 0, VI = 0;      // S_max: the longest view's Gaussians
     int c1 = 0, cb = 0, cb_view = 0, pblk = 0, n_runs = 0;     // cb_view: binning chunks of the longest view
     std::vector<int32_t> view_q, c1_base, cb_base, q_view, q_pblk;
@@ -608,6 +609,7 @@ static void plan_batches(const reloc_ctx *ctx, const std::vector<QuerySpec> &qs,
             vglob += qs[q].V;
             ++q;
         }
+        sb.bytes = bytes;
         sb.q1 = q;
         sb.v1 = vglob;
         const int nq = sb.q1 - sb.q0, nv = sb.v1 - sb.v0;
@@ -691,7 +693,8 @@ static void stage_tables(SubBatch &sb, char *host, char *dev)
     sb.d_views = (const ViewParams *)put(sb.views.data(), sizeof(ViewParams) * (size_t)nv);
 }
 
-// A sub-batch's renders kept for its pose gradients, up to a bound on the memory.
+// A sub-batch's renders kept for its pose gradients, up to a bound on the memory; without
+// them the backward walk composites each view once more.
 constexpr int64_t GRAD_IMAGE_MAX = (int64_t)1 << 30;
 
 static void stage_mark(reloc_ctx *ctx, int sbi, int s, cudaStream_t st, bool capturing)
@@ -914,9 +917,11 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         // ---- workspace: the largest sub-batch --------------------------------
         int64_t S_tot = 1, VS = 1, VI = 1, c1 = 1, cb = 1, V = 1, Qm = 1;
         size_t tab = 0;
+        int64_t work = 0;               // bytes of the largest sub-batch's workspace
         bool passes = false;            // a sub-batch whose depth sort takes a launch chain per pass
         for (auto &sb : sbs) {
             passes = passes || sb.S_max > DEPTH_SORT_CLUSTER_MAX;
+            work = std::max(work, sb.bytes);
             S_tot = std::max(S_tot, sb.S_tot);
             VS = std::max(VS, sb.VS);
             VI = std::max(VI, sb.VI);
@@ -962,8 +967,6 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             for (auto &sb : sbs) pb = std::max<int64_t>(pb, (int64_t)sb.pblk * (sb.v1 - sb.v0));
             CKS(ctx->gbuf.ensure(20 * (size_t)VS));
             CKS(ctx->gcoef.ensure(32 * (size_t)V));
-            o.keep_rgb = 12 * V * HW <= GRAD_IMAGE_MAX;
-            if (o.keep_rgb) CKS(ctx->trgb.ensure(12 * (size_t)V * HW));
             CKS(ctx->gpart.ensure(48 * (size_t)pb));
         }
         CKS(ctx->qpart.ensure(16 * QS_BLOCKS * (size_t)Qm));
@@ -973,6 +976,13 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         result_block(ctx->res.as<char>(), Vtot, Q, (int64_t)sbs.size(), &ctx->res_at);
         CKS(ctx->bqueue.ensure(4 * (size_t)blend_list_ints(cp, std::max<int64_t>(V, Qm))));
         CKS(ctx->tables.ensure(tab));
+        // the render kept for the pose gradients, after all that the call needs: where it
+        // fits the memory budget beside the workspace, and if the memory is to be had
+        if (o.grad) {
+            const int64_t image = 12 * V * HW;
+            o.keep_rgb = image <= std::min(GRAD_IMAGE_MAX, ctx->mem_budget - work) &&
+                         ctx->trgb.ensure((size_t)image) == RELOC_OK;
+        }
         // pinned staging: tables, then readback
         const size_t rb_off = align256(tab);
         CKS(ctx->pin.ensure(rb_off + res_bytes));
