@@ -52,7 +52,10 @@ reloc_status fail(reloc_status st, const char *fmt, ...)
 #define CK(call)                                                                                        \
     do {                                                                                                \
         cudaError_t e_ = (call);                                                                        \
-        if (e_ != cudaSuccess) return fail(RELOC_ECUDA, "%s: %s", #call, cudaGetErrorString(e_));       \
+        if (e_ != cudaSuccess) {                                                                        \
+            cudaGetLastError();      /* a refused launch leaves it set: the next call would report it */ \
+            return fail(RELOC_ECUDA, "%s: %s", #call, cudaGetErrorString(e_));                          \
+        }                                                                                               \
     } while (0)
 
 #define CKS(call)                                                                                       \
@@ -1024,6 +1027,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             for (size_t k = 0; k < sbs.size() && rs == RELOC_OK; ++k)
                 rs = enqueue_subbatch(ctx, sbs[k], (int)k, cp, o, st, true, launches);
             cudaError_t ce_ = cudaStreamEndCapture(st, &g);
+            if (ce_ != cudaSuccess) cudaGetLastError();
             if (rs != RELOC_OK) {
                 if (g) cudaGraphDestroy(g);
                 return rs;
