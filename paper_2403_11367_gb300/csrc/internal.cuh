@@ -254,8 +254,15 @@ inline int blend_units(const CamParams &cam) { return cam.n_tiles * (cam.tile_w 
 // entries stay far inside int32.  Sub-batches are cut to respect it.
 constexpr int64_t BLEND_MAX_UNITS = (int64_t)1 << 29;
 inline int64_t blend_list_ints(const CamParams &cam, int64_t n) { return n * cam.n_tiles; }
-// Image launches of fewer views take half blocks.
-constexpr int BLEND_HALF_VIEWS = 4;
+// Image launches of at most this many 64-pixel blocks take half blocks: two to each of
+// the 28 x 152 resident warps of the whole-block form.  Fewer end on their longest lists,
+// more are bound by their instructions, which half blocks raise.  Whole -> half, us: a
+// street's view at 1408 x 376 (8,448 blocks) 98 -> 84, four at 704 x 188 (8,448) 166 ->
+// 131, sixteen at 352 x 94 (8,448) 357 -> 272; past the line two views at 1408 x 376
+// (16,896) 115 -> 137, one at 2816 x 752 (33,088) 132 -> 193, at 5632 x 1504 366 -> 633.
+// Sparse maps gain less and lose a little at the line (one object: 352 x 94 31 -> 21,
+// 704 x 188 26 -> 27, 1408 x 376 37 -> 41).
+constexpr int64_t BLEND_HALF_UNITS = 2 * 28 * 152;
 inline int blend_launches(bool selected) { return selected ? 2 : 1; }
 
 // K7: NCC per view from its n_units partials and its query's partial sums

@@ -438,7 +438,7 @@ __device__ __forceinline__ void blend_unit(const Records &rec, const Layout &L,
 }
 
 // Half of a 64-pixel block (its left or right columns), a pixel to a lane: image
-// launches of few views, where the SMs run out of units before the longest lists
+// launches of few blocks (BLEND_HALF_UNITS), where the SMs run out of units before the longest lists
 // end.  Half a block's record takes 22 instructions instead of 33 and half a block
 // keeps fewer of them, so the last units end sooner; all units together take more
 // (every record is tested twice).  One view of a driving map (653,141 list entries,
@@ -612,7 +612,7 @@ __global__ void k_blend_heavy(const int2 *__restrict__ ranges, const int *__rest
     if (r.y - r.x >= BLEND_HEAVY) queue.list[atomicAdd(queue.count + 1, 1)] = (int)i;
 }
 
-// HALF: units of half a block (image launches of few views, no NCC).
+// HALF: units of half a block (image launches of few blocks, no NCC).
 template <int TW, int TH, int RPL, bool DA, bool HALF>
 __global__ void __launch_bounds__(32, HALF ? 16 : RPL == 1 ? (DA ? 28 : 32) : 24)
 k_blend(Records rec, Layout L, const uint32_t *__restrict__ inst_gauss,
@@ -728,11 +728,8 @@ static cudaError_t blend_t(Records rec, const Layout &L, const uint32_t *inst_ga
                               cam, partials, rgb, depth, alpha, view_sel, nv, overflow, queue);
     };
     const bool da = depth || alpha;
-    // Image launches that end on their longest lists take half blocks (the figures are
-    // blend_half's); from four views on a launch is bound by its instructions, which
-    // half blocks raise.
     if constexpr (RPL == 1) {
-        if (!partials && nv < BLEND_HALF_VIEWS)
+        if (!partials && units <= BLEND_HALF_UNITS)
             return da ? run(k_blend<TW, TH, 1, true, true>, blend_resident<k_blend<TW, TH, 1, true, true>>(), 2 * units)
                       : run(k_blend<TW, TH, 1, false, true>, blend_resident<k_blend<TW, TH, 1, false, true>>(), 2 * units);
     }
