@@ -190,6 +190,7 @@ struct reloc_ctx {
     int64_t adam_t = 0;
     PinBuf pin, gemm_status, pnp_out, prop_loss;
     double inst_ratio = 3.0;        // instance capacity per (view, subset Gaussian), learned
+    double vis_ratio = 1.0 / 3.0;   // visible share of the (view, subset Gaussian) pairs, the last call's
     // batch options
     int use_graph = 1;
     int64_t mem_budget = (int64_t)16 << 30;
@@ -558,6 +559,7 @@ struct SubBatch {
     int q0 = 0, q1 = 0, v0 = 0, v1 = 0;
     int64_t bytes = 0;                                  // workspace (query_bytes)
     int64_t S_tot = 0, S_max = 0, VS = 0, VI = 0;      // S_max: the longest view's Gaussians
+    bool sort_cluster = true;                           // depth sort in one cluster launch, else a chain of passes
     int c1 = 0, cb = 0, cb_view = 0, pblk = 0, n_runs = 0;     // cb_view: binning chunks of the longest view
     std::vector<int32_t> view_q, c1_base, cb_base, q_view, q_pblk;
     std::vector<int64_t> vd_off, io_off, q_gsub, run_begin, run_off;
@@ -727,7 +729,7 @@ static reloc_status enqueue_subbatch(reloc_ctx *ctx, SubBatch &sb, int sbi, cons
         launches += 1;
     }
     stage_mark(ctx, sbi, RELOC_STAGE_DEPTH_SORT, st, capturing);
-    if (sb.c1 > 0 && sb.S_max <= DEPTH_SORT_CLUSTER_MAX) {
+    if (sb.c1 > 0 && sb.sort_cluster) {
         // the rectangles in depth order are written after the sort: their buffer serves as scratch
         CK(launch_depth_sort(ctx->dkey.as<uint32_t>(), ctx->kva.as<uint2>(), ctx->srect.as<uint2>(),
                              ctx->v1b.as<uint32_t>(), L, sb.S_max, nvis, st));
@@ -923,7 +925,11 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
         int64_t work = 0;               // bytes of the largest sub-batch's workspace
         bool passes = false;            // a sub-batch whose depth sort takes a launch chain per pass
         for (auto &sb : sbs) {
-            passes = passes || sb.S_max > DEPTH_SORT_CLUSTER_MAX;
+            // few views end with the longest; many fill the GPU, and their sum counts
+            const int nv = sb.v1 - sb.v0;
+            const double S = nv > 32 ? (double)sb.VS / nv : (double)sb.S_max;
+            sb.sort_cluster = sb.S_max <= DEPTH_SORT_CLUSTER_MAX && ctx->vis_ratio * S <= DEPTH_SORT_CLUSTER_VISIBLE;
+            passes = passes || !sb.sort_cluster;
             work = std::max(work, sb.bytes);
             S_tot = std::max(S_tot, sb.S_tot);
             VS = std::max(VS, sb.VS);
@@ -1079,6 +1085,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
                 ctx->counts.n_visible += h_nvis[v];
                 ctx->counts.n_instances += h_ninst[v];
             }
+            if (pairs > 0) ctx->vis_ratio = (double)ctx->counts.n_visible / (double)pairs;
             ctx->counts.inst_stride = sbs[0].io_off.size() > 1 ? sbs[0].io_off[1] - sbs[0].io_off[0] : 0;
             ctx->counts.retries = retries;
             ctx->counts.kernel_launches = launches;

@@ -165,12 +165,16 @@ cudaError_t launch_project(const float *mx, const float *my, const float *mz, co
 // per (view, Gaussian); longest: the most Gaussians of one view.
 cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, const Layout &L,
                               int64_t longest, uint32_t *n_vis, cudaStream_t st);
-// Calls with a view of more Gaussians than this take the passes below, one launch
-// chain each, over the whole GPU.  The line lies where a driving view sees about
-// a third of its subset: 64 views of 320k Gaussians (100k visible) 278 us in
-// clusters, 470 in passes; 64 views of 500k with 270k visible 928 and 819; one
-// view of 500k with 443k visible 110 and 82; of 2M with 1.8M visible 369 and 155.
+// Sub-batches whose longest view has more Gaussians, or whose views are expected to see
+// more (by the visible share of the context's last call), take the passes below, one
+// launch chain each, over the whole GPU.  A cluster's time goes with the visible ones, a
+// chain's with all (chain / cluster, us).  One view: 320k all visible 80 / 79, 512k half
+// 77 / 78, all 84 / 118, 1M a third 96 / 111.  16 views: 256k all 194 / 207, 512k half 246 /
+// 241, all 326 / 423.  64 views: 320k a third (driving) 454 / 262, 512k half 798 / 708, all
+// 1122 / 1794.  A batch of 334 driving views (370k on average, 639k at most, 41% visible):
+// 21.4 / 20.5 ms the whole call.
 constexpr int64_t DEPTH_SORT_CLUSTER_MAX = (int64_t)1 << 20;
+constexpr double DEPTH_SORT_CLUSTER_VISIBLE = 262144.0;
 
 // Stable LSD radix sort pass over segments (views).  Segment s holds
 // seg_off[s+1] - seg_off[s] slots at seg_off[s], of which len[s] are valid

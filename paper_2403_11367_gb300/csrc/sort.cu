@@ -259,8 +259,8 @@ cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, ui
 }
 
 // --------------------------------------- depth sort, launches per pass -----
-// For views of more than DEPTH_SORT_CLUSTER_MAX Gaussians, whose passes need
-// the whole GPU: upsweep, digit offsets and scatter over SORT_CHUNK items a
+// For views of more Gaussians than a cluster suits (DEPTH_SORT_CLUSTER_VISIBLE),
+// whose passes need the whole GPU: upsweep, digit offsets and scatter over SORT_CHUNK items a
 // block.
 // Per chunk digit counts -> hist[s][d][k] (digit-major inside a segment, so
 // one exclusive scan of the segment's block gives every chunk's offsets).
