@@ -20,6 +20,8 @@
 // Every per-view array sits at a host-planned offset with a host-planned
 // capacity, and chunk tables map a block to its view and chunk, so valid
 // lengths stay in device memory: no host round trip between stages.
+#include <atomic>
+
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
@@ -241,6 +243,36 @@ k_depth_sort(const uint32_t *__restrict__ dkey, uint2 *bufA, uint2 *bufB, uint32
     depth_sort_pass<NW, false, true>(sm, n, 24, nullptr, A, nullptr, out + off);
 }
 
+// Blocks of the largest cluster of k_depth_sort<NW> that the current device can place
+// (16 is beyond the portable 8; a device with fewer usable SMs in its GPCs takes less), 0
+// on error; asked once per device.
+template <int NW>
+static int depth_sort_cluster()
+{
+    static std::atomic<int> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int c = cached[dev].load();
+    for (int C = DS_MAX_CLUSTER; !c && C >= 1; C /= 2) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = C;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(32 * NW);
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_depth_sort<NW>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        if (n > 0) cached[dev].store(c = C);
+    }
+    return c;
+}
+
 cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, uint32_t *out, const Layout &L,
                               int64_t longest, uint32_t *n_vis, cudaStream_t st)
 {
@@ -249,13 +281,15 @@ cudaError_t launch_depth_sort(const uint32_t *dkey, uint2 *bufA, uint2 *bufB, ui
     // half of it once the views alone fill the GPU: 64 driving views 278 us at 8
     // blocks, 339 at 16, 298 at 4; 16 views 153 at 16, 168 at 8; one view 50 at
     // 16, 77 at 8; a view of 10k keys 27 at 8, 35 at 2
-    const int most = L.V <= 32 ? DS_MAX_CLUSTER : DS_MAX_CLUSTER / 2;
+    const bool wide = L.V <= DS_WIDE_VIEWS;
+    const int fits = wide ? depth_sort_cluster<32>() : depth_sort_cluster<16>();
+    if (fits <= 0) return cudaErrorInvalidConfiguration;
+    const int most = min(fits, L.V <= 32 ? DS_MAX_CLUSTER : DS_MAX_CLUSTER / 2);
     int C = 1;
     while (C < most && (int64_t)C * 2048 < longest) C *= 2;
     const dim3 grid((unsigned)(C * L.V));
-    return L.V <= DS_WIDE_VIEWS
-               ? launch_chained(k_depth_sort<32>, grid, dim3(1024), 0, st, C, dkey, bufA, bufB, out, L, n_vis)
-               : launch_chained(k_depth_sort<16>, grid, dim3(512), 0, st, C, dkey, bufA, bufB, out, L, n_vis);
+    return wide ? launch_chained(k_depth_sort<32>, grid, dim3(1024), 0, st, C, dkey, bufA, bufB, out, L, n_vis)
+                : launch_chained(k_depth_sort<16>, grid, dim3(512), 0, st, C, dkey, bufA, bufB, out, L, n_vis);
 }
 
 // --------------------------------------- depth sort, launches per pass -----
@@ -1089,6 +1123,7 @@ cudaError_t configure_sort_kernels()
     cudaError_t e = cudaFuncSetAttribute(k_depth_sort<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_depth_sort<32>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
+    if (depth_sort_cluster<16>() <= 0 || depth_sort_cluster<32>() <= 0) return cudaErrorInvalidConfiguration;
     return cudaFuncSetAttribute(k_tile_emit_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_EMIT_SMEM_MAX);
 }
 
