@@ -194,7 +194,8 @@ k_relu_back(const float *__restrict__ d, Col2Im g, const __nv_bfloat16 *__restri
                 *reinterpret_cast<uint2 *>(o + N) = *reinterpret_cast<const uint2 *>(l);
             }
         if (rows == 1) {
-            *reinterpret_cast<float4 *>(part + (int64_t)blockIdx.x * N + c) = sum;
+            // (widths between half a block's threads and all of them leave some without a row)
+            if (r == 0) *reinterpret_cast<float4 *>(part + (int64_t)blockIdx.x * N + c) = sum;
             continue;
         }
         if (r < rows) s_sum[r * NG + c / 4] = sum;
