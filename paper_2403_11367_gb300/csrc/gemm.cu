@@ -31,7 +31,7 @@
 //     lane's own row written straight from its registers put every lane of a
 //     store on another line, and the write took several times as long as the
 //     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us, and 53 with the
-//     waits below; 8192 x 8192 x 8192, where the write is a fortieth, 1060 and 1102).  Bias and
+//     waits below; 8192 x 8192 x 8192 1043 and 688).  Bias and
 //     ReLU are applied there.
 // An MN-major operand's tile is loaded as boxes of 64 columns (128 bytes) by the
 // 64 rows of the K step, in the canonical MN-major SWIZZLE_128B layout; its
@@ -62,7 +62,7 @@ constexpr int GEMM_EPI_LD = 36;                     // floats per staged row: 16
 constexpr unsigned long long GEMM_WAIT_NS = 1000000000ull;   // 1 s per wait
 // Tries between two looks at the timer.  A timer read before the first try and after
 // every further one stood in the chain from a stage's MMAs over its refill to its
-// next MMAs: 8192 x 8192 x 8192 1360 us, 1135 so (one try that sleeps up to 20 us in
+// next MMAs: 8192 x 8192 x 8192 in 128-column tiles 1360 us, 1135 so (one try that sleeps up to 20 us in
 // hardware: 1178); 8192 x 1024 x 1536 57.5 -> 53.
 constexpr int GEMM_TRIES = 64;
 constexpr int GEMM_BAND = 16;                       // row tiles of a band of the tile order
@@ -213,7 +213,7 @@ struct GemmSmem {
 // Row and column tile of tile mn: bands of 16 row tiles, columns after one another
 // within a band, so that the tiles in flight share their operands in both directions
 // (one row of tiles after the other reads all of B again for every five rows of A).
-// 8192 x 8192 x 8192: 1135 -> 1102 us; bands of 8 1140, of 32 1120, one band 1170.
+// 8192 x 8192 x 8192: one band 714 us, bands of 16 683, of 8 700, of 32 681.
 __device__ __forceinline__ int2 gemm_tile(int mn, int n_tm, int n_tn)
 {
     const int per = GEMM_BAND * n_tn, band = mn / per, r = mn - band * per, rows = min(GEMM_BAND, n_tm - GEMM_BAND * band);
@@ -555,15 +555,22 @@ static cudaError_t gemm_t(const GemmOperand &A, const GemmOperand &B, GemmArgs g
     return cudaGetLastError();
 }
 
-// The widest tile that N fills, halved while that leaves fewer columns to the
-// busiest SM: rounds of one tile an SM x BN is the time of the MMAs, and 128
-// rows by 1024 columns would run on 4 SMs at BN = 256.
+// The widest tile that N fills, halved while that shortens the busiest SM's time: its
+// rounds of one tile times a K step's, which goes with BN + 600 (8192 x 8192 x 8192: 0.383
+// us a step at 256 columns, 0.326 at 128, 0.297 at 64, 0.292 at 32; the chain from a
+// stage's MMAs over its refill does not shorten with the tile).  So narrow tiles pay only
+// where they cost no round: 128 rows by 1024 columns would run on 4 SMs at BN = 256.
+// Counting the columns of a round alone took 128 for that product, 1074 us, so 688; 32
+// for 5000 x 2000 x 1024, 94 us, so 31.
+constexpr int GEMM_STEP_COLUMNS = 600;
 static int gemm_bn(int M, int N, int split_k, int least)
 {
     int BN = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
     if (BN < least) BN = least;
-    auto columns = [&](int bn) { return ceil_div(ceil_div(M, GEMM_BM) * ceil_div(N, bn) * split_k, 152) * bn; };
-    while (BN / 2 >= (least > 32 ? least : 32) && columns(BN / 2) < columns(BN)) BN /= 2;
+    auto time = [&](int bn) {
+        return ceil_div(ceil_div(M, GEMM_BM) * ceil_div(N, bn) * split_k, 152) * (bn + GEMM_STEP_COLUMNS);
+    };
+    while (BN / 2 >= (least > 32 ? least : 32) && time(BN / 2) < time(BN)) BN /= 2;
     return BN;
 }
 
