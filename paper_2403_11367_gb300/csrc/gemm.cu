@@ -31,8 +31,7 @@
 //     lane's own row written straight from its registers put every lane of a
 //     store on another line, and the write took several times as long as the
 //     tile's MMAs: a call at 8192 x 1024 x 1536 134 us, so 57 us, and 53 with the
-//     waits below; 8192 x 8192 x 8192 1043 and 688).  Bias and
-//     ReLU are applied there.
+//     waits below; 8192 x 8192 x 8192 1043 and 688).  Bias and ReLU are applied there.
 // An MN-major operand's tile is loaded as boxes of 64 columns (128 bytes) by the
 // 64 rows of the K step, in the canonical MN-major SWIZZLE_128B layout; its
 // transposed copy (four launches per weight gradient, two per input gradient,
@@ -62,8 +61,8 @@ constexpr int GEMM_EPI_LD = 36;                     // floats per staged row: 16
 constexpr unsigned long long GEMM_WAIT_NS = 1000000000ull;   // 1 s per wait
 // Tries between two looks at the timer.  A timer read before the first try and after
 // every further one stood in the chain from a stage's MMAs over its refill to its
-// next MMAs: 8192 x 8192 x 8192 in 128-column tiles 1360 us, 1135 so (one try that sleeps up to 20 us in
-// hardware: 1178); 8192 x 1024 x 1536 57.5 -> 53.
+// next MMAs: 8192 x 8192 x 8192 in 128-column tiles 1360 us, 1135 so (one try that
+// sleeps up to 20 us in hardware: 1178); 8192 x 1024 x 1536 57.5 -> 53.
 constexpr int GEMM_TRIES = 64;
 constexpr int GEMM_BAND = 16;                       // row tiles of a band of the tile order
 
