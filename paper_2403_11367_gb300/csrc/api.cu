@@ -489,19 +489,23 @@ static reloc_status make_cam(const reloc_ctx *ctx, const reloc_camera *cam, CamP
     return RELOC_OK;
 }
 
-// Depth-ordered Gaussians per tile-binning chunk for a call of `pairs` (view,
-// Gaussian) pairs: 2048 where that gives BIN_CHUNKS_WANTED chunks or more, else
-// the smaller chunk that does, down to 256.  A chunk's row of tiles is written
-// by one warp in depth order, and the row through the horizon meets nearly all
-// of a chunk: a driving view's 51 chunks of 2048 left 113 us to that row's warps
-// on an idle GPU, 409 chunks of 256 take 29 us; 16 views (6.4 M pairs) emit in
-// 133 us at 1024 to a chunk, 138 at 512 (and count in 87 for 62 us); 64 views gain 4 us
-// at 1024 and count 28 us longer: every chunk costs a row of per-tile counts.
-static void set_bin_chunk(CamParams &cp, int64_t pairs)
+// Depth-ordered Gaussians per tile-binning chunk for a call that is expected to see
+// `visible` (view, Gaussian) pairs: 256 to 2048 in steps of 256, the least that gives
+// no more than BIN_CHUNKS chunks and BIN_CELLS (chunk, tile) counts.
+// Small chunks shorten the emission where a row of tiles meets nearly all of a chunk (one
+// warp writes the row in depth order: the horizon of a street); every chunk costs a row of
+// per-tile counts, written, scanned and read, which is all that many visible Gaussians or
+// tiles feel of them.  Counts and emission at 256 / 512 / 1024 / 2048, us: a driving view
+// (80k visible, 2112 tiles) 49 / 63 / 86 / 133, sixteen (1.3M) 205 / 156 / 152 / 179; 300k
+// small Gaussians seen whole there 74 / 60 / 51 / 49, at 1920 x 1080 (8160 tiles) 114 / 82 / 69 /
+// 66; a million at 1920 x 1080 526 / 201 / 148 / 134.
+static void set_bin_chunk(CamParams &cp, double visible)
 {
-    int chunk = BIN_CHUNK_MAX;
-    while (chunk > BIN_CHUNK_MIN && pairs / chunk < BIN_CHUNKS_WANTED) chunk /= 2;
-    cp.bin_chunk = chunk * (int)std::max<int64_t>(1, ceil_div(cp.n_tiles, BIN_TILES_PER_CHUNK_STEP));
+    const int step = (int)std::max<int64_t>(1, ceil_div(cp.n_tiles, BIN_TILES_PER_CHUNK_STEP));
+    const double chunks = std::min((double)BIN_CHUNKS, (double)BIN_CELLS / cp.n_tiles);
+    const double least = visible / chunks / (256.0 * step);
+    const int units = least >= BIN_CHUNK_MAX / 256 ? BIN_CHUNK_MAX / 256 : std::max(1, (int)std::ceil(least));
+    cp.bin_chunk = 256 * units * step;
 }
 
 static reloc_status make_view(const double *W, int v, ViewParams &P)
@@ -908,7 +912,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
                         cp.height, (long long)BLEND_MAX_UNITS);
     int64_t pairs = 0;
     for (auto &q : qs) pairs += q.S * q.V;
-    set_bin_chunk(cp, pairs);
+    set_bin_chunk(cp, ctx->vis_ratio * (double)pairs);
     CK(cudaSetDevice(ctx->device));
     ctx->last_valid = false;
     const int64_t HW = (int64_t)cp.width * cp.height;

@@ -51,8 +51,9 @@ constexpr int SORT_CHUNK = SORT_THREADS * SORT_IPT;   // 2048 items per block
 constexpr int RADIX = 256;
 // Tile binning (sort.cu): chunks of bin_chunk depth-ordered Gaussians, 256 to
 // 2048 of them (more on very large tile grids).
-constexpr int BIN_CHUNK_MAX = 2048, BIN_CHUNK_MIN = 256;
-constexpr int64_t BIN_CHUNKS_WANTED = 4096;
+constexpr int BIN_CHUNK_MAX = 2048;
+constexpr int BIN_CHUNKS = 1024;                      // non-empty chunks of a call at most, while below 2048
+constexpr int BIN_CELLS = 1 << 21;                    // and (chunk, tile) counts of those
 constexpr int BIN_TILES_PER_CHUNK_STEP = 8192;        // bin_chunk grows in proportion past 8192 tiles
 constexpr int TILE_COUNT_SMEM = 48 * 1024;            // difference-array band
 constexpr int TILE_EMIT_WARPS = 8;                    // tile rows per K4 block
