@@ -982,7 +982,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
             CKS(ctx->gcoef.ensure(32 * (size_t)V));
             CKS(ctx->gpart.ensure(48 * (size_t)pb));
         }
-        CKS(ctx->qpart.ensure(16 * QS_BLOCKS * (size_t)Qm));
+        CKS(ctx->qpart.ensure(16 * (size_t)query_blocks(cp.ncc_gray ? HW : 3 * HW) * (size_t)Qm));
         CKS(ctx->view_sel.ensure(4 * (size_t)Q));
         const size_t res_bytes = result_block(nullptr, Vtot, Q, (int64_t)sbs.size(), nullptr);
         CKS(ctx->res.ensure(res_bytes));

@@ -151,9 +151,13 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
 // = q_pblk[Q] (host copy).  run_begin, run_off: n_runs block-ordered runs and the
 // exclusive prefix of their lengths (device); the subset's map positions are
 // written to gidx.  qpart non-null: also the query images' partial sums
-// (QS_BLOCKS pairs of doubles a query: sum, sum of squares over the 3 H W
+// (query_blocks pairs of doubles a query: sum, sum of squares over the 3 H W
 // samples, or over the H W gray values (R + G + B) / 3 when cam.ncc_gray).
-constexpr int QS_BLOCKS = 304;
+// Blocks of a query of n samples: two to an SM for images up to a driving view's, one for
+// every 8192 samples beyond, so that they spread evenly over the SMs that the projection's
+// blocks leave (24.9M samples: the launch 328 us with 304 blocks, 163 with 2432; the
+// projection alone 18).  They follow from the image alone, so a query's sums do not depend on the call.
+__host__ __device__ __forceinline__ int query_blocks(int64_t n) { return (int)max64(304, min64(2432, n / 8192)); }
 cudaError_t launch_project(const float *mx, const float *my, const float *mz, const void *attr,
                            int precision, int sh_degree, int64_t n_map, const int64_t *run_begin,
                            const int64_t *run_off, int n_runs, uint32_t *gidx,

@@ -30,15 +30,15 @@ __device__ __forceinline__ uint32_t subset_position(const int64_t *__restrict__ 
 // ------------------------------------------------------ query statistics ---
 // Sum and sum of squares of block b's share of query q's samples, in FP64 (its
 // rate bounds this, so it runs in blocks beside the projection's, which wait on
-// memory); the QS_BLOCKS partials of a query are added by k_ncc_finalize.  Fixed
+// memory); the query_blocks partials of a query are added by k_ncc_finalize.  Fixed
 // shares and order: the sums are deterministic.
-__device__ __forceinline__ void query_partial(const float *__restrict__ q, int b, int64_t HW, int gray,
+__device__ __forceinline__ void query_partial(const float *__restrict__ q, int b, int n_b, int64_t HW, int gray,
                                               double *__restrict__ out)
 {
     __shared__ double s[2][PROJ_THREADS / 32];
     const int64_t n = gray ? HW : 3 * HW;
     double a = 0, c = 0;
-    constexpr int64_t STEP = (int64_t)QS_BLOCKS * PROJ_THREADS;
+    const int64_t STEP = (int64_t)n_b * PROJ_THREADS;
     for (int64_t j = (int64_t)b * PROJ_THREADS + threadIdx.x; j < n; j += 4 * STEP) {
         float v[4][3];                           // the samples of four steps in flight
 #pragma unroll
@@ -178,8 +178,10 @@ k_project(const float *__restrict__ mx, const float *__restrict__ my, const floa
     __shared__ ViewParams s_view[PROJ_VIEW_BATCH];
     chain_wait();
     if ((int)blockIdx.x >= n_blocks) {           // the query images' blocks
-        const int k = (int)blockIdx.x - n_blocks, q = k / QS_BLOCKS;
-        query_partial(L.q_img[q], k - q * QS_BLOCKS, (int64_t)cam.width * cam.height, cam.ncc_gray, qpart + 2 * (int64_t)k);
+        const int64_t HW = (int64_t)cam.width * cam.height;
+        const int n_b = query_blocks(cam.ncc_gray ? HW : 3 * HW);
+        const int k = (int)blockIdx.x - n_blocks, q = k / n_b;
+        query_partial(L.q_img[q], k - q * n_b, n_b, HW, cam.ncc_gray, qpart + 2 * (int64_t)k);
         return;
     }
 
@@ -333,7 +335,8 @@ cudaError_t launch_project(const float *mx, const float *my, const float *mz, co
                            uint32_t *gidx, const Layout &L, int n_blocks, const ViewParams *views, const CamParams &cam,
                            Records rec, uint2 *rect, uint32_t *dkey, double *qpart, cudaStream_t st)
 {
-    const int64_t grid = n_blocks + (qpart ? (int64_t)QS_BLOCKS * L.Q : 0);
+    const int64_t HW = (int64_t)cam.width * cam.height;
+    const int64_t grid = n_blocks + (qpart ? (int64_t)query_blocks(cam.ncc_gray ? HW : 3 * HW) * L.Q : 0);
     if (grid <= 0) return cudaSuccess;
     if (grid > 0x7fffffff) return cudaErrorInvalidValue;
 #define RELOC_PROJECT_CASE(P_, T_, D_)                                                                              \

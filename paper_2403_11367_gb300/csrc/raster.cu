@@ -788,9 +788,10 @@ k_ncc_finalize(const double *__restrict__ partials, const double *__restrict__ q
     c = warp_sum_d(c);
     // the query's partial sums
     double d = 0, e = 0;
-    for (int t = threadIdx.x; t < QS_BLOCKS; t += NCC_THREADS) {
-        d += qpart[2 * ((int64_t)q * QS_BLOCKS + t)];
-        e += qpart[2 * ((int64_t)q * QS_BLOCKS + t) + 1];
+    const int n_b = query_blocks(n);
+    for (int t = threadIdx.x; t < n_b; t += NCC_THREADS) {
+        d += qpart[2 * ((int64_t)q * n_b + t)];
+        e += qpart[2 * ((int64_t)q * n_b + t) + 1];
     }
     d = warp_sum_d(d);
     e = warp_sum_d(e);
