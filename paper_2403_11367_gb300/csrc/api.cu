@@ -163,6 +163,11 @@ size_t result_block(char *base, int64_t V, int64_t Q, int64_t n_sb, ResultBlock 
 
 }  // namespace
 
+// The visible share that a call is expected to have is at least this, whatever the last one
+// saw: after a view of nothing the next call would be binned in the smallest chunks however
+// much it sees, with up to eight times the counts.
+constexpr double VIS_RATIO_MIN = 1.0 / 8.0;
+
 struct reloc_ctx {
     reloc_config cfg{};
     int device = 0;
@@ -1089,7 +1094,7 @@ static reloc_status run_batch(reloc_ctx *ctx, std::vector<QuerySpec> &qs, const 
                 ctx->counts.n_visible += h_nvis[v];
                 ctx->counts.n_instances += h_ninst[v];
             }
-            if (pairs > 0) ctx->vis_ratio = (double)ctx->counts.n_visible / (double)pairs;
+            if (pairs > 0) ctx->vis_ratio = std::max(VIS_RATIO_MIN, (double)ctx->counts.n_visible / (double)pairs);
             ctx->counts.inst_stride = sbs[0].io_off.size() > 1 ? sbs[0].io_off[1] - sbs[0].io_off[0] : 0;
             ctx->counts.retries = retries;
             ctx->counts.kernel_launches = launches;
