@@ -34,10 +34,11 @@
 //     update formed with an entry per lane; reciprocals and inverse square roots
 //     take an FP32 seed and Newton's iteration to FP64, the rotation its power
 //     series for angles below half a radian.
-// Some 7,000 pairs on the driving street: 641 us a call with one block per 256
-// pairs, five barriers and two passes an iteration, 196 us so; 6,124 pairs 201 us
-// with one pass, one barrier and a thread's serial solve, 167 us so (15 us an
-// iteration, 13 of them with a single block: the chain, not the pairs).
+// Some 7,000 pairs on the driving street: 600 to 640 us a call with one block per 256
+// pairs, five barriers and two passes an iteration, 180 to 230 us so (157 to 196 with
+// steps judged by summed costs); of 6,124 pairs 201 us with one pass, one barrier and a
+// thread's serial solve, 167 with the lanes' (15 us an iteration, 13 of them with a single
+// block: the chain, not the pairs).
 #include <algorithm>
 
 #include <cooperative_groups.h>
